@@ -192,7 +192,7 @@ __global__ void k_inc_fill(const int *tris, int ntri, const int *off, int *cur, 
 // lanes rank 32 entries at a time against the whole list into sorted[], then sum it in chunks
 // of 32.  One thread per node that searched the list for each next triangle took 227 us on a
 // 4098-node mesh whose two poles have 128 triangles (all other nodes 6 or fewer), serial in the
- of the valence; this takes 9 us there.
+// square of the valence; this takes 27 us there.
 constexpr int NODE_THREADS = 128;
 __global__ void __launch_bounds__(NODE_THREADS) k_node_forces(const int *off, const int *list, const double *share,
                                                               long long nvert, int *sorted, double *F) {
