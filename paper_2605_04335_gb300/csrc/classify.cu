@@ -23,6 +23,7 @@
 #include <cstring>
 
 #include "ibm_internal.cuh"
+#include "scan.cuh"
 
 namespace ibm {
 namespace {
@@ -135,26 +136,6 @@ __global__ void k_tri_setup(const double *verts, const int *tris, int ntri, cons
   T.area = area;
   out[t] = T;
   count[t] = cnt;
-}
-
-// exclusive scan of n int64 counts in one block; out has n+1 entries
-__global__ void k_scan_single(const long long *in, long long *out, int n) {
-  __shared__ long long part[1024];
-  int tid = threadIdx.x, nt = blockDim.x;
-  int per = (n + nt - 1) / nt;
-  int b = tid * per, e = min(n, b + per);
-  long long s = 0;
-  for (int i = b; i < e; ++i) s += in[i];
-  part[tid] = s;
-  __syncthreads();
-  if (tid == 0) {
-    long long run = 0;
-    for (int i = 0; i < nt; ++i) { long long v = part[i]; part[i] = run; run += v; }
-    out[n] = run;
-  }
-  __syncthreads();
-  long long run = part[tid];
-  for (int i = b; i < e; ++i) { out[i] = run; run += in[i]; }
 }
 
 __device__ __forceinline__ bool in_closed_tri2d(long long pu0, long long pv0, long long pu1, long long pv1,
@@ -1200,15 +1181,17 @@ cudaError_t build_bins(Scratch &S, const double *tv, int ntri, const TriStats &t
   B.h = h;
   B.inv = 1.0 / h;
   const long long nb = (long long)B.nb[0] * B.nb[1] * B.nb[2];
-  long long *cnt = nullptr, *off = nullptr;
+  long long *cnt = nullptr, *off = nullptr, *tmp = nullptr;
   int *tri = nullptr;
   cudaError_t e;
-  if ((e = S.get(&cnt, nb)) != cudaSuccess || (e = S.get(&off, nb + 1)) != cudaSuccess) return e;
+  if ((e = S.get(&cnt, nb)) != cudaSuccess || (e = S.get(&off, nb + 1)) != cudaSuccess ||
+      (e = S.get(&tmp, scan_scratch(nb))) != cudaSuccess)
+    return e;
   uint2 *range = nullptr;
   if ((e = S.get(&range, ntri)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(cnt, 0, sizeof(long long) * nb, st)) != cudaSuccess) return e;
   k_bin_count<<<nblk(ntri, 128), 128, 0, st>>>(tv, ntri, B, cnt, range);
-  k_scan_single<<<1, 1024, 0, st>>>(cnt, off, (int)nb);
+  launch_scan(cnt, off, (int)nb, tmp, st);
   long long total = 0;
   if ((e = cudaMemcpyAsync(&total, off + nb, sizeof(long long), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
@@ -1317,12 +1300,13 @@ ibm_status membrane_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
   MTRY(cudaMemsetAsync(linktri, 0x7f, sizeof(int) * 3 * ncell, st));   // every link: NO_TRI
   if (ntri > 0) {
     MTri *recs = nullptr;
-    long long *cnt = nullptr, *off = nullptr;
+    long long *cnt = nullptr, *off = nullptr, *tmp = nullptr;
     MTRY(S.get(&recs, 3 * (size_t)ntri));
     MTRY(S.get(&cnt, 3 * (size_t)ntri));
     MTRY(S.get(&off, 3 * (size_t)ntri + 1));
+    MTRY(S.get(&tmp, scan_scratch(3LL * ntri)));
     k_mem_setup<<<nblk(3 * ntri, 128), 128, 0, st>>>(tv, ntri, ax, recs, cnt);
-    k_scan_single<<<1, 1024, 0, st>>>(cnt, off, 3 * ntri);
+    launch_scan(cnt, off, 3 * ntri, tmp, st);
     long long total = 0;
     MTRY(cudaMemcpyAsync(&total, off + 3 * ntri, sizeof(long long), cudaMemcpyDeviceToHost, st));
     MTRY(cudaStreamSynchronize(st));
@@ -1336,11 +1320,12 @@ ibm_status membrane_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
   // ghost entries in (cell, side) order
   const long long chunk = (long long)GM_THREADS * GM_PER;
   const unsigned nb = (unsigned)((ncell + chunk - 1) / chunk);
-  long long *bc = nullptr, *bo = nullptr;
+  long long *bc = nullptr, *bo = nullptr, *tmp = nullptr;
   MTRY(S.get(&bc, nb));
   MTRY(S.get(&bo, nb + 1));
   k_mem_count<<<nb, GM_THREADS, 0, st>>>(T->cut, T->cside, ncell, bc);
-  k_scan_single<<<1, 1024, 0, st>>>(bc, bo, (int)nb);
+  MTRY(S.get(&tmp, scan_scratch(nb)));
+  launch_scan(bc, bo, (int)nb, tmp, st);
   long long ng = 0;
   MTRY(cudaMemcpyAsync(&ng, bo + nb, sizeof(long long), cudaMemcpyDeviceToHost, st));
   MTRY(cudaStreamSynchronize(st));
@@ -1468,11 +1453,11 @@ ibm_status classify_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
       const int nt = meshes[m].ntris;
       if (nt == 0) continue;
       Tri *tr = nullptr;
-      long long *cnt = nullptr, *off = nullptr;
-      CTRY(S.get(&tr, nt)); CTRY(S.get(&cnt, nt)); CTRY(S.get(&off, nt + 1));
+      long long *cnt = nullptr, *off = nullptr, *tmp = nullptr;
+      CTRY(S.get(&tr, nt)); CTRY(S.get(&cnt, nt)); CTRY(S.get(&off, nt + 1)); CTRY(S.get(&tmp, scan_scratch(nt)));
       k_tri_setup<<<nblk(nt, 128), 128, 0, st>>>(dverts + 3LL * vbase[m], dtris + 3LL * tbase[m], nt, ds[0], nx,
                                                   ds[1], ny, ds[2], nz, tr, cnt);
-      k_scan_single<<<1, 1024, 0, st>>>(cnt, off, nt);
+      launch_scan(cnt, off, nt, tmp, st);
       long long total = 0;
       CTRY(cudaMemcpyAsync(&total, off + nt, sizeof(long long), cudaMemcpyDeviceToHost, st));
       CTRY(cudaStreamSynchronize(st));
@@ -1506,12 +1491,12 @@ ibm_status classify_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
   const unsigned nb = (unsigned)((ncell + chunk - 1) / chunk);
   unsigned long long *cellcnt = nullptr;
   {
-    long long *bc = nullptr, *bo = nullptr;
-    CTRY(S.get(&bc, nb)); CTRY(S.get(&bo, nb + 1));
+    long long *bc = nullptr, *bo = nullptr, *tmp = nullptr;
+    CTRY(S.get(&bc, nb)); CTRY(S.get(&bo, nb + 1)); CTRY(S.get(&tmp, scan_scratch(nb)));
     CTRY(S.get(&cellcnt, 2));
     CTRY(cudaMemsetAsync(cellcnt, 0, 16, st));
     k_ghost_count<<<nb, GM_THREADS, 0, st>>>(T->iblank, nx, ny, nz, ncell, bc);
-    k_scan_single<<<1, 1024, 0, st>>>(bc, bo, (int)nb);
+    launch_scan(bc, bo, (int)nb, tmp, st);
     long long ng = 0;
     CTRY(cudaMemcpyAsync(&ng, bo + nb, sizeof(long long), cudaMemcpyDeviceToHost, st));
     CTRY(cudaStreamSynchronize(st));

@@ -27,6 +27,7 @@
 
 #include "ibm_internal.cuh"
 #include "dfloat.cuh"
+#include "scan.cuh"
 #include "zmarch.cuh"
 
 namespace ibm {
@@ -1599,26 +1600,6 @@ constexpr int CUT_THREADS = 256, CUT_PER = 16;   // compaction: cells per thread
 constexpr int CUT_BLOCKS = 152;                  // grid of the cut-cell kernels (grid-stride; fixed
                                                  // reduction width)
 
-// exclusive scan of n int64 counts in one block; out has n+1 entries
-__global__ void k_scan1(const long long *in, long long *out, int n) {
-  __shared__ long long part[1024];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int per = (n + nt - 1) / nt;
-  const int b = tid * per, e = min(n, b + per);
-  long long s = 0;
-  for (int i = b; i < e; ++i) s += in[i];
-  part[tid] = s;
-  __syncthreads();
-  if (tid == 0) {
-    long long run = 0;
-    for (int i = 0; i < nt; ++i) { long long v = part[i]; part[i] = run; run += v; }
-    out[n] = run;
-  }
-  __syncthreads();
-  long long run = part[tid];
-  for (int i = b; i < e; ++i) { out[i] = run; run += in[i]; }
-}
-
 // cells of one colour ((i + j + k) mod 2) with a cut link, per block of CUT_THREADS x CUT_PER
 __global__ void k_cut_count(const uint8_t *cut, const uint8_t *ib, int nx, int ny, long long ncell, int colour,
                             long long *bcount) {
@@ -2627,14 +2608,15 @@ static ibm_status refresh_geometry_t(ibm_tables *t, Hierarchy *h, cudaStream_t s
     if (h->scan_cap < need) {
       if (h->scan_buf) cudaFree(h->scan_buf);
       h->scan_buf = nullptr; h->scan_cap = 0;
-      IBM_TRY(cudaMalloc((void **)&h->scan_buf, sizeof(long long) * 4 * need));
+      IBM_TRY(cudaMalloc((void **)&h->scan_buf, sizeof(long long) * 5 * need));
       h->scan_cap = need;
     }
-    long long *bc = h->scan_buf, *bo[2] = {h->scan_buf + 2 * need, h->scan_buf + 3 * need};
+    long long *bc = h->scan_buf, *bo[2] = {h->scan_buf + 2 * need, h->scan_buf + 3 * need},
+              *tmp = h->scan_buf + 4 * need;   // the scans' scratch: fewer than need values
     long long counts[2];
     for (int colour = 0; colour < 2; ++colour) {
       k_cut_count<<<nb, CUT_THREADS, 0, st>>>(t->cut, t->iblank, L0.g.nx, L0.g.ny, ncell, colour, bc + colour * need);
-      k_scan1<<<1, 1024, 0, st>>>(bc + colour * need, bo[colour], (int)nb);
+      launch_scan(bc + colour * need, bo[colour], (int)nb, tmp, st);
     }
     IBM_TRY(cudaMemcpyAsync(&counts[0], bo[0] + nb, sizeof(long long), cudaMemcpyDeviceToHost, st));
     IBM_TRY(cudaMemcpyAsync(&counts[1], bo[1] + nb, sizeof(long long), cudaMemcpyDeviceToHost, st));
@@ -2660,7 +2642,7 @@ static ibm_status refresh_geometry_t(ibm_tables *t, Hierarchy *h, cudaStream_t s
     if (!h->par_flag) IBM_TRY(alloc_zero<uint8_t>((void **)&h->par_flag, L1.g.ntot, st));
     k_par_flag<<<FIXED_BLOCKS, 256, 0, st>>>(h->cut_id, h->cut_ijk, h->d_cnt, L1.g, h->par_flag);
     k_par_count<<<nbp, CUT_THREADS, 0, st>>>(h->par_flag, L1.g.ntot, bc);
-    k_scan1<<<1, 1024, 0, st>>>(bc, bo[0], (int)nbp);
+    launch_scan(bc, bo[0], (int)nbp, tmp, st);
     long long npar = 0;
     IBM_TRY(cudaMemcpyAsync(&npar, bo[0] + nbp, sizeof(long long), cudaMemcpyDeviceToHost, st));
     IBM_TRY(cudaStreamSynchronize(st));

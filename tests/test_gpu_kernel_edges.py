@@ -7,7 +7,7 @@ import synth
 from oracle import classify as OC
 from oracle import forces as OF
 from oracle.grid import Grid
-from tests.gpu_util import require_gpu, torch
+from tests.gpu_util import assert_tables_equal, classify_both, require_gpu, torch
 
 pytestmark = pytest.mark.gpu
 
@@ -46,4 +46,25 @@ def test_nodal_forces_by_valence(ctx, n):
     ps, _, F = OF.surface_forces(grid, ib, [m], p)
     assert np.array_equal(out["p_side"].cpu().numpy(), ps)
     assert np.array_equal(out["f_node"].cpu().numpy(), F)
+    T.close()
+
+
+@pytest.mark.parametrize("n", [3, 511, 512, 513, 1024, 1025])
+def test_classification_by_triangle_count(ctx, n):
+    """2 n triangles (the scans run 1024 counts at a time): tables bit for bit the oracle's."""
+    pkg, c = ctx
+    f = synth.faces_uniform(24)
+    _, T, ex, ib, G = classify_both(pkg, c, f, f, f, [_double_cone(n)])
+    assert_tables_equal(ex, ib, G)
+    T.close()
+
+
+@pytest.mark.parametrize("shape", [(64, 64, 1023), (64, 64, 1024), (67, 64, 1024), (129, 131, 260)])
+def test_ghost_compaction_by_grid_size(ctx, shape):
+    """Ghost lists of grids around 1024 blocks of the compaction (4096 cells each)."""
+    pkg, c = ctx
+    xf, yf, zf = [synth.faces_uniform(n) for n in shape]
+    _, T, ex, ib, _ = classify_both(pkg, c, xf, yf, zf, [synth.octa_sphere(3, (0.5, 0.5, 0.5), 0.41)], oracle_ghosts=False)
+    assert np.array_equal(ex["iblank"], ib)
+    assert np.array_equal(ex["cell"], np.flatnonzero(ib.ravel() == 3))
     T.close()
