@@ -441,6 +441,10 @@ struct GhostArgs {
   const double *tv;        // ntri x 9 vertex coordinates
   const float4 *blo, *bhi; // triangle boxes, outward-rounded to float
   const float4 *cen;       // triangle centroids (float)
+  const float4 *tf;        // ntri x 3 vertices (float); w of the first: the longest edge, of the
+                           // second: 1 for a sliver (see closest_bounds)
+  int *cand;               // candidates of each ghost (closed bodies): CAND_OUT each, and their number
+  int *ncand;
   TriBins bins;
   long long ng;
   const long long *gcell;
@@ -460,9 +464,8 @@ __device__ __forceinline__ void base_t(const double *c, int n, double v, int &i0
   t = tt < 0.0 ? 0.0 : (tt > 1.0 ? 1.0 : tt);
 }
 
-// one warp per ghost: the lanes split the triangle loops, then a warp reduction picks the
-// minimum squared distance (lowest triangle index on exact ties), the same result as a
-// sequential scan; lane 0 finishes the row
+// minimum squared distance over the warp (lowest triangle index on exact ties), the same result
+// as a sequential scan
 __device__ __forceinline__ void warp_argmin(double &d, int &t, float &f) {
   for (int o = 16; o > 0; o >>= 1) {
     double od = __shfl_xor_sync(0xffffffffu, d, o);
@@ -600,6 +603,240 @@ __device__ void find_closest(const GhostArgs &a, const double P[3], int lane, do
   for (int d = 0; d < 3; ++d) Q[d] = __shfl_sync(0xffffffffu, lq[d], src);
 }
 
+// FP32 bounds of the distance from the float point p to triangle t: |d - d_true| <= m with
+// m = 4e-6 + 4e-3 (d + longest edge).  The float vertices and p lie within 5e-7 of the true ones
+// (coordinates up to 4), and a distance moves no more than they do; the normal equations of a
+// triangle with sin^2 of its angle at the first vertex >= 1e-3 and both edges there above 1e-4
+// give the closest point to about 1e-3 |p - A| in FP32.  Others (slivers) are not bounded from
+// above, and from below by their box alone.
+constexpr float BOUND_ABS = 4e-6f, BOUND_REL = 4e-3f;
+__device__ __forceinline__ void closest_bounds(const GhostArgs &a, int t, const float p[3], float box2, float &lo,
+                                               float &up) {
+  const float4 A = a.tf[3 * t], B = a.tf[3 * t + 1], C = a.tf[3 * t + 2];
+  if (B.w != 0.f) {
+    lo = sqrtf(box2) - BOUND_ABS;
+    up = 3.4e38f;
+    return;
+  }
+  const float ab[3] = {B.x - A.x, B.y - A.y, B.z - A.z}, ac[3] = {C.x - A.x, C.y - A.y, C.z - A.z};
+  const float bc[3] = {C.x - B.x, C.y - B.y, C.z - B.z};
+  const float ap[3] = {p[0] - A.x, p[1] - A.y, p[2] - A.z}, bp[3] = {p[0] - B.x, p[1] - B.y, p[2] - B.z};
+  auto dot = [](const float x[3], const float y[3]) { return fmaf(x[0], y[0], fmaf(x[1], y[1], x[2] * y[2])); };
+  const float aa = dot(ab, ab), bb = dot(ab, ac), cc = dot(ac, ac), d = dot(ab, ap), e = dot(ac, ap);
+  const float det = aa * cc - bb * bb, su = cc * d - bb * e, sv = aa * e - bb * d;
+  auto off2 = [](const float x[3], const float y[3], float s) {   // |x - s y|^2
+    const float u = fmaf(-s, y[0], x[0]), v = fmaf(-s, y[1], x[1]), w = fmaf(-s, y[2], x[2]);
+    return fmaf(u, u, fmaf(v, v, w * w));
+  };
+  float d2;
+  if (su >= 0.f && sv >= 0.f && su + sv <= det) {
+    const float r = 1.f / det, u = su * r;
+    const float q[3] = {fmaf(-u, ab[0], ap[0]), fmaf(-u, ab[1], ap[1]), fmaf(-u, ab[2], ap[2])};
+    d2 = off2(q, ac, sv * r);
+  } else {
+    d2 = off2(ap, ab, __saturatef(d / aa));
+    d2 = fminf(d2, off2(ap, ac, __saturatef(e / cc)));
+    d2 = fminf(d2, off2(bp, bc, __saturatef(dot(bc, bp) / dot(bc, bc))));
+  }
+  const float dist = sqrtf(d2), m = fmaf(BOUND_REL, dist + A.w, BOUND_ABS);
+  lo = dist - m;
+  up = dist + m;
+}
+
+// The few triangles that can be the closest one to each ghost's centre, by FP32 bounds: every
+// triangle whose lower bound does not exceed the least upper bound found, so the minimum of the
+// FP64 distances, and every tie with it, is among them.  One warp per ghost walks the bins in
+// Chebyshev shells as find_closest does; a shell's bins are contiguous runs of the triangle list
+// (a row of bins along x, or its two end bins), whose entries the lanes share evenly.  A ghost
+// with more than CAND_OUT candidates (slivers, points nearly equally far from many triangles)
+// has them compared in FP64 by its warp, one with more than CAND_LIST is searched by
+// find_closest.  FP64 issues at 1/64 of the FP32 rate and a warp instruction
+// costs the same however few of its lanes are on, so the search leaves the FP64 distances (one
+// or two per ghost) and the rows to k_ghost_tables, one thread per ghost: twelve spheres at
+// 512^3 took 2520 us with FP64 distances and rows in the search's warp, 630 us
+// with both kernels now.
+constexpr int CAND_OUT = 6, CAND_LIST = 128;
+__global__ void __launch_bounds__(TABLE_THREADS) k_ghost_candidates(GhostArgs a) {
+  __shared__ int ct_s[TABLE_THREADS / 32][CAND_LIST];
+  __shared__ float cl_s[TABLE_THREADS / 32][CAND_LIST];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const long long g = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  if (g >= a.ng) return;   // whole warps
+  int *ct = ct_s[threadIdx.x >> 5];
+  float *cl = cl_s[threadIdx.x >> 5];
+  const long long lin = a.gcell[g];
+  const double P[3] = {a.xc[lin % a.nx], a.yc[(lin / a.nx) % a.ny], a.zc[lin / ((long long)a.nx * a.ny)]};
+  const float Pf[3] = {(float)P[0], (float)P[1], (float)P[2]};
+  const TriBins &B = a.bins;
+  int c[3];
+  for (int d = 0; d < 3; ++d)
+    c[d] = (int)fmin(fmax(floor((P[d] - B.lo[d]) * B.inv), 0.0), (double)(B.nb[d] - 1));
+  float thr = 3.4e38f;   // an upper bound of the distance (box margin included)
+  int n = 0;             // candidates in the list
+  bool over = false;
+  auto compact = [&]() {   // drop the candidates above the current bound
+    __syncwarp();
+    constexpr int H = CAND_LIST / 32;
+    int t[H];
+    float l[H];
+    bool k[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      const int q = lane + 32 * h;
+      k[h] = q < n && cl[q] <= thr;
+      t[h] = q < n ? ct[q] : 0;
+      l[h] = q < n ? cl[q] : 0.f;
+    }
+    __syncwarp();
+    int m = 0;
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      const unsigned b = __ballot_sync(full, k[h]);
+      if (k[h]) {
+        const int at = m + __popc(b & ((1u << lane) - 1u));
+        ct[at] = t[h];
+        cl[at] = l[h];
+      }
+      m += __popc(b);
+    }
+    n = m;
+    __syncwarp();
+  };
+  for (int r = 1; !over; ++r) {
+    const int w = 2 * r + 1;
+    int vl[3], vh[3], pl[3], ph[3];   // visited block after this shell, and before it
+    for (int d = 0; d < 3; ++d) {
+      vl[d] = max(c[d] - r, 0); vh[d] = min(c[d] + r, B.nb[d] - 1);
+      pl[d] = max(c[d] - r + 1, 0); ph[d] = min(c[d] + r - 1, B.nb[d] - 1);
+    }
+    // run u of the shell: row u / 2 of the w x w rows along x; rows on the shell's y or z faces
+    // whole (u even), the others their left and right end bins
+    auto run = [&](int u, long long &b, long long &e, int &y, int &z) {
+      b = e = 0;
+      const int row = u >> 1, dy = row % w - r, dz = row / w - r;
+      y = c[1] + dy;
+      z = c[2] + dz;
+      if (row >= w * w || y < 0 || z < 0 || y >= B.nb[1] || z >= B.nb[2]) return;
+      const long long at = ((long long)z * B.nb[1] + y) * B.nb[0];
+      int x0 = vl[0], x1 = vh[0];
+      if (r == 1 || abs(dy) == r || abs(dz) == r) {
+        if (u & 1) return;
+      } else {
+        x0 = x1 = (u & 1) ? c[0] + r : c[0] - r;
+        if (x0 < 0 || x0 >= B.nb[0]) return;
+      }
+      b = B.off[at + x0];
+      e = B.off[at + x1 + 1];
+    };
+    for (int pass = 0; pass < 2; ++pass) {   // centroids bound the distance, then the triangles
+      float cb = 3.4e38f;
+      for (int u0 = 0; u0 < 2 * w * w; u0 += 32) {
+        long long b, e;
+        int y, z;
+        run(u0 + lane, b, e, y, z);
+        const int len = (int)(e - b);
+        int pre = len;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(full, pre, o);
+          if (lane >= o) pre += v;
+        }
+        const int total = __shfl_sync(full, pre, 31);
+        for (int q0 = 0; q0 < total; q0 += 32) {
+          const int q = q0 + lane;
+          int own = 0;   // the run that holds entry q: the first with pre > q
+          for (int s = 16; s > 0; s >>= 1) {
+            const int v = __shfl_sync(full, pre, own + s - 1);
+            if (v <= q) own += s;
+          }
+          const long long rb = __shfl_sync(full, b, own);
+          const int rl = __shfl_sync(full, pre, own) - __shfl_sync(full, len, own);
+          const int ry = __shfl_sync(full, y, own), rz = __shfl_sync(full, z, own);
+          const bool live = q < total;
+          const long long en = rb + (q - rl);
+          const int t = live ? B.tri[en] : 0;
+          if (pass == 0) {
+            if (live) {
+              const float4 cc = a.cen[t];
+              const float dx = cc.x - Pf[0], dy = cc.y - Pf[1], dz = cc.z - Pf[2];
+              cb = fminf(cb, dx * dx + dy * dy + dz * dz);
+            }
+            continue;
+          }
+          float lo = 3.4e38f, up = 3.4e38f;
+          if (live) {
+            const float box2 = box_dist2(Pf, a.blo[t], a.bhi[t]);
+            if (box2 <= thr * thr) {
+              // taken once: from the first bin of its range inside the block, and only if no
+              // earlier shell met its range
+              const uint2 rg = B.range[t];
+              int f[3], f2[3];
+              range_meets(rg, vl, vh, f);
+              bool mine = f[1] == ry && f[2] == rz && (r == 1 || !range_meets(rg, pl, ph, f2));
+              if (mine) {
+                const long long at = ((long long)rz * B.nb[1] + ry) * B.nb[0] + f[0];
+                mine = en >= B.off[at] && en < B.off[at + 1];
+              }
+              if (mine) closest_bounds(a, t, Pf, box2, lo, up);
+            }
+          }
+          float least = up;
+          for (int o = 16; o > 0; o >>= 1) least = fminf(least, __shfl_xor_sync(full, least, o));
+          thr = fminf(thr, least < 3e38f ? least + BOUND_ABS : 3.4e38f);
+          bool keep = lo <= thr && lo < 3e38f;
+          unsigned kb = __ballot_sync(full, keep);
+          if (n + __popc(kb) > CAND_LIST) compact();
+          if (n + __popc(kb) > CAND_LIST) { over = true; break; }
+          if (keep) {
+            const int at = n + __popc(kb & ((1u << lane) - 1u));
+            ct[at] = t;
+            cl[at] = lo;
+          }
+          n += __popc(kb);
+        }
+        if (over) break;
+      }
+      if (pass == 0) {
+        for (int o = 16; o > 0; o >>= 1) cb = fminf(cb, __shfl_xor_sync(full, cb, o));
+        if (cb < 3.4e38f) thr = fminf(thr, sqrtf(cb) * (1.0f + 1e-5f) + BOUND_ABS);
+      }
+      if (over) break;
+    }
+    double lv = 1e300;   // distance from P to the bins outside the visited cube
+    bool more = false;
+    for (int d = 0; d < 3; ++d) {
+      if (c[d] - r - 1 >= 0) { more = true; lv = fmin(lv, P[d] - (B.lo[d] + (c[d] - r) * B.h)); }
+      if (c[d] + r + 1 < B.nb[d]) { more = true; lv = fmin(lv, (B.lo[d] + (c[d] + r + 1) * B.h) - P[d]); }
+    }
+    if (!more || lv > (double)thr) break;
+  }
+  if (!over) compact();
+  if (over || n > CAND_OUT) {   // FP64 over the warp: the list, or the whole search
+    double best = 1e300, Q[3];
+    int bidx = 0x7fffffff;
+    if (over) {
+      __syncwarp();
+      find_closest(a, P, lane, best, bidx, Q, ct);
+    } else {
+      for (int q = lane; q < n; q += 32) {
+        const int t = ct[q];
+        double d2, Qt[3];
+        closest_on_tri(P, a.tv + 9 * t, a.tv + 9 * t + 3, a.tv + 9 * t + 6, Qt, d2);
+        if (d2 < best || (d2 == best && t < bidx)) { best = d2; bidx = t; }
+      }
+      float unused = 0.f;
+      warp_argmin(best, bidx, unused);
+    }
+    if (lane == 0) {
+      a.cand[CAND_OUT * g] = bidx;
+      a.ncand[g] = 1;
+    }
+    return;
+  }
+  if (lane < n) a.cand[CAND_OUT * g + lane] = ct[lane];
+  if (lane == 0) a.ncand[g] = n;
+}
+
 // Neumann coefficient of a row (moving-boundary datum): g = p(IP) - l q with l = |IP - GC|
 // and q the derivative along (IP - GC) / l, so g - sum w v = kappa q, kappa = -l, divided by
 // 1 - w_self when the row's own weight was moved to the left-hand side
@@ -617,10 +854,10 @@ __device__ __forceinline__ double fallback_kappa(const GhostArgs &a, const doubl
   return -sqrt((fx * fx + fy * fy) + fz * fz);
 }
 
+// the closest of each ghost's candidates in FP64 (lowest index on exact ties) and its row, one
+// thread per ghost
 __global__ void __launch_bounds__(TABLE_THREADS) k_ghost_tables(GhostArgs a) {
-  __shared__ int cand[TABLE_THREADS / 32][CAND_MAX];
-  const int lane = threadIdx.x & 31;
-  long long g = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (g >= a.ng) return;
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   long long lin = a.gcell[g];
@@ -628,10 +865,17 @@ __global__ void __launch_bounds__(TABLE_THREADS) k_ghost_tables(GhostArgs a) {
   int gj = (int)((lin / nx) % ny);
   int gk = (int)(lin / ((long long)nx * ny));
   double P[3] = {a.xc[gi], a.yc[gj], a.zc[gk]};
-  double best, BQ[3];
-  int bidx;
-  find_closest(a, P, lane, best, bidx, BQ, cand[threadIdx.x >> 5]);
-  if (lane != 0) return;
+  double best = 1e300, BQ[3] = {0.0, 0.0, 0.0};
+  int bidx = 0x7fffffff;
+  for (int q = 0; q < a.ncand[g]; ++q) {
+    const int t = a.cand[CAND_OUT * g + q];
+    double d2, Q[3];
+    closest_on_tri(P, a.tv + 9 * t, a.tv + 9 * t + 3, a.tv + 9 * t + 6, Q, d2);
+    if (d2 < best || (d2 == best && t < bidx)) {
+      best = d2; bidx = t;
+      BQ[0] = Q[0]; BQ[1] = Q[1]; BQ[2] = Q[2];
+    }
+  }
   double IP[3];
   for (int d = 0; d < 3; ++d) {
     IP[d] = (BQ[d] + BQ[d]) - P[d];
@@ -722,7 +966,7 @@ __global__ void __launch_bounds__(TABLE_THREADS) k_ghost_tables(GhostArgs a) {
 }
 
 // triangle boxes (outward-rounded to float) and centroids, for the pruned search
-__global__ void k_tri_boxes(const double *tv, int ntri, float4 *blo, float4 *bhi, float4 *cen) {
+__global__ void k_tri_boxes(const double *tv, int ntri, float4 *blo, float4 *bhi, float4 *cen, float4 *tf) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ntri) return;
   const double *v = tv + 9 * t;
@@ -736,6 +980,30 @@ __global__ void k_tri_boxes(const double *tv, int ntri, float4 *blo, float4 *bhi
   blo[t] = make_float4(lo[0], lo[1], lo[2], 0.f);
   bhi[t] = make_float4(hi[0], hi[1], hi[2], 0.f);
   cen[t] = make_float4(c[0], c[1], c[2], 0.f);
+  if (!tf) return;
+  // float vertices, the longest edge (rounded up) and whether the triangle is a sliver
+  double e2[3], dot = 0.0;
+  for (int q = 0; q < 3; ++q) {
+    const double *p = v + 3 * q, *o = v + 3 * ((q + 1) % 3);
+    const double x = o[0] - p[0], y = o[1] - p[1], z = o[2] - p[2];
+    e2[q] = (x * x + y * y) + z * z;
+  }
+  // first vertex: the one with the largest sin^2 of its angle (the least product of its edges), so
+  // a needle counts as a sliver only when its short edge is tiny
+  int o = 0;
+  for (int q = 1; q < 3; ++q)
+    if (e2[q] * e2[(q + 2) % 3] < e2[o] * e2[(o + 2) % 3]) o = q;
+  const int p1 = (o + 1) % 3, p2 = (o + 2) % 3;
+  for (int d = 0; d < 3; ++d) dot += (v[3 * p1 + d] - v[3 * o + d]) * (v[3 * p2 + d] - v[3 * o + d]);
+  const double aacc = e2[o] * e2[p2];
+  const float len = __double2float_ru(sqrt(fmax(e2[0], fmax(e2[1], e2[2]))) * (1.0 + 1e-6));
+  const float sliver = aacc - dot * dot >= 1e-3 * aacc && fmin(e2[o], e2[p2]) > 1e-8 ? 0.f : 1.f;
+  const int ord[3] = {o, p1, p2};
+  const float w[3] = {len, sliver, 0.f};
+  for (int q = 0; q < 3; ++q) {
+    const double *p = v + 3 * ord[q];
+    tf[3 * t + q] = make_float4((float)p[0], (float)p[1], (float)p[2], w[q]);
+  }
 }
 
 __global__ void k_gather_tris(const double *verts, const int *tris, int ntri, double *tv) {
@@ -1335,8 +1603,8 @@ ibm_status membrane_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
     k_mem_scatter<<<nb, GM_THREADS, 0, st>>>(T->cut, T->cside, ncell, bo, T->gcell, T->gside, T->gkeys);
     float4 *blo = nullptr, *bhi = nullptr, *cen = nullptr;
     MTRY(S.get(&blo, ntri)); MTRY(S.get(&bhi, ntri)); MTRY(S.get(&cen, ntri));
-    k_tri_boxes<<<nblk(ntri, 128), 128, 0, st>>>(tv, ntri, blo, bhi, cen);
-    GhostArgs ga;
+    k_tri_boxes<<<nblk(ntri, 128), 128, 0, st>>>(tv, ntri, blo, bhi, cen, nullptr);
+    GhostArgs ga{};
     MTRY(build_bins(S, tv, ntri, ts, st, ga.bins));
     ga.nx = nx; ga.ny = ny; ga.nz = nz;
     ga.xc = dc[0]; ga.yc = dc[1]; ga.zc = dc[2];
@@ -1524,8 +1792,13 @@ ibm_status classify_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
                                                     tv + 9LL * tbase[m]);
       ts.add(meshes[m]);
     }
-    k_tri_boxes<<<nblk(tottris, 128), 128, 0, st>>>(tv, (int)tottris, blo, bhi, cen);
-    GhostArgs ga;
+    float4 *tf = nullptr;
+    CTRY(S.get(&tf, 3 * (size_t)tottris));
+    k_tri_boxes<<<nblk(tottris, 128), 128, 0, st>>>(tv, (int)tottris, blo, bhi, cen, tf);
+    GhostArgs ga{};
+    ga.tf = tf;
+    CTRY(S.get(&ga.cand, (size_t)CAND_OUT * ng));
+    CTRY(S.get(&ga.ncand, (size_t)ng));
     CTRY(build_bins(S, tv, (int)tottris, ts, st, ga.bins));
     ga.nx = nx; ga.ny = ny; ga.nz = nz;
     ga.xc = dc[0]; ga.yc = dc[1]; ga.zc = dc[2];
@@ -1536,7 +1809,8 @@ ibm_status classify_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
     ga.bi = T->gbi; ga.ip = T->gip; ga.w = T->gw; ga.scale = T->gscale;
     ga.base = T->gbase; ga.flags = T->gflags; ga.ref = T->gref;
     ga.kappa = T->gkappa; ga.tri = T->gtri; ga.wself = T->gwself;
-    k_ghost_tables<<<nblk(32 * ng, TABLE_THREADS), TABLE_THREADS, 0, st>>>(ga);
+    k_ghost_candidates<<<nblk(32 * ng, TABLE_THREADS), TABLE_THREADS, 0, st>>>(ga);
+    k_ghost_tables<<<nblk(ng, TABLE_THREADS), TABLE_THREADS, 0, st>>>(ga);
     CTRY(cudaGetLastError());
   }
   unsigned long long hc[2];
@@ -1548,7 +1822,7 @@ ibm_status classify_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
   T->nsolid = (long long)hc[1];
   CTRY(S.finish());
   T->geom_version += 1;
-  ctx->launches += 2 + 2 * (long long)nmesh * 3 + 5 + (T->nghost > 0 ? 5 + (long long)nmesh : 0);
+  ctx->launches += 2 + 2 * (long long)nmesh * 3 + 5 + (T->nghost > 0 ? 6 + (long long)nmesh : 0);
 #undef CTRY
   if (hleak) return IBM_ERR_MESH_NOT_CLOSED;
   return T->nfluid == 0 ? IBM_ERR_NO_FLUID : IBM_OK;

@@ -68,3 +68,31 @@ def test_ghost_compaction_by_grid_size(ctx, shape):
     assert np.array_equal(ex["iblank"], ib)
     assert np.array_equal(ex["cell"], np.flatnonzero(ib.ravel() == 3))
     T.close()
+
+
+@pytest.mark.parametrize("case", ["cone", "fine_mesh", "coarse_mesh", "far_coordinates", "tiny_triangles", "boxes"])
+def test_closest_triangle_search(ctx, case):
+    """Boundary intercepts bit for bit the oracle's: slivers, many triangles per cell, many cells
+    per triangle, coordinates near the limit of 4, edges below the FP32 bounds' range, flat faces
+    with equally near triangles."""
+    pkg, c = ctx
+    n, lo, hi = 24, 0.0, 1.0
+    if case == "cone":
+        meshes = [_double_cone(150)]
+    elif case == "fine_mesh":
+        n, meshes = 14, [synth.octa_sphere(5, (0.5, 0.49, 0.51), 0.3)]
+    elif case == "coarse_mesh":
+        n, meshes = 40, [synth.octa_sphere(0, (0.5, 0.49, 0.51), 0.33)]
+    elif case == "far_coordinates":
+        lo, hi = 3.0, 4.0
+        meshes = [synth.ellipsoid(4, (0.2, 0.11, 0.08), 20.0, (3.52, 3.48, 3.51))]
+    elif case == "tiny_triangles":
+        lo, hi = 0.5, 0.504
+        meshes = [synth.octa_sphere(5, (0.50203, 0.50198, 0.50201), 0.0011)]
+    else:
+        meshes = [synth.box_mesh((0.1, 0.1, 0.1), (0.4, 0.45, 0.9)), synth.octa_sphere(3, (0.7, 0.5, 0.5), 0.17)]
+    f = lo + (hi - lo) * synth.faces_uniform(n)
+    _, T, ex, ib, G = classify_both(pkg, c, f, f, f, meshes)
+    assert len(G) > 20
+    assert_tables_equal(ex, ib, G)
+    T.close()
