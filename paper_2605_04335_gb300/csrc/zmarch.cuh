@@ -16,19 +16,25 @@
 // result is exactly one red half-sweep followed by one black half-sweep (deterministic,
 // independent of the tiling).
 //
-// Warps 0..6 own the tile, one row per warp and strip set: each thread keeps two strips of 4
-// consecutive x-cells (rows y and y + SR) in registers for planes q-2 .. q+1 (the rhs and
-// mask are read from shared memory by each pass).  Red
-// results go back to the plane's buffer (their y-neighbours in other warps read them in the
-// next step) and stay in the registers (the strip's black update two steps later reads its
-// z-1 neighbours there); black results go only to registers and global memory.
-// x-neighbours across strips move by warp shuffle; the two edge lanes of a row read the
-// ring from shared memory at a per-lane address, so the update is branch-free.  Warp 7 owns
-// the ring -- its two rows of 32 strips and its 14 red column cells per plane (coefficients
-// from a shared table) -- and issues the copies; its work per step is below a tile warp's,
-// so no warp of the tile waits for it at the barrier.  A red update reads only black cells and
-// a black update only red ones, so the in-place writes never change a value another thread
-// reads in the same step: one barrier per step suffices.
+// Warps 0..6 own the tile, two adjacent rows each: each thread keeps two strips of 4
+// consecutive x-cells (rows y and y + 1) in registers for planes q-2 .. q+1, so each strip is
+// the other's y-neighbour; the rows outside the pair and the x-neighbour beside each strip come
+// from the plane's shared buffer.  Red results go back to that buffer (other warps and lanes read
+// them in the next step) and stay in the registers (the strip's black update two steps later
+// reads its z-1 neighbours there); black results go only to registers and global memory.  A
+// plane's rhs and mask are read once, by its red pass, which keeps the black cells' share for
+// the next step.  Warp 7 owns the ring -- its two rows of 32 strips and its 14 red column cells
+// per plane (coefficients from a shared table) -- and issues the copies; its work per step is
+// below a tile warp's, so no warp of the tile waits for it at the barrier.  A red update reads
+// only black cells and a black update only red ones, so the in-place writes never change a value
+// another thread reads in the same step: one barrier per step suffices.
+//
+// Bound by the instructions and the shared-memory latency of a plane step (16 warps per SM; the
+// same traffic without the arithmetic runs at 0.92 of the copy bandwidth).  Rows y and y + 7 in a
+// thread (both outer rows of each strip from shared memory, x-neighbours by two shuffles and a
+// select, rhs and mask read by both passes, the division intrinsic) took 2853 us per sweep at
+// 1024^3, 364 us at 512^3 and 57 us at 256^3; this takes 2467, 312 and 49 us: 0.83, 0.82 and 0.65
+// of the measured copy bandwidth.  A third plane of prefetch (DP = 3) is slower: 2676 us.
 //
 // Coarse levels (COARSE = true) carry face fractions (the area fraction of open fine faces)
 // in their coefficients.  Their mask here is the z-march mask: 0 for a regular fluid cell
@@ -59,29 +65,28 @@ namespace ibm {
 namespace zm {
 
 constexpr int TX = 128;         // tile width (cells): 32 lanes x 4 cells
-constexpr int SR = 7;           // rows of one strip set: one per tile warp
-constexpr int NS = 2;           // interior strips per thread: rows y and y + SR
-constexpr int TY = SR * NS;     // tile height
+constexpr int NS = 2;           // interior strips per thread: rows y and y + 1
+constexpr int TILE_WARPS = 7;                  // NS rows of strips each
+constexpr int TY = TILE_WARPS * NS;            // tile height
 constexpr int BX = TX + 8;      // staged width of e and rhs: x in [-4, TX + 4)
 constexpr int BXM = TX + 16;    // staged width of the mask (an 8-bit box row must be 16-byte multiple)
 constexpr int EY = TY + 4;      // e rows: y in [-2, TY + 2)
 constexpr int RY = TY + 2;      // rhs / mask rows: y in [-1, TY + 1)
-constexpr int TILE_WARPS = SR;                 // one row of strips each
 constexpr int RING_WARP = TILE_WARPS;          // the ring and the copies
 constexpr int THREADS = (TILE_WARPS + 1) * 32;
 constexpr int MIN_CTAS = 2;
 constexpr int COL_LANES = TY;                  // ring warp lanes with a column cell (pairs of rows)
 static_assert(TX == 128 && THREADS == 256 && TY % 2 == 0 && COL_LANES <= 32,
               "a warp's 32 lanes cover one row of the tile; the ring warp's lanes its column cells");
-static_assert(NS == 2 && SR % 2 == 1, "strip 1 lies an odd number of rows below strip 0: the other colour");
+static_assert(NS == 2, "strip 1 is the row below strip 0: the other colour, and its neighbour");
 constexpr int WAIT_LIMIT = 1 << 22;
 constexpr int KZ_MAX = 256;     // planes per item at most (the z-coefficient table)
 
 // prefetch distance in planes; rings hold the planes in use at step q (e: q-1 .. q+1,
-// rhs/mask: q-1 and q) plus the ones in flight
+// rhs/mask: q) plus the ones in flight
 constexpr int DP = 2;
 constexpr int NE = 3 + DP;
-constexpr int NR = 2 + DP;
+constexpr int NR = 1 + DP;
 
 constexpr int pad128(int bytes) { return (bytes + 127) / 128 * 128; }
 template <typename T> constexpr int esz() { return pad128(EY * BX * (int)sizeof(T)) / (int)sizeof(T); }  // per e buffer
@@ -208,6 +213,13 @@ __device__ __forceinline__ vec4<T> make4(T a, T b, T c, T d) {
 // in a fixed order; the relaxation factor omega / D uses an approximate reciprocal (it does
 // not move the fixed point, the exact FP32 solution of the row).  Every path (tile strips,
 // ring strips, ring columns) calls this, so a ring cell gets the bits its owner computes.
+// omega x the hardware reciprocal (about 1 ulp; denormals as zero, which no diagonal is): two
+// instructions, where the division intrinsic guards against divisors above 2^126 with several.
+__device__ __forceinline__ float relax_factor(float om, float D) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(D));
+  return om * r;
+}
 __device__ __forceinline__ float relax1(float c, float w, float ea, float n, float s, float zm, float zp, float cxm,
                                        float cxp, float cym, float cyp, float czm, float czp, float D, float rsh,
                                        float om) {
@@ -218,7 +230,7 @@ __device__ __forceinline__ float relax1(float c, float w, float ea, float n, flo
   acc = fmaf(cyp, s, acc);
   acc = fmaf(czm, zm, acc);
   acc = fmaf(czp, zp, acc);
-  return fmaf(acc, __fdividef(om, D), c);
+  return fmaf(acc, relax_factor(om, D), c);
 }
 
 // The same cell in FP64 (the FP64 solve's smoother): the residual in FP64 in the same order; the
@@ -235,7 +247,7 @@ __device__ __forceinline__ double relax1(double c, double w, double ea, double n
   acc = fma(cyp, s, acc);
   acc = fma(czm, zm, acc);
   acc = fma(czp, zp, acc);
-  return fma(acc, dfl::widen(__fdividef(om, dfl::narrow_trunc(D))), c);
+  return fma(acc, dfl::widen(relax_factor(om, dfl::narrow_trunc(D))), c);
 }
 
 // z-march mask byte of an irregular coarse cell
@@ -265,43 +277,41 @@ struct XCoef {
   vec4<T> m, p, s;   // cxm, cxp, cxm + cxp
 };
 
-// Relax the cells u = UA and UA + 2 of strip C (a warp's strips share UA): west/east are the
-// cells left of u = 0 and right of u = 3, N/S the strip in rows y -1 / +1, Zm/Zp in planes
-// k -1 / +1, R the rhs, mm the mask bytes (nonzero: not updated, except IRREGULAR on coarse
+// Relax the cells u = UA and UA + 2 of strip C (a warp's strips share UA): edge is the cell left
+// of u = 0 (UA = 0) or right of u = 3 (UA = 1), N/S the strip in rows y -1 / +1, Zm/Zp in planes
+// k -1 / +1, ra and rb the two cells' rhs, mm the mask bytes (nonzero: not updated, except IRREGULAR on coarse
 // levels; invalid cells carry 0xff); gid the padded index of the strip's first cell (coarse
 // levels' fractions).  Called by all 32 lanes of a warp.
 template <int UA, bool COARSE, typename T>
-__device__ __forceinline__ void relax_strip(vec4<T> &C, T west, T east, const vec4<T> &N, const vec4<T> &S,
-                                            const vec4<T> &Zm, const vec4<T> &Zp, const vec4<T> &R, unsigned mm,
+__device__ __forceinline__ void relax_strip(vec4<T> &C, T edge, const vec4<T> &N, const vec4<T> &S,
+                                            const vec4<T> &Zm, const vec4<T> &Zp, T ra, T rb, unsigned mm,
                                             const XCoef<T> &X, T cym, T cyp, T syz, T czm, T czp, T sh, float om,
                                             const Args<T> &a, long long gid) {
   const T c0 = UA == 0 ? C.x : C.y, c1 = UA == 0 ? C.z : C.w;
-  const T w0 = UA == 0 ? west : C.x, e0 = UA == 0 ? C.y : C.z;
-  const T w1 = UA == 0 ? C.y : C.z, e1 = UA == 0 ? C.w : east;
+  const T w0 = UA == 0 ? edge : C.x, e0 = UA == 0 ? C.y : C.z;
+  const T w1 = UA == 0 ? C.y : C.z, e1 = UA == 0 ? C.w : edge;
   const T n0 = UA == 0 ? N.x : N.y, n1 = UA == 0 ? N.z : N.w, s0 = UA == 0 ? S.x : S.y, s1 = UA == 0 ? S.z : S.w;
   const T zm0 = UA == 0 ? Zm.x : Zm.y, zm1 = UA == 0 ? Zm.z : Zm.w;
   const T zp0 = UA == 0 ? Zp.x : Zp.y, zp1 = UA == 0 ? Zp.z : Zp.w;
-  const T r0 = (UA == 0 ? R.x : R.y) - sh, r1 = (UA == 0 ? R.z : R.w) - sh;
+  const T r0 = ra - sh, r1 = rb - sh;
   const T xm0 = UA == 0 ? X.m.x : X.m.y, xm1 = UA == 0 ? X.m.z : X.m.w;
   const T xp0 = UA == 0 ? X.p.x : X.p.y, xp1 = UA == 0 ? X.p.z : X.p.w;
   const T xs0 = UA == 0 ? X.s.x : X.s.y, xs1 = UA == 0 ? X.s.z : X.s.w;
   T v0 = relax1(c0, w0, e0, n0, s0, zm0, zp0, xm0, xp0, cym, cyp, czm, czp, xs0 + syz, r0, om);
   T v1 = relax1(c1, w1, e1, n1, s1, zm1, zp1, xm1, xp1, cym, cyp, czm, czp, xs1 + syz, r1, om);
-  unsigned b0 = (mm >> (8 * UA)) & 0xffu, b1 = (mm >> (8 * (UA + 2))) & 0xffu;
+  constexpr unsigned B0 = 0xffu << (8 * UA), B1 = 0xffu << (8 * (UA + 2));
   if constexpr (COARSE) {
-    if (__any_sync(0xffffffffu, b0 == IRREGULAR || b1 == IRREGULAR)) {
-      if (b0 == IRREGULAR) {
-        v0 = relax_frac(a, gid + UA, c0, w0, e0, n0, s0, zm0, zp0, xm0, xp0, cym, cyp, czm, czp, r0, om);
-        b0 = 0u;
-      }
-      if (b1 == IRREGULAR) {
+    // irregular cells: bit 3 set and bit 0 not (the other bytes are 0, 1 and 0xff)
+    const unsigned irr = mm & ~(mm << 3) & (0x08080808u & (B0 | B1));
+    if (__any_sync(0xffffffffu, irr != 0u)) {
+      if (irr & B0) v0 = relax_frac(a, gid + UA, c0, w0, e0, n0, s0, zm0, zp0, xm0, xp0, cym, cyp, czm, czp, r0, om);
+      if (irr & B1)
         v1 = relax_frac(a, gid + UA + 2, c1, w1, e1, n1, s1, zm1, zp1, xm1, xp1, cym, cyp, czm, czp, r1, om);
-        b1 = 0u;
-      }
+      mm &= ~irr;
     }
   }
-  v0 = b0 ? c0 : v0;
-  v1 = b1 ? c1 : v1;
+  v0 = mm & B0 ? c0 : v0;
+  v1 = mm & B1 ? c1 : v1;
   if constexpr (UA == 0) {
     C.x = v0;
     C.z = v1;
@@ -354,22 +364,21 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
   const bool ring = warp == RING_WARP;
   const bool issuer = ring && lane == 0;
   const unsigned ebytes = EY * BX * sizeof(S), rbytes = RY * BX * sizeof(S) + RY * BXM;
-  // this thread's strips: tile warp w takes row w (strip 0) and row w + SR (strip 1), lane l
+  // this thread's strips: tile warp w takes rows 2 w (strip 0) and 2 w + 1 (strip 1), lane l
   // the cells 4 l .. 4 l + 3, so the lanes of a warp share each strip's colour parity.  The
   // ring warp's lanes take the ring strips at x = 4 l of rows -1 and TY, and lanes
   // l < COL_LANES the column cell x = -1 (l < TY / 2) or TX (the rest), the red one of the
   // pair of rows 2 (l mod TY / 2), 2 (l mod TY / 2) + 1.
   const int xs = 4 * lane;
-  const int ys = ring ? 0 : warp;
+  const int ys = ring ? 0 : NS * warp;
   const int ie0 = (ys + 2) * BX + (xs + 4), ir0 = (ys + 1) * BX + (xs + 4), im0 = (ys + 1) * BXM + (xs + 4);
-  const int eoff = lane == 0 ? -1 : 4;   // edge lanes: the ring cell beside the strip
   // coefficients of this thread's strips (registers for the item's whole march)
   const XCoef<T> X = load_x(a, x0 + xs);
   T cym[NS], cyp[NS], sy[NS];
   unsigned inval[NS];
 #pragma unroll
   for (int t = 0; t < NS; ++t) {
-    const int gj = y0 + ys + SR * t;
+    const int gj = y0 + ys + t;
     const bool jok = gj < a.ny;
     inval[t] = invalid_bytes(x0 + xs, a.nx, jok);
     cym[t] = jok ? a.cym[gj] : (T)0;
@@ -446,7 +455,7 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
   // for e plane q+1 and rhs/mask plane q and, after the step's barrier (so no thread still
   // reads the buffers being refilled), prefetches e plane q+1+DP (into the buffer of plane
   // q-2, last read in step q-1) and rhs/mask plane q+DP (buffer of plane q-2, last read by
-  // the black pass of step q-1).  Every load is issued once and waited for once.
+  // the red pass of step q-1).  Every load is issued once and waited for once.
   if (issuer) {
     fence_proxy_async();
     for (int pl = k0 - 2, b = se0; pl <= min(k0 - 1 + DP, k1 + 1); ++pl, b = wrap_e(b + 1)) load_e(pl, b);
@@ -460,10 +469,13 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
   vec4<T> Cm2[NS], Cm1[NS], C0[NS];
 #pragma unroll
   for (int t = 0; t < NS; ++t) {
-    Cm1[t] = lds4(s.e[se0] + ie0 + SR * t * BX);
-    C0[t] = lds4(s.e[sq] + ie0 + SR * t * BX);
+    Cm1[t] = lds4(s.e[se0] + ie0 + t * BX);
+    C0[t] = lds4(s.e[sq] + ie0 + t * BX);
     Cm2[t] = Cm1[t];
   }
+  // the rhs of the strips' black cells and their mask bytes in plane q-1, kept from its red pass
+  T Ra[NS] = {(T)0, (T)0}, Rb[NS] = {(T)0, (T)0};
+  unsigned mk[NS] = {0xffffffffu, 0xffffffffu};
   S *const dst0 = static_cast<S *>(a.out) + (long long)(y0 + ys + 1) * a.px + (x0 + xs + 4);
   // not unrolled: with the coarse levels' irregular-cell path, three copies of the step
   // overflow the instruction cache (measured: most stalls waiting for instructions), and the
@@ -484,71 +496,93 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
     }
     S *P = s.e[sq], *Pm = s.e[sm1];
     const S *Pp = s.e[sp1];
-    const int rqm = rq == 0 ? NR - 1 : rq - 1;   // rhs/mask slot of plane q-1
-    const S *R = s.r[rq], *Rm = s.r[rqm];
-    const uint8_t *M = s.m[rq], *Mm = s.m[rqm];
+    const S *R = s.r[rq];
+    const uint8_t *M = s.m[rq];
     // z coefficients of planes q (red pass) and q-1 (black pass)
     const ZC<T> zq = s.zc[q - (k0 - 2)], zb = s.zc[q - 1 - (k0 - 2)];
     const T zmr = zq.m, zpr = zq.p, szr = zq.s, zmb = zb.m, zpb = zb.p, szb = zb.s;
     const bool red = q >= 0 && q < a.nz;
-    // x0 + xs is even: strip t relaxes u = (y0 + ys + SR t + q) & 1 (SR is odd, so strip 1 has
-    // the other colour of strip 0)
+    // x0 + xs is even: strip t relaxes u = (y0 + ys + t + q) & 1
     const bool parq = ((y0 + ys + q) & 1) == 0;
     vec4<T> U[NS];   // the strips in plane q+1
 #pragma unroll
-    for (int t = 0; t < NS; ++t) U[t] = lds4(Pp + ie0 + SR * t * BX);
+    for (int t = 0; t < NS; ++t) U[t] = lds4(Pp + ie0 + t * BX);
     // red cells of strip t of plane q (ua: its colour's u, a compile-time constant):
-    // x-edges from the adjacent lanes, or the ring at the edges
-    // In FP32 a pass gathers both strips' inputs (x-edges, the rows above and below, rhs,
-    // mask) before relaxing either, so the shared-memory loads of the two strips overlap (the
-    // kernel's main stall is their latency); the FP64 form, bound by the FP64 pipe and short
-    // of registers, takes one strip at a time.
+    // the x-neighbour beside the strip from the plane's buffer; each strip is the other's
+    // y-neighbour (a pass relaxes cells of one colour, so neither reads a value that the other's
+    // update changes), the outer rows come from shared memory.
+    // In FP32 a pass gathers both strips' inputs before relaxing either, so the shared-memory
+    // loads of the two strips overlap; the FP64 form, bound by the FP64 pipe and short of
+    // registers, takes one strip at a time.
     struct In {
-      T w, e;
-      vec4<T> N, So, Rr;
+      T edge;
+      vec4<T> out;   // the row above strip 0, or below strip 1
+      T ra, rb;      // the rhs of the cells to relax, and the mask bytes
       unsigned mm;
     };
-    auto red_load = [&](const int t) {
-      const int ie = ie0 + SR * t * BX;
+    auto gather = [&](auto ua, const S *Q, const int t) {
       In in;
-      const T ep = ld1(P + ie + eoff);
-      T w = __shfl_up_sync(0xffffffffu, C0[t].w, 1);
-      T e = __shfl_down_sync(0xffffffffu, C0[t].x, 1);
-      in.w = lane == 0 ? ep : w;
-      in.e = lane == 31 ? ep : e;
-      in.N = lds4(P + ie - BX);
-      in.So = lds4(P + ie + BX);
-      in.Rr = lds4(R + ir0 + SR * t * BX);
-      in.mm = *reinterpret_cast<const unsigned *>(M + im0 + SR * t * BXM) | inval[t];
+      in.edge = ld1(Q + ie0 + t * BX + (decltype(ua)::value == 0 ? -1 : 4));
+      in.out = lds4(Q + ie0 + (t == 0 ? -BX : 2 * BX));
+      return in;
+    };
+    // red cells at u = UA and UA + 2; the black ones' rhs and the mask bytes replace plane q-1's
+    auto red_load = [&](auto ua, const int t) {
+      In in = gather(ua, P, t);
+      const vec4<T> r = lds4(R + ir0 + t * BX);
+      in.mm = mk[t] = *reinterpret_cast<const unsigned *>(M + im0 + t * BXM) | inval[t];
+      constexpr bool even = decltype(ua)::value == 0;
+      in.ra = even ? r.x : r.y;
+      in.rb = even ? r.z : r.w;
+      Ra[t] = even ? r.y : r.x;
+      Rb[t] = even ? r.w : r.z;
       return in;
     };
     auto red_do = [&](auto ua, const int t, const In &in) {
-      const int ie = ie0 + SR * t * BX;
-      const long long gid = (long long)(q + 1) * a.sz + (long long)(y0 + ys + SR * t + 1) * a.sy + (x0 + xs + 4);
-      relax_strip<decltype(ua)::value, COARSE>(C0[t], in.w, in.e, in.N, in.So, Cm1[t], U[t], in.Rr, in.mm, X, cym[t],
-                                               cyp[t], sy[t] + szr, zmr, zpr, sh, om, a, gid);
+      const long long gid = (long long)(q + 1) * a.sz + (long long)(y0 + ys + t + 1) * a.sy + (x0 + xs + 4);
+      relax_strip<decltype(ua)::value, COARSE>(C0[t], in.edge, t == 0 ? in.out : C0[0], t == 0 ? C0[1] : in.out,
+                                               Cm1[t], U[t], in.ra, in.rb, in.mm, X, cym[t], cyp[t], sy[t] + szr,
+                                               zmr, zpr, sh, om, a, gid);
       C0[t] = stored4<S>(C0[t]);   // the registers hold what every reader of the buffer sees
-      sts4(P + ie, C0[t]);
+      sts4(P + ie0 + t * BX, C0[t]);
     };
-    if (!ring && red) {
-      if constexpr (sizeof(T) == 4) {
-        const In i0 = red_load(0), i1 = red_load(1);
-        if (parq) {
-          red_do(U0{}, 0, i0);
-          red_do(U1{}, 1, i1);
+    // black cells of plane q-1: neighbours all red, updated by now (in-plane ones in
+    // shared memory and the other strip, the z-neighbours in Cm2 and C0); store the strips from
+    // registers.  They sit at the same u as the red cells of plane q.  Their rhs and mask are
+    // taken before the red pass of plane q replaces them.
+    const int kb = q - 1;
+    const T Ka[NS] = {Ra[0], Ra[1]}, Kb[NS] = {Rb[0], Rb[1]};
+    const unsigned km[NS] = {mk[0], mk[1]};
+    auto black_do = [&](auto ua, const int t, const In &in, S *const dk) {
+      const long long gid = (long long)q * a.sz + (long long)(y0 + ys + t + 1) * a.sy + (x0 + xs + 4);
+      relax_strip<decltype(ua)::value, COARSE>(Cm1[t], in.edge, t == 0 ? in.out : Cm1[0], t == 0 ? Cm1[1] : in.out,
+                                               Cm2[t], C0[t], Ka[t], Kb[t], km[t], X, cym[t], cyp[t], sy[t] + szb, zmb,
+                                               zpb, sh, om, a, gid);
+      if ((inval[t] & 0xffu) == 0u) {   // the strip's row is in the grid
+        S *dst = dk + (long long)t * a.px;
+        if (inval[t] == 0u) {
+          sts4(dst, Cm1[t]);
         } else {
-          red_do(U1{}, 0, i0);
-          red_do(U0{}, 1, i1);
-        }
-      } else {
-        if (parq) {
-          red_do(U0{}, 0, red_load(0));
-          red_do(U1{}, 1, red_load(1));
-        } else {
-          red_do(U1{}, 0, red_load(0));
-          red_do(U0{}, 1, red_load(1));
+          if (!(inval[t] & 0xff00u)) st1(dst + 1, Cm1[t].y);
+          if (!(inval[t] & 0xff0000u)) st1(dst + 2, Cm1[t].z);
+          if (!(inval[t] & 0xff000000u)) st1(dst + 3, Cm1[t].w);
+          st1(dst, Cm1[t].x);
         }
       }
+    };
+    if (!ring && red) {
+      auto pass = [&](auto u0, auto u1) {
+        if constexpr (sizeof(T) == 4) {
+          const In i0 = red_load(u0, 0), i1 = red_load(u1, 1);
+          red_do(u0, 0, i0);
+          red_do(u1, 1, i1);
+        } else {
+          red_do(u0, 0, red_load(u0, 0));
+          red_do(u1, 1, red_load(u1, 1));
+        }
+      };
+      if (parq) pass(U0{}, U1{});
+      else pass(U1{}, U0{});
     }
     if (ring && red) {
       // ring row strips (rows -1 and TY, this lane's x): red cells of plane q, in place
@@ -561,17 +595,12 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
         const vec4<T> N = lds4(P + iq0 - BX), So = lds4(P + iq0 + BX), Zm = lds4(Pm + iq0), Zp = lds4(Pp + iq0);
         const vec4<T> Rr = lds4(R + irq0);
         const unsigned mm = *reinterpret_cast<const unsigned *>(M + imq0) | s.ccu[lane][h];
-        const T ep = ld1(P + iq0 + eoff);
-        T w = __shfl_up_sync(0xffffffffu, C.w, 1);
-        T e = __shfl_down_sync(0xffffffffu, C.x, 1);
-        w = lane == 0 ? ep : w;
-        e = lane == 31 ? ep : e;
         const long long gid = (long long)(q + 1) * a.sz + (long long)(y0 + yr + 1) * a.sy + (x0 + xs + 4);
         if (((y0 + yr + q) & 1) == 0)
-          relax_strip<0, COARSE>(C, w, e, N, So, Zm, Zp, Rr, mm, X, cc[0], cc[1], cc[2] + szr, zmr, zpr, sh, om,
+          relax_strip<0, COARSE>(C, ld1(P + iq0 - 1), N, So, Zm, Zp, Rr.x, Rr.z, mm, X, cc[0], cc[1], cc[2] + szr, zmr, zpr, sh, om,
                                  a, gid);
         else
-          relax_strip<1, COARSE>(C, w, e, N, So, Zm, Zp, Rr, mm, X, cc[0], cc[1], cc[2] + szr, zmr, zpr, sh, om,
+          relax_strip<1, COARSE>(C, ld1(P + iq0 + 4), N, So, Zm, Zp, Rr.y, Rr.w, mm, X, cc[0], cc[1], cc[2] + szr, zmr, zpr, sh, om,
                                  a, gid);
         sts4(P + iq0, C);
       }
@@ -599,60 +628,20 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
         if (((s.ccu[lane][2] >> h) & 1u) && mb == 0u) st1(P + ic, v);
       }
     }
-    // black cells of plane q-1: neighbours all red, updated by now (in-plane ones in
-    // shared memory, the z-neighbours in Cm2 and C0); store the strips from registers
-    const int kb = q - 1;
-    // black cells of strip t of plane q-1 (they sit at the same u as the red cells of plane q)
-    auto black_load = [&](const int t) {
-      const int ie = ie0 + SR * t * BX;
-      In in;
-      const T ep = ld1(Pm + ie + eoff);
-      T w = __shfl_up_sync(0xffffffffu, Cm1[t].w, 1);
-      T e = __shfl_down_sync(0xffffffffu, Cm1[t].x, 1);
-      in.w = lane == 0 ? ep : w;
-      in.e = lane == 31 ? ep : e;
-      in.N = lds4(Pm + ie - BX);
-      in.So = lds4(Pm + ie + BX);
-      in.Rr = lds4(Rm + ir0 + SR * t * BX);
-      in.mm = *reinterpret_cast<const unsigned *>(Mm + im0 + SR * t * BXM) | inval[t];
-      return in;
-    };
-    auto black_do = [&](auto ua, const int t, const In &in, S *const dk) {
-      const long long gid = (long long)q * a.sz + (long long)(y0 + ys + SR * t + 1) * a.sy + (x0 + xs + 4);
-      relax_strip<decltype(ua)::value, COARSE>(Cm1[t], in.w, in.e, in.N, in.So, Cm2[t], C0[t], in.Rr, in.mm, X,
-                                               cym[t], cyp[t], sy[t] + szb, zmb, zpb, sh, om, a, gid);
-      if ((inval[t] & 0xffu) == 0u) {   // the strip's row is in the grid
-        S *dst = dk + (long long)(SR * t) * a.px;
-        if (inval[t] == 0u) {
-          sts4(dst, Cm1[t]);
-        } else {
-          if (!(inval[t] & 0xff00u)) st1(dst + 1, Cm1[t].y);
-          if (!(inval[t] & 0xff0000u)) st1(dst + 2, Cm1[t].z);
-          if (!(inval[t] & 0xff000000u)) st1(dst + 3, Cm1[t].w);
-          st1(dst, Cm1[t].x);
-        }
-      }
-    };
     if (!ring && kb >= k0 && kb < k1) {
       S *const dk = dst0 + (long long)(kb + 1) * a.sz;
-      if constexpr (sizeof(T) == 4) {
-        const In i0 = black_load(0), i1 = black_load(1);
-        if (parq) {
-          black_do(U0{}, 0, i0, dk);
-          black_do(U1{}, 1, i1, dk);
+      auto pass = [&](auto u0, auto u1) {
+        if constexpr (sizeof(T) == 4) {
+          const In i0 = gather(u0, Pm, 0), i1 = gather(u1, Pm, 1);
+          black_do(u0, 0, i0, dk);
+          black_do(u1, 1, i1, dk);
         } else {
-          black_do(U1{}, 0, i0, dk);
-          black_do(U0{}, 1, i1, dk);
+          black_do(u0, 0, gather(u0, Pm, 0), dk);
+          black_do(u1, 1, gather(u1, Pm, 1), dk);
         }
-      } else {
-        if (parq) {
-          black_do(U0{}, 0, black_load(0), dk);
-          black_do(U1{}, 1, black_load(1), dk);
-        } else {
-          black_do(U1{}, 0, black_load(0), dk);
-          black_do(U0{}, 1, black_load(1), dk);
-        }
-      }
+      };
+      if (parq) pass(U0{}, U1{});
+      else pass(U1{}, U0{});
     }
 #pragma unroll
     for (int t = 0; t < NS; ++t) {
