@@ -52,6 +52,8 @@ struct LV {          // kernel-side view of one level
   const double *dx, *dy, *dz;
   const T *wx, *wy, *wz;     // widths in T
   const T *sdx, *sdy, *sdz;  // finest level: separable diagonal parts (else nullptr)
+  const uint8_t *zmask;      // 0 regular fluid, 8 irregular fluid (coarse levels), else not relaxed
+  const T *rdx, *rdy, *rdz;  // diagonal parts of the regular cells
 };
 
 template <typename T>
@@ -68,6 +70,9 @@ LV<T> view(const Level &L) {
   v.wx = w; v.wy = w ? w + L.g.nx : nullptr; v.wz = w ? w + L.g.nx + L.g.ny : nullptr;
   const T *d = (const T *)L.sdiag;
   v.sdx = d; v.sdy = d ? d + L.g.nx : nullptr; v.sdz = d ? d + L.g.nx + L.g.ny : nullptr;
+  v.zmask = L.zmask ? L.zmask : L.mask;
+  const T *z = L.zsd ? (const T *)L.zsd : d;
+  v.rdx = z; v.rdy = z ? z + L.g.nx : nullptr; v.rdz = z ? z + L.g.nx + L.g.ny : nullptr;
   return v;
 }
 
@@ -385,29 +390,127 @@ struct VGrid {
   __device__ __forceinline__ int gy() const { return ny; }
 };
 
-template <typename T, class G>
-__device__ __forceinline__ void rbgs_body(const LV<T> &v, T *e, const T *r, const double *shift, int colour, T omega,
-                                          const G &gr) {
-  int ti = gr.bx() * blockDim.x + threadIdx.x;
-  int j = gr.by(), k = gr.bz();
-  int i = 2 * ti + ((j + k + colour) & 1);
-  if (i >= v.nx) return;
-  long long id = vidx(v, i, j, k);
-  if (v.mask[id] != 0) return;
-  T c[6];
-  coefs(v, i, j, k, id, c);
-  T D = v.sdx ? (v.sdx[i] + v.sdy[j]) + v.sdz[k] : ((c[0] + c[1]) + (c[2] + c[3])) + (c[4] + c[5]);
-  if (D == (T)0) return;
-  T rhs = r[id] - (shift ? (T)(*shift) : (T)0);
-  T res = stencil_sum(v, e, id, c) - D * e[id] - rhs;
-  // FP32 relaxation step: the fixed point (res = 0 in T) is unchanged, FP64 work stays minimal
-  e[id] += (T)__fdividef((float)omega * (float)res, (float)D);
+// four consecutive cells of a row
+__device__ __forceinline__ void ld4v(const float *p, float v[4]) {
+  const float4 a = *reinterpret_cast<const float4 *>(p);
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void ld4v(const double *p, double v[4]) {
+  const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
 
-template <typename T>
-__global__ void k_rbgs(LV<T> v, T *e, const T *r, const double *shift, int colour, T omega) {
-  rbgs_body(v, e, r, shift, colour, omega, HwGrid{});
+// omega res / D in FP32 (the relaxation step: the fixed point, res = 0 in T, does not depend on
+// its rounding); FP64 arguments are narrowed and the result widened on the integer pipe
+__device__ __forceinline__ float relax_update(float e, float res, float D, float om) {
+  return fmaf(res, zm::relax_factor(om, D), e);
 }
+__device__ __forceinline__ double relax_update(double e, double res, double D, float om) {
+  return fma(res, dfl::widen(zm::relax_factor(om, dfl::narrow_trunc(D))), e);
+}
+
+// One colour of red-black Gauss-Seidel, in place, on every cell of colour (i + j + k) mod 2 of a
+// level: each thread relaxes the two cells of that colour in a strip of four x-cells, in KZ
+// consecutive planes.  Bound by latency (the levels it serves fit the L2, and the smallest launch
+// too few warps to fill the chip), so all loads of a thread -- whole strips, 16 bytes each in
+// FP32, and the planes above and below once -- are issued before the arithmetic, and strips are
+// numbered along x then y, so that short rows leave no lanes idle.  Regular cells (every
+// face with a coefficient fully open) take the rediscretised coefficients and the separable
+// diagonal, ten FP64 operations in the FP64 form; irregular ones (zmask 8) read their six face
+// fractions.  One cell per thread, blocks of 128 along x and six fractions for every coarse cell
+// took 75.7 us per launch over 48 problems' levels and 21.6 us in FP64 at 97 x 81 x 65; this
+// takes 55.8 and 13.4.
+constexpr int RELAX_THREADS = 128;
+template <class Geom>
+inline int relax_gx(const Geom &g) {   // blocks of strips per chunk of planes
+  return (int)((((long long)g.nx + 3) / 4 * g.ny + RELAX_THREADS - 1) / RELAX_THREADS);
+}
+template <typename T, int KZ, class G>
+__device__ __forceinline__ void relax_body(const LV<T> &v, T *e, const T *r, const double *shift, int colour, float om,
+                                           const G &gr) {
+  static_assert(KZ == 1 || KZ == 2, "the planes of one thread");
+  const int groups = (v.nx + 3) >> 2;
+  const int strip = gr.bx() * RELAX_THREADS + (int)threadIdx.x;
+  const int j = strip / groups, g = strip - j * groups, k0 = gr.by() * KZ;
+  if (j >= v.ny) return;
+  const T sh = shift ? (T)(*shift) : (T)0;
+  const long long id0 = vidx(v, 4 * g, j, k0);
+  T C[KZ + 2][4], N[KZ][4], S[KZ][4], R[KZ][4], edge[KZ], xm[4], xp[4], xd[4];
+  unsigned mm[KZ];
+  const bool more = KZ == 1 || k0 + 1 < v.nz;   // an odd level's last chunk has one plane
+#pragma unroll
+  for (int q = 0; q < KZ; ++q) {
+    const long long id = id0 + q * v.sz;
+    const bool in = q == 0 || more;
+    mm[q] = in ? *reinterpret_cast<const unsigned *>(v.zmask + id) : 0xffffffffu;
+    ld4v(e + id, C[q + 1]);   // plane nz is the halo
+    if (in) {
+      ld4v(e + id - v.sy, N[q]);
+      ld4v(e + id + v.sy, S[q]);
+      ld4v(r + id, R[q]);
+      edge[q] = ((j + k0 + q + colour) & 1) ? e[id + 4] : e[id - 1];
+    }
+  }
+  ld4v(e + id0 - v.sz, C[0]);
+  if (more) ld4v(e + id0 + KZ * v.sz, C[KZ + 1]);
+  const T cym = v.cym[j], cyp = v.cyp[j], sdy = v.rdy[j];
+  if constexpr (KZ == 1) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = min(4 * g + u, v.nx - 1);   // cells past nx: any valid index
+      xm[u] = v.cxm[i]; xp[u] = v.cxp[i]; xd[u] = v.rdx[i];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < KZ; ++q) {
+    const int k = min(k0 + q, v.nz - 1);
+    const T czm = v.czm[k], czp = v.czp[k], syz = sdy + v.rdz[k];
+    const int ua = (j + k0 + q + colour) & 1;   // the strip starts at an even x
+    auto pick = [&](const T (&a)[4], int h) { return ua ? a[2 * h + 1] : a[2 * h]; };
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // cell u = ua + 2 h
+      const unsigned m = (mm[q] >> (8 * (ua + 2 * h))) & 0xffu;
+      const bool live = m == 0u || m == zm::IRREGULAR;
+      if (KZ > 1 && !live) continue;
+      const T c = pick(C[q + 1], h);
+      // the neighbours to the left and right: inside the strip, or the one beside it
+      const T w = ua ? C[q + 1][2 * h] : (h ? C[q + 1][1] : edge[q]);
+      const T ea = ua ? (h ? edge[q] : C[q + 1][2]) : C[q + 1][2 * h + 1];
+      const int i = min(4 * g + ua + 2 * h, v.nx - 1);
+      T cf[6] = {KZ == 1 ? pick(xm, h) : v.cxm[i], KZ == 1 ? pick(xp, h) : v.cxp[i], cym, cyp, czm, czp};
+      T D = (KZ == 1 ? pick(xd, h) : v.rdx[i]) + syz;
+      if (m == zm::IRREGULAR) {   // coefficients scaled by the open fractions, the diagonal their sum
+        const long long id = id0 + q * v.sz + ua + 2 * h;
+        cf[0] = mul_rn(cf[0], v.fx[id - 1]); cf[1] = mul_rn(cf[1], v.fx[id]);
+        cf[2] = mul_rn(cf[2], v.fy[id - v.sy]); cf[3] = mul_rn(cf[3], v.fy[id]);
+        cf[4] = mul_rn(cf[4], v.fz[id - v.sz]); cf[5] = mul_rn(cf[5], v.fz[id]);
+        D = ((cf[0] + cf[1]) + (cf[2] + cf[3])) + (cf[4] + cf[5]);
+      }
+      T res = fma_t<T>(-D, c, -(pick(R[q], h) - sh));
+      res = fma_t<T>(cf[0], w, res);
+      res = fma_t<T>(cf[1], ea, res);
+      res = fma_t<T>(cf[2], pick(N[q], h), res);
+      res = fma_t<T>(cf[3], pick(S[q], h), res);
+      res = fma_t<T>(cf[4], pick(C[q], h), res);
+      res = fma_t<T>(cf[5], pick(C[q + 2], h), res);
+      // a cell with no open face keeps its value
+      if (live && D > (T)0) e[id0 + q * v.sz + ua + 2 * h] = relax_update(c, res, D, om);
+    }
+  }
+}
+
+template <typename T, int KZ>
+__global__ void __launch_bounds__(RELAX_THREADS) k_relax(LV<T> v, T *e, const T *r, const double *shift, int colour,
+                                                         float om) {
+  relax_body<T, KZ>(v, e, r, shift, colour, om, HwGrid{});
+}
+
+// planes per thread of a launch over `cells` cells: two in FP32 where the launch fills the chip
+// several times over (they halve the loads of z-neighbours: 48 against 84 us per colour at 256^3),
+// one below (more threads with less to do each: 2.5 us shorter at 2^18 cells) and in FP64, whose
+// wider registers leave two planes too few warps (20.6 against 13.4 us at 97 x 81 x 65)
+template <typename T>
+inline int relax_kz(long long cells) { return sizeof(T) == 4 && cells >= (1LL << 20) ? 2 : 1; }
 
 // ghost rows (Jacobi): gnew = sum_k w_k e[src_k] (+ rhs at the ghost cell)
 template <typename T, typename W, class G>
@@ -2278,8 +2381,13 @@ static void setup_zmarch(Hierarchy *h, void *e0, void *r0) {
 
 // Coarse levels swept by the fused z-march: levels >= 1 of at least ZM_COARSE_CELLS cells in
 // FP32 hierarchies whose finest level uses it.  Tensor maps over the level's e (both buffers),
-// r and z-march mask.
-constexpr long long ZM_COARSE_CELLS = 1LL << 18;
+// r and z-march mask.  Its traffic is half the two-launch relaxation's, but a tile that crosses a
+// body waits for face fractions in every plane step (a sweep of 256^3 cells around twelve
+// spheres takes 133 us, around none 49), which the relaxation's many warps hide: 96 us at 256^3
+// and 18 against 34 us at 128^3, whose data stay in L2; at 512^3 cells the fused sweep is faster
+// (600 against about 760 us).
+constexpr long long ZM_COARSE_CELLS = 1LL << 26;
+constexpr long long BF16_CELLS = 1LL << 18;   // with BF16 coarse storage: levels stored (and swept so) from here
 constexpr int ZM_COARSE_KZ = 64;   // planes per chunk of a coarse level's dynamic schedule at most
 
 // With BF16 coarse storage those levels' e and r maps are BF16 (the kernel's BF16 form); a
@@ -2407,7 +2515,7 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
     // the finest level's arrays end with one slot per membrane ghost entry; coarse levels
     // that the fused sweep takes store e and r in BF16 when asked
     const long long nel = l == 0 ? L.g.ntot + slotcap : L.g.ntot;
-    L.bf16 = h->coarse_bf16 && l >= 1 && (long long)nx * ny * nz >= ZM_COARSE_CELLS;
+    L.bf16 = h->coarse_bf16 && l >= 1 && (long long)nx * ny * nz >= BF16_CELLS;
     if (L.bf16) {
       HTRY(alloc_zero<bf16>(&L.e, nel, st));
       HTRY(alloc_zero<bf16>(&L.r, nel, st));
@@ -2434,21 +2542,23 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
   }
   h->nslot = h->lv[0].g.ntot + slotcap;
   HTRY(alloc_zero<int>((void **)&h->zcount, nl, st));
-  // coarse levels for the fused sweep: z-march mask, second e buffer, separable diagonals
-  if (sizeof(T) == 4)
-    for (int l = 1; l < nl; ++l) {
-      Level &L = h->lv[l];
-      if ((long long)L.g.nx * L.g.ny * L.g.nz < ZM_COARSE_CELLS) continue;
-      HTRY(cudaMalloc((void **)&L.zmask, L.g.ntot));
-      HTRY(cudaMemsetAsync(L.zmask, 1, L.g.ntot, st));
+  // coarse levels: mask of regular and irregular cells, separable diagonals of the regular ones;
+  // the ones swept by the fused sweep: a second e buffer
+  for (int l = 1; l < nl; ++l) {
+    Level &L = h->lv[l];
+    HTRY(cudaMalloc((void **)&L.zmask, L.g.ntot));
+    HTRY(cudaMemsetAsync(L.zmask, 1, L.g.ntot, st));
+    HTRY(cudaMalloc(&L.zsd, sizeof(T) * (L.g.nx + L.g.ny + L.g.nz)));
+    k_sdiag<T><<<nblk(L.g.nx + L.g.ny + L.g.nz, 128), 128, 0, st>>>((const T *)L.c1d, L.g.nx, L.g.ny, L.g.nz,
+                                                                    (T *)L.zsd);
+    HTRY(cudaGetLastError());
+    const long long cells = (long long)L.g.nx * L.g.ny * L.g.nz;
+    if (sizeof(T) == 4 && (L.bf16 || cells >= ZM_COARSE_CELLS)) {
       if (L.bf16) HTRY(alloc_zero<bf16>(&L.ealt, L.g.ntot, st));
       else HTRY(alloc_zero<T>(&L.ealt, L.g.ntot, st));
-      HTRY(cudaMalloc(&L.zsd, sizeof(T) * (L.g.nx + L.g.ny + L.g.nz)));
-      k_sdiag<T><<<nblk(L.g.nx + L.g.ny + L.g.nz, 128), 128, 0, st>>>((const T *)L.c1d, L.g.nx, L.g.ny, L.g.nz,
-                                                                      (T *)L.zsd);
-      HTRY(cudaGetLastError());
       L.zm = true;
     }
+  }
   for (int l = 0; l + 1 < nl; ++l) {
     Level &Fl = h->lv[l], &C = h->lv[l + 1];
     HTRY(alloc_zero<uint8_t>((void **)&C.inner, C.g.ntot, st));
@@ -2536,7 +2646,7 @@ static ibm_status refresh_geometry_t(ibm_tables *t, Hierarchy *h, cudaStream_t s
                                                   wf, wf + Fl.g.nx, wf + Fl.g.nx + Fl.g.ny, C.g, wc, wc + C.g.nx,
                                                   wc + C.g.nx + C.g.ny, (T *)C.fx, (T *)C.fy, (T *)C.fz,
                                                   l == 0 && t->membrane ? t->cut : nullptr);
-    if (C.zm) k_zmask<T><<<nblk(nc, 256), 256, 0, st>>>(view<T>(C), C.zmask);
+    k_zmask<T><<<nblk(nc, 256), 256, 0, st>>>(view<T>(C), C.zmask);
   }
   IBM_TRY(cudaGetLastError());
   // fluid volume and count per level (one read-back for all levels)
@@ -2802,7 +2912,8 @@ template <typename T>
 void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool fine, const T *ghost_rhs, int sweeps) {
   Level &L = S.h->lv[l];
   LV<T> v = view<T>(L);
-  dim3 grid(nblk((L.g.nx + 1) / 2, 128), L.g.ny, L.g.nz);
+  const int kz = relax_kz<T>((long long)L.g.nx * L.g.ny * L.g.nz);
+  const dim3 grid(relax_gx(L.g), (L.g.nz + kz - 1) / kz);
   for (int s = 0; s < sweeps; ++s) {
     const bool timed = fine && S.sweep_events && S.sweep_events->size() >= 2 * (size_t)(s + 1);
     if (timed) cudaEventRecord((*S.sweep_events)[2 * s], S.st);
@@ -2831,7 +2942,9 @@ void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool
       continue;
     } else {
       for (int colour = 0; colour < 2; ++colour)
-        k_rbgs<T><<<grid, 128, 0, S.st>>>(v, e, r, shift, colour, (T)S.omega);
+        if (kz == 1) k_relax<T, 1><<<grid, RELAX_THREADS, 0, S.st>>>(v, e, r, shift, colour, (float)S.omega);
+        else if constexpr (sizeof(T) == 4)
+          k_relax<T, 2><<<grid, RELAX_THREADS, 0, S.st>>>(v, e, r, shift, colour, (float)S.omega);
       if (timed) cudaEventRecord((*S.sweep_events)[2 * s + 1], S.st);
       S.ctx->launches += 2;
       if (fine) cut_relax<T>(S, e, e, r, shift);
@@ -2946,6 +3059,8 @@ LV<double> fine_view64(Hierarchy *h) {
   const double *d = c + 2 * (v.nx + v.ny + v.nz);
   v.sdx = d; v.sdy = d + v.nx; v.sdz = d + v.nx + v.ny;
   v.wx = v.wy = v.wz = nullptr;
+  v.zmask = v.mask;
+  v.rdx = v.sdx; v.rdy = v.sdy; v.rdz = v.sdz;
   return v;
 }
 
@@ -3464,7 +3579,7 @@ __device__ __forceinline__ VGrid vgrid(int lb, int gx, int gy) {
   return g;
 }
 
-struct PRbgs {
+struct PRelax {
   LV<float> v;
   float *e;
   const float *r;
@@ -3518,9 +3633,10 @@ static_assert(sizeof(BL<PProlong>) <= 32764 && sizeof(BL<PRestrict>) <= 32764, "
   const auto &p = L.p[q];                     \
   const int lb = (int)blockIdx.x - L.b0[q];
 
-__global__ void kb_rbgs(const __grid_constant__ BL<PRbgs> L, int colour, float omega) {
+template <int KZ>
+__global__ void __launch_bounds__(RELAX_THREADS) kb_relax(const __grid_constant__ BL<PRelax> L, int colour, float omega) {
   BL_BLOCK(L)
-  rbgs_body<float>(p.v, p.e, p.r, p.shift, colour, omega, vgrid(lb, p.gx, p.gy));
+  relax_body<float, KZ>(p.v, p.e, p.r, p.shift, colour, omega, vgrid(lb, p.gx, p.gy));
 }
 __global__ void kb_ghost_pp(const __grid_constant__ BL<PGhost> L) {
   BL_BLOCK(L)
@@ -3772,21 +3888,28 @@ void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
     std::vector<int> zg, rg;
     for (int i : grp) (lk_h(K, i)->lv[l].zm ? zg : rg).push_back(i);
     if (!zg.empty()) lk_zmarch(K, l, zg);
+    long long cells = 0;
+    for (int i : rg) {
+      const LevelGeom &g = lk_h(K, i)->lv[l].g;
+      cells += (long long)g.nx * g.ny * g.nz;
+    }
+    const int kz = relax_kz<float>(cells);
     for (int colour = 0; colour < 2; ++colour)
-      bl_launch<PRbgs>(rg,
+      bl_launch<PRelax>(rg,
                        [&](int i) {
                          const LevelGeom &g = lk_h(K, i)->lv[l].g;
-                         return (int)nblk((g.nx + 1) / 2, 128) * g.ny * g.nz;
+                         return relax_gx(g) * ((g.nz + kz - 1) / kz);
                        },
                        [&](int i) {
                          const Level &L = lk_h(K, i)->lv[l];
-                         PRbgs p;
+                         PRelax p;
                          p.v = view<float>(L); p.e = K.E[l][i]; p.r = lk_r(K, i, l); p.shift = lk_shift(K, i, l);
-                         p.gx = (int)nblk((L.g.nx + 1) / 2, 128); p.gy = L.g.ny;
+                         p.gx = relax_gx(L.g); p.gy = (L.g.nz + kz - 1) / kz;
                          return p;
                        },
-                       [&](const BL<PRbgs> &L, int b) {
-                         kb_rbgs<<<b, 128, 0, K.st>>>(L, colour, K.omega);
+                       [&](const BL<PRelax> &L, int b) {
+                         if (kz == 2) kb_relax<2><<<b, RELAX_THREADS, 0, K.st>>>(L, colour, K.omega);
+                         else kb_relax<1><<<b, RELAX_THREADS, 0, K.st>>>(L, colour, K.omega);
                          K.ctx->launches += 1;
                        });
   }

@@ -96,3 +96,26 @@ def test_closest_triangle_search(ctx, case):
     assert len(G) > 20
     assert_tables_equal(ex, ib, G)
     T.close()
+
+
+@pytest.mark.parametrize("shape", [(33, 18, 21), (34, 19, 20), (35, 17, 18), (65, 31, 40), (130, 12, 15), (24, 9, 70)])
+def test_solves_at_odd_sizes(ctx, shape):
+    """Every precision against the oracle's direct solve: rows of 1, 2 and 3 cells beyond a strip,
+    odd and even planes, long and short rows on the coarse levels."""
+    from oracle import solve as OS
+    pkg, c = ctx
+    n = max(shape)
+    f = [m / n * synth.faces_tanh(m, 1.5) for m in shape]
+    size = min(shape) / n
+    mid = [0.5 * m / n for m in shape]
+    mesh = synth.ellipsoid(3, (0.33 * size, 0.26 * size, 0.29 * size), 25.0, mid)
+    g, T, _, ib, G = classify_both(pkg, c, *f, [mesh])
+    b = synth.rhs_divergence(*f, 3)
+    p_o, _ = OS.solve_sparse(g, ib, G, b)
+    fl = ib == 0
+    for prec in (0, 1, 2):
+        p = torch.zeros(b.shape, dtype=torch.float64, device="cuda")
+        T.solve(torch.from_numpy(b).cuda(), p, 1e-11, pkg.SolveOpts(precision=prec))
+        err = np.linalg.norm((p.cpu().numpy() - p_o)[fl]) / np.linalg.norm(p_o[fl])
+        assert err < 1e-8, (prec, err)
+    T.close()
