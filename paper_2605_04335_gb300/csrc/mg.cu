@@ -33,7 +33,8 @@
 namespace ibm {
 
 constexpr int MAX_COARSE = 128;
-constexpr int PROLONG_KC = 32;          // coarse planes per thread of the prolongation's z-march
+constexpr int PROLONG_KC = 16;          // coarse planes per thread of the prolongation's z-march
+constexpr long long PROLONG_BPS = 16;   // its blocks per SM at least, while chunks can be shortened
 constexpr int RESTRICT_BLOCKS = 1216;   // restriction blocks (at most; one partial sum each; fixed width)
 constexpr size_t GJ_SMEM_MAX = 160 * 1024;   // coarsest Gauss-Jordan in shared memory up to this size
 
@@ -161,7 +162,9 @@ __global__ void k_mask_coarse(const uint8_t *mf, LevelGeom gf, uint8_t *mc, Leve
   mc[pidx(gc, I, J, K)] = m;
 }
 
-// inner[c] = 1 where cell c and its 26 neighbours (halo included) are all fluid
+// inner[c] = 1 where cell c and its 26 neighbours within the grid are all fluid (a child's weight on
+// a neighbour outside the grid is zero, so the prolongation's denominator is 1 there too; counting
+// the halo as solid took every warp that holds an end of a row through the masked sums)
 __global__ void k_inner(const uint8_t *m, LevelGeom g, uint8_t *inner) {
   long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (l >= (long long)g.nx * g.ny * g.nz) return;
@@ -171,7 +174,9 @@ __global__ void k_inner(const uint8_t *m, LevelGeom g, uint8_t *inner) {
   for (int dz = -1; dz <= 1; ++dz)
     for (int dy = -1; dy <= 1; ++dy)
       for (int dx = -1; dx <= 1; ++dx)
-        if (m[c + dz * g.sz + dy * g.sy + dx] != 0) ok = 0;
+        if ((unsigned)(i + dx) < (unsigned)g.nx && (unsigned)(j + dy) < (unsigned)g.ny &&
+            (unsigned)(k + dz) < (unsigned)g.nz && m[c + dz * g.sz + dy * g.sy + dx] != 0)
+          ok = 0;
   inner[c] = ok;
 }
 
@@ -588,19 +593,37 @@ template <> struct Pair<double> {
   }
 };
 
+// Threads along x of a block of 128 (log2): 128, 64 or 32, whichever leaves the fewest idle on
+// rows of n coarse cells; the others take further rows.
+inline int row_lg(int n) {
+  int best = 7;
+  for (int lg = 6; lg >= 5; --lg)
+    if ((n + (1 << lg) - 1) >> lg << lg < (n + (1 << best) - 1) >> best << best) best = lg;
+  return best;
+}
+
 // Restriction of the level-f residual to level c, one thread per coarse cell (I,J,K) with
-// coarse rows strided over blockIdx.y: rc = sum over the fluid children of V_f r_f / V_c,
+// coarse rows strided over blockIdx.y (2^lg threads along x, 128 / 2^lg rows per block): rc = sum over the fluid children of V_f r_f / V_c,
 // with r_f = r - shift - (A e)_f; ec = 0 (the coarse correction starts from zero); block
 // partials of sum V_c rc at partials[by * gx + bx] (block (bx, by) of a gx x gy grid).  Every load of a
 // coarse cell (the 2x2x2 children of e, r and mask and their 24 face neighbours) is issued
 // before the arithmetic; children past an odd fine extent are halo cells (mask 1) whose
-// outward neighbours are not read.
-template <typename T, typename SF, typename SC, class G>
+// outward neighbours are not read.  Regular children use the separable diagonal, irregular ones
+// (zmask 8, coarse levels only: the finest level's form holds no fractions and fewer registers)
+// their six face fractions.  HBM-bound at large sizes, latency-bound in practice: 2692 us at
+// 1024^3 (0.59 of the copy bandwidth for 10 bytes a cell), 43 us at 256^3, 374 us over the finest
+// levels of 48 problems of edges 64 to 192; with 128 threads along x and fractions for every coarse
+// child 2870, 46 and 562 us (and 149 against 128 us in FP64 at 193 x 161 x 129, bound by the FP64 pipe).
+// A z-march that keeps two fine planes in registers loads a third of the values but has half the
+// loads in flight: 4490 us at 1024^3.  The FP32 sum keeps its order: in a chain starting from D e the
+// rounding moved the 1024^3 solution by 1e-9.
+template <typename T, bool FINEST, typename SF, typename SC, class G>
 __device__ __forceinline__ void restrict8_body(const LV<T> &f, const SF *e, const SF *r, const double *shift,
-                                               const LV<T> &cv, SC *rc, SC *ec, double *partials, const G &gr) {
+                                               const LV<T> &cv, SC *rc, SC *ec, double *partials, int lg,
+                                               const G &gr) {
   __shared__ double sm[128];
   double acc_all = 0.0;
-  const int I = gr.bx() * blockDim.x + threadIdx.x;
+  const int I = (gr.bx() << lg) + ((int)threadIdx.x & ((1 << lg) - 1)), rpb = 128 >> lg;
   const T sh = shift ? (T)(*shift) : (T)0;
   const int crows = cv.ny * cv.nz;
   // the children's 1D coefficients: x parts fixed per thread, y and z parts per row
@@ -610,10 +633,10 @@ __device__ __forceinline__ void restrict8_body(const LV<T> &f, const SF *e, cons
   for (int a = 0; a < 2; ++a) {
     const int i = min(i0 + a, f.nx - 1);
     cxm[a] = f.cxm[i]; cxp[a] = f.cxp[i]; wxf[a] = f.wx[i];
-    sdx[a] = f.sdx ? f.sdx[i] : (T)0;
+    sdx[a] = f.rdx[i];
   }
   if (I < cv.nx)
-    for (int row = gr.by(); row < crows; row += gr.gy()) {
+    for (int row = gr.by() * rpb + ((int)threadIdx.x >> lg); row < crows; row += gr.gy() * rpb) {
       const int J = row % cv.ny, K = row / cv.ny;
       const long long ic = vidx(cv, I, J, K);
       const int j0 = 2 * J, k0 = 2 * K;
@@ -624,8 +647,8 @@ __device__ __forceinline__ void restrict8_body(const LV<T> &f, const SF *e, cons
         const int j = min(j0 + b, f.ny - 1), k = min(k0 + b, f.nz - 1);
         cym[b] = f.cym[j]; cyp[b] = f.cyp[j]; wyf[b] = f.wy[j];
         czm[b] = f.czm[k]; czp[b] = f.czp[k]; wzf[b] = f.wz[k];
-        sdy[b] = f.sdx ? f.sdy[j] : (T)0;
-        sdz[b] = f.sdx ? f.sdz[k] : (T)0;
+        sdy[b] = f.rdy[j];
+        sdz[b] = f.rdz[k];
       }
       const long long fb = vidx(f, i0, j0, k0);
       T E[2][2][2], R[2][2][2], XM[2][2], XP[2][2], YM[2][2], YP[2][2], ZM[2][2], ZP[2][2];
@@ -637,7 +660,7 @@ __device__ __forceinline__ void restrict8_body(const LV<T> &f, const SF *e, cons
           const long long q = fb + d * f.sz + b * f.sy;
           ld2(e + q, E[d][b]);
           ld2(r + q, R[d][b]);
-          M[d][b] = *reinterpret_cast<const uchar2 *>(f.mask + q);
+          M[d][b] = *reinterpret_cast<const uchar2 *>(f.zmask + q);
           XM[d][b] = ld1(e + q - 1);
           XP[d][b] = vx1 ? ld1(e + q + 2) : (T)0;
         }
@@ -660,30 +683,49 @@ __device__ __forceinline__ void restrict8_body(const LV<T> &f, const SF *e, cons
 #pragma unroll
       for (int d = 0; d < 2; ++d)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
+        for (int b = 0; b < 2; ++b) {
+          T row = (T)0;   // FP64: sum over the row's two children of dx_f r_f
 #pragma unroll
           for (int a = 0; a < 2; ++a) {
             const uint8_t m = a ? M[d][b].y : M[d][b].x;
-            const long long id = fb + d * f.sz + b * f.sy + a;
             T c[6] = {cxm[a], cxp[a], cym[b], cyp[b], czm[d], czp[d]};
-            if (f.fx) {
+            T D = (sdx[a] + sdy[b]) + sdz[d];
+            if (!FINEST && m == zm::IRREGULAR) {   // coarse levels near a body: face fractions
+              const long long id = fb + d * f.sz + b * f.sy + a;
               c[0] = mul_rn(c[0], f.fx[id - 1]); c[1] = mul_rn(c[1], f.fx[id]);
               c[2] = mul_rn(c[2], f.fy[id - f.sy]); c[3] = mul_rn(c[3], f.fy[id]);
               c[4] = mul_rn(c[4], f.fz[id - f.sz]); c[5] = mul_rn(c[5], f.fz[id]);
+              D = ((c[0] + c[1]) + (c[2] + c[3])) + (c[4] + c[5]);
             }
-            const T D = f.sdx ? (sdx[a] + sdy[b]) + sdz[d] : ((c[0] + c[1]) + (c[2] + c[3])) + (c[4] + c[5]);
             const T xm = a ? E[d][b][0] : XM[d][b], xp = a ? XP[d][b] : E[d][b][1];
             const T ym = b ? E[d][0][a] : YM[d][a], yp = b ? YP[d][a] : E[d][1][a];
-            const T zm = d ? E[0][b][a] : ZM[b][a], zp = d ? ZP[b][a] : E[1][b][a];
-            // the first product rounded on its own: every sum then has one product, fused into it
-            const T s = mul_rn(c[0], xm) + c[1] * xp + c[2] * ym + c[3] * yp + c[4] * zm + c[5] * zp;
-            const T res = (R[d][b][a] - sh) - (s - D * E[d][b][a]);
-            if (m == 0) acc += (wxf[a] * wyf[b]) * wzf[d] * res;
+            const T zl = d ? E[0][b][a] : ZM[b][a], zr = d ? ZP[b][a] : E[1][b][a];
+            const bool live = m == 0 || (!FINEST && m == zm::IRREGULAR);
+            if constexpr (sizeof(T) == 4) {
+              // the first product rounded on its own: every sum then has one product, fused into it
+              const T s = mul_rn(c[0], xm) + c[1] * xp + c[2] * ym + c[3] * yp + c[4] * zl + c[5] * zr;
+              const T res = (R[d][b][a] - sh) - (s - D * E[d][b][a]);
+              if (live) acc += (wxf[a] * wyf[b]) * wzf[d] * res;
+            } else {   // the fewest FP64 operations: one chain, the weights of a row applied once
+              T res = fma_t<T>(D, E[d][b][a], R[d][b][a] - sh);
+              res = fma_t<T>(-c[0], xm, res);
+              res = fma_t<T>(-c[1], xp, res);
+              res = fma_t<T>(-c[2], ym, res);
+              res = fma_t<T>(-c[3], yp, res);
+              res = fma_t<T>(-c[4], zl, res);
+              res = fma_t<T>(-c[5], zr, res);
+              if (live) row = fma_t<T>(wxf[a], res, row);
+            }
           }
+          if constexpr (sizeof(T) == 8) acc = fma_t<T>(wyf[b] * wzf[d], row, acc);
+        }
       const T vc = (cv.wx[I] * cv.wy[J]) * cv.wz[K];
       st1(rc + ic, cfl ? acc / vc : (T)0);
       st1(ec + ic, (T)0);
-      if (cfl) acc_all += (double)acc;
+      if (cfl) {
+        if constexpr (sizeof(T) == 4) acc_all += dfl::widen(acc);
+        else acc_all += acc;
+      }
     }
   sm[threadIdx.x] = acc_all;
   __syncthreads();
@@ -694,10 +736,10 @@ __device__ __forceinline__ void restrict8_body(const LV<T> &f, const SF *e, cons
   if (threadIdx.x == 0) partials[gr.by() * gr.gx() + gr.bx()] = sm[0];
 }
 
-template <typename T, typename SF = T, typename SC = T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1) k_restrict8(LV<T> f, const SF *e, const SF *r, const double *shift, LV<T> cv,
-                                                   SC *rc, SC *ec, double *partials) {
-  restrict8_body<T, SF, SC>(f, e, r, shift, cv, rc, ec, partials, HwGrid{});
+template <typename T, bool FINEST, typename SF = T, typename SC = T>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 && FINEST ? 5 : 4)
+    k_restrict8(LV<T> f, const SF *e, const SF *r, const double *shift, LV<T> cv, SC *rc, SC *ec, double *partials, int lg) {
+  restrict8_body<T, FINEST, SF, SC>(f, e, r, shift, cv, rc, ec, partials, lg, HwGrid{});
 }
 
 // deterministic sum of nb partials (stride `stride`, offset `off`) in one block
@@ -737,34 +779,41 @@ __global__ void k_finalize_shift(const double *partials, int nb, const double *f
 // renormalising denominator (sum of the weights of the fluid corners) is 1 where the whole
 // 3x3x3 block is fluid (inner flag), else summed the same way over the fluid indicator.
 // Children that are not fluid rows are left unchanged; rows past the fine extent (odd sizes)
-// are halo rows (mask 1), never updated.
+// are halo rows (mask 1), never updated.  Latency-bound: 2112 us at 1024^3 (0.72 of the copy
+// bandwidth for 9.6 bytes a fine cell), 35 us at 256^3, 270 us over the finest levels of 48 problems
+// of edges 64 to 192, 166 us in FP64 at 193 x 161 x 129; 2220, 44, 455 and 235 us with 128 threads
+// along x, weights converted at each use and the ends of every row in the masked sums.  Six blocks per
+// SM (no spills at 80 registers) beat eight.
 template <typename T, typename SC, typename SF, class G>
 __device__ __forceinline__ void prolong8_body(const LV<T> &cv, const SC *ec, const uint8_t *inner, const LV<T> &f,
                                               SF *ef, const int8_t *offx, const int8_t *offy, const int8_t *offz,
-                                              const float *tx, const float *ty, const float *tz, int kc,
+                                              const float *tx, const float *ty, const float *tz, int kc, int lg,
                                               const G &gr) {
-  const int I = gr.bx() * blockDim.x + threadIdx.x, J = gr.by();
+  const int I = (gr.bx() << lg) + ((int)threadIdx.x & ((1 << lg) - 1)),
+            J = gr.by() * (128 >> lg) + ((int)threadIdx.x >> lg);
   const int K0 = gr.bz() * kc, K1 = min(cv.nz, K0 + kc);
-  if (I >= cv.nx || K0 >= K1) return;
-  auto axis = [](int c0, int nf, const int8_t *off, const float *t, float w[2][3]) {
+  if (I >= cv.nx || J >= cv.ny || K0 >= K1) return;
+  // w[a][1] the parent's weight, w[0][0] and w[1][2] the neighbour's; FP64 forms widen them here, on
+  // the integer pipe (a conversion at each use would fill the FP64 pipe)
+  auto axis = [](int c0, int nf, const int8_t *off, const float *t, T w[2][3]) {
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
       const bool v = c0 + a < nf;
       const int o = v ? off[c0 + a] : 0;
       const float tt = v ? t[c0 + a] : 0.f;
-      w[a][0] = o < 0 ? tt : 0.f;
-      w[a][1] = 1.f - tt;
-      w[a][2] = o > 0 ? tt : 0.f;
+      const float l = o < 0 ? tt : 0.f, m = 1.f - tt, r = o > 0 ? tt : 0.f;
+      if constexpr (sizeof(T) == 4) { w[a][0] = l; w[a][1] = m; w[a][2] = r; }
+      else { w[a][0] = dfl::widen(l); w[a][1] = dfl::widen(m); w[a][2] = dfl::widen(r); }
     }
   };
-  float wx[2][3], wy[2][3];
+  T wx[2][3], wy[2][3];
   axis(2 * I, f.nx, offx, tx, wx);
   axis(2 * J, f.ny, offy, ty, wy);
   // The first child of a coarse cell lies left of its centre and the second right (the coarse
   // faces are every other fine face), so child 0 weighs columns 0 and 1 and child 1 columns 1
   // and 2: two terms per child, the third weight being zero.
-  auto two = [](const float (&w)[2][3], int a, T v0, T v1, T v2) {
-    return a == 0 ? fma_t<T>((T)w[0][1], v1, (T)w[0][0] * v0) : fma_t<T>((T)w[1][2], v2, (T)w[1][1] * v1);
+  auto two = [](const T (&w)[2][3], int a, T v0, T v1, T v2) {
+    return a == 0 ? fma_t<T>(w[0][1], v1, w[0][0] * v0) : fma_t<T>(w[1][2], v2, w[1][1] * v1);
   };
   // x then y contraction of a 3x3 neighbourhood: o[a][b] for children a (x) and b (y)
   auto contract_xy = [&](const T (&v)[3][3], T (&o)[2][2]) {
@@ -807,7 +856,7 @@ __device__ __forceinline__ void prolong8_body(const LV<T> &cv, const SC *ec, con
     const long long c0 = vidx(cv, I, J, K);
     const bool inr = inner[c0] != 0;
     plane(K + 1, pp);
-    float wz[2][3];
+    T wz[2][3];
     axis(2 * K, f.nz, offz, tz, wz);
     T num[2][2][2], den[2][2][2];
 #pragma unroll
@@ -859,10 +908,10 @@ __device__ __forceinline__ void prolong8_body(const LV<T> &cv, const SC *ec, con
 }
 
 template <typename T, typename SC = T, typename SF = T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 4)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 5)
     k_prolong8(LV<T> cv, const SC *ec, const uint8_t *inner, LV<T> f, SF *ef, const int8_t *offx,
-               const int8_t *offy, const int8_t *offz, const float *tx, const float *ty, const float *tz, int kc) {
-  prolong8_body<T, SC, SF>(cv, ec, inner, f, ef, offx, offy, offz, tx, ty, tz, kc, HwGrid{});
+               const int8_t *offy, const int8_t *offz, const float *tx, const float *ty, const float *tz, int kc, int lg) {
+  prolong8_body<T, SC, SF>(cv, ec, inner, f, ef, offx, offy, offz, tx, ty, tz, kc, lg, HwGrid{});
 }
 
 // ------------------------------------------------------------------ coarse tail
@@ -2616,8 +2665,10 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
   // one wave of the row-strided restriction
   {
     int sms = t->ctx->sm_count > 0 ? t->ctx->sm_count : 152, pr = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pr, k_restrict8<T>, 128, 0) != cudaSuccess || pr < 1) pr = 4;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pr, k_restrict8<T, true>, 128, 0) != cudaSuccess || pr < 1) pr = 4;
     h->grid_blocks[0] = pr * sms;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pr, k_restrict8<T, false>, 128, 0) != cudaSuccess || pr < 1) pr = 4;
+    h->grid_blocks[1] = pr * sms;
   }
 #undef HTRY
   *out = h;
@@ -2953,6 +3004,25 @@ void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool
   }
 }
 
+// launch grid of the restriction from level l: columns and rows of blocks, one wave of its form
+void restrict_grid(const Hierarchy *h, int l, int &gx, int &gy) {
+  const LevelGeom &C = h->lv[l + 1].g;
+  const int lg = row_lg(C.nx), rpb = 128 >> lg;
+  gx = (C.nx + (1 << lg) - 1) >> lg;
+  gy = std::max(1, std::min((C.ny * C.nz + rpb - 1) / rpb, std::min(RESTRICT_BLOCKS, h->grid_blocks[l > 0]) / gx));
+}
+
+// coarse columns (2^lg along x per block, 128 / 2^lg rows) and chunks of kc planes: up to
+// PROLONG_KC, shorter on small levels so that a launch over so many problems still has about
+// PROLONG_BPS blocks per SM
+int prolong_grid(const ibm_ctx *ctx, const LevelGeom &C, int problems, int &gx, int &gy) {
+  const int lg = row_lg(C.nx), rpb = 128 >> lg;
+  gx = (C.nx + (1 << lg) - 1) >> lg;
+  gy = (C.ny + rpb - 1) / rpb;
+  const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
+  return (int)std::max(1LL, std::min<long long>(PROLONG_KC, (long long)gx * gy * C.nz * problems / (PROLONG_BPS * sms)));
+}
+
 // V-cycle for level l: e_l (in/out) approximately solves A_l e_l = r_l - shift_l.  On the
 // finest level e is the hierarchy's own pointer: the fused sweep swaps it between two buffers.
 template <typename T>
@@ -2992,14 +3062,21 @@ void vcycle(Solver &S, int l, T *&e, const T *r, const double *shift, const T *g
   smooth_level<T>(S, l, e, r, shift, fine, ghost_rhs, S.nu1);
   Level &F = h->lv[l], &C = h->lv[l + 1];
   T *ec = (T *)C.e, *rc = (T *)C.r;
-  const int gx = (int)nblk(C.g.nx, 128),
-            gy = std::max(1, std::min(C.g.ny * C.g.nz, std::min(RESTRICT_BLOCKS, h->grid_blocks[0]) / gx));
+  const int lg = row_lg(C.g.nx);
+  int gx, gy;
+  restrict_grid(h, l, gx, gy);
   // storage of the two levels (BF16 on coarse levels of a BF16-storage hierarchy)
   auto restrict_into = [&](auto sf, auto sc) {
     using SF = decltype(sf);
     using SC = decltype(sc);
-    k_restrict8<T, SF, SC><<<dim3(gx, gy), 128, 0, S.st>>>(view<T>(F), (const SF *)e, (const SF *)r, shift, view<T>(C),
-                                                           (SC *)rc, (SC *)ec, S.part);
+    if constexpr (sizeof(SF) >= 4)   // the finest level is never stored in BF16
+      if (l == 0) {
+        k_restrict8<T, true, SF, SC><<<dim3(gx, gy), 128, 0, S.st>>>(view<T>(F), (const SF *)e, (const SF *)r, shift,
+                                                                     view<T>(C), (SC *)rc, (SC *)ec, S.part, lg);
+        return;
+      }
+    k_restrict8<T, false, SF, SC><<<dim3(gx, gy), 128, 0, S.st>>>(view<T>(F), (const SF *)e, (const SF *)r, shift,
+                                                                  view<T>(C), (SC *)rc, (SC *)ec, S.part, lg);
   };
   if constexpr (sizeof(T) == 4) {
     if (F.bf16 && C.bf16) restrict_into(bf16{}, bf16{});
@@ -3019,19 +3096,16 @@ void vcycle(Solver &S, int l, T *&e, const T *r, const double *shift, const T *g
   double *cshift = S.scal + S_LEVEL_SHIFT + (l + 1);
   k_finalize_shift<<<1, 256, 0, S.st>>>(S.part, nparts, h->d_fvol + (l + 1), cshift);
   vcycle<T>(S, l + 1, ec, rc, cshift, nullptr);
-  // coarse columns (x: 128 per block, y: one per block) and chunks of kc planes: up to
-  // PROLONG_KC, shorter on small levels so that a launch still has about two waves of blocks
-  const long long pcols = nblk(C.g.nx, 128) * (long long)C.g.ny;
-  const long long sms = S.ctx->sm_count > 0 ? S.ctx->sm_count : 152;
-  const int kc = (int)std::max(1LL, std::min<long long>(PROLONG_KC, pcols * C.g.nz / (16LL * sms)));
-  dim3 gp((unsigned)nblk(C.g.nx, 128), (unsigned)C.g.ny, (unsigned)((C.g.nz + kc - 1) / kc));
+  int pgx, pgy;
+  const int kc = prolong_grid(S.ctx, C.g, 1, pgx, pgy);
+  const dim3 gp(pgx, pgy, (C.g.nz + kc - 1) / kc);
   const int nxf = F.g.nx, nyf = F.g.ny;
   auto prolong_from = [&](auto sc, auto sf) {
     using SC = decltype(sc);
     using SF = decltype(sf);
     k_prolong8<T, SC, SF><<<gp, 128, 0, S.st>>>(view<T>(C), (const SC *)ec, C.inner, view<T>(F), (SF *)e, F.poff,
                                                 F.poff + nxf, F.poff + nxf + nyf, F.pt, F.pt + nxf, F.pt + nxf + nyf,
-                                                kc);
+                                                kc, lg);
   };
   if constexpr (sizeof(T) == 4) {
     if (C.bf16 && F.bf16) prolong_from(bf16{}, bf16{});
@@ -3600,7 +3674,7 @@ struct PRestrict {
   const double *shift;
   float *rc, *ec;
   double *part;
-  int gx, gy;
+  int lg, gx, gy;
 };
 struct PShift {
   const double *part, *fvol;
@@ -3614,7 +3688,7 @@ struct PProlong {
   float *ef;
   const int8_t *offx, *offy, *offz;
   const float *tx, *ty, *tz;
-  int kc, gx, gy;
+  int kc, lg, gx, gy;
 };
 struct PCoarsest {
   const float *minv, *r;
@@ -3650,19 +3724,20 @@ __global__ void kb_ghost_store(const __grid_constant__ BL<PGhost> L) {
   BL_BLOCK(L)
   ghost_store_body<float>(p.dst, p.ng, p.ngp, p.gtmp, p.e, vgrid(lb, 1 << 30, 1));
 }
-__global__ void __launch_bounds__(128, 5) kb_restrict8(const __grid_constant__ BL<PRestrict> L) {
+template <bool FINEST>
+__global__ void __launch_bounds__(128, 4) kb_restrict8(const __grid_constant__ BL<PRestrict> L) {
   BL_BLOCK(L)
-  restrict8_body<float, float, float>(p.f, p.e, p.r, p.shift, p.c, p.rc, p.ec, p.part, vgrid(lb, p.gx, p.gy));
+  restrict8_body<float, FINEST, float, float>(p.f, p.e, p.r, p.shift, p.c, p.rc, p.ec, p.part, p.lg, vgrid(lb, p.gx, p.gy));
 }
 __global__ void kb_finalize_shift(const __grid_constant__ BL<PShift> L) {
   BL_BLOCK(L)
   (void)lb;
   finalize_shift_body(p.part, p.nb, p.fvol, p.shift);
 }
-__global__ void __launch_bounds__(128, 8) kb_prolong8(const __grid_constant__ BL<PProlong> L) {
+__global__ void __launch_bounds__(128, 6) kb_prolong8(const __grid_constant__ BL<PProlong> L) {
   BL_BLOCK(L)
   prolong8_body<float, float, float>(p.c, p.ec, p.inner, p.f, p.ef, p.offx, p.offy, p.offz, p.tx, p.ty, p.tz, p.kc,
-                                     vgrid(lb, p.gx, p.gy));
+                                     p.lg, vgrid(lb, p.gx, p.gy));
 }
 __global__ void kb_coarsest(const __grid_constant__ BL<PCoarsest> L) {
   BL_BLOCK(L)
@@ -3916,11 +3991,7 @@ void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
 }
 
 // the restriction's grid of level l -> l + 1, as the single-problem V-cycle takes it
-void lk_restrict_grid(Hierarchy *h, int l, int &gx, int &gy) {
-  const Level &C = h->lv[l + 1];
-  gx = (int)nblk(C.g.nx, 128);
-  gy = std::max(1, std::min(C.g.ny * C.g.nz, std::min(RESTRICT_BLOCKS, h->grid_blocks[0]) / gx));
-}
+void lk_restrict_grid(Hierarchy *h, int l, int &gx, int &gy) { restrict_grid(h, l, gx, gy); }
 
 void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
   std::vector<int> tail, coarsest, mid;
@@ -3967,11 +4038,13 @@ void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
                          p.e = K.E[l][i]; p.r = lk_r(K, i, l); p.shift = lk_shift(K, i, l);
                          p.rc = (float *)h->lv[l + 1].r; p.ec = (float *)h->lv[l + 1].e;
                          p.part = (*K.R)[i].S.part;
+                         p.lg = row_lg(p.c.nx);
                          lk_restrict_grid(h, l, p.gx, p.gy);
                          return p;
                        },
                        [&](const BL<PRestrict> &L, int b) {
-                         kb_restrict8<<<b, 128, 0, K.st>>>(L);
+                         if (l == 0) kb_restrict8<true><<<b, 128, 0, K.st>>>(L);
+                         else kb_restrict8<false><<<b, 128, 0, K.st>>>(L);
                          K.ctx->launches += 1;
                        });
   bl_launch<PShift>(mid, [](int) { return 1; },
@@ -3990,16 +4063,12 @@ void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
                     });
   for (int i : mid) K.E[l + 1][i] = (float *)lk_h(K, i)->lv[l + 1].e;
   lk_vcycle(K, l + 1, mid);
-  const long long sms = K.ctx->sm_count > 0 ? K.ctx->sm_count : 152;
-  auto kc_of = [&](const LevelGeom &C) {
-    const long long pcols = nblk(C.nx, 128) * (long long)C.ny;
-    return (int)std::max(1LL, std::min<long long>(PROLONG_KC, pcols * C.nz / (16LL * sms)));
-  };
   bl_launch<PProlong>(mid,
                       [&](int i) {
                         const LevelGeom &C = lk_h(K, i)->lv[l + 1].g;
-                        const int kc = kc_of(C);
-                        return (int)nblk(C.nx, 128) * C.ny * ((C.nz + kc - 1) / kc);
+                        int gx, gy;
+                        const int kc = prolong_grid(K.ctx, C, (int)mid.size(), gx, gy);
+                        return gx * gy * ((C.nz + kc - 1) / kc);
                       },
                       [&](int i) {
                         Hierarchy *h = lk_h(K, i);
@@ -4010,8 +4079,8 @@ void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
                         p.ec = K.E[l + 1][i]; p.inner = C.inner; p.ef = K.E[l][i];
                         p.offx = F.poff; p.offy = F.poff + nxf; p.offz = F.poff + nxf + nyf;
                         p.tx = F.pt; p.ty = F.pt + nxf; p.tz = F.pt + nxf + nyf;
-                        p.kc = kc_of(C.g);
-                        p.gx = (int)nblk(C.g.nx, 128); p.gy = C.g.ny;
+                        p.lg = row_lg(C.g.nx);
+                        p.kc = prolong_grid(K.ctx, C.g, (int)mid.size(), p.gx, p.gy);
                         return p;
                       },
                       [&](const BL<PProlong> &L, int b) {
