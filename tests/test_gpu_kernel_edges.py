@@ -119,3 +119,27 @@ def test_solves_at_odd_sizes(ctx, shape):
         err = np.linalg.norm((p.cpu().numpy() - p_o)[fl]) / np.linalg.norm(p_o[fl])
         assert err < 1e-8, (prec, err)
     T.close()
+
+
+@pytest.mark.parametrize("shape", [(2, 2, 2), (31, 3, 16), (32, 5, 17), (33, 2, 15), (62, 4, 33), (63, 7, 32), (100, 9, 40)])
+def test_noalloc_residual_at_march_edges(ctx, shape):
+    """The allocation-free residual (marches of 16 planes, 31 or 32 cells along x) against the oracle's,
+    with a large mean in p and in the right-hand side; p undefined (NaN) inside the body."""
+    from oracle import system as OY
+    pkg, c = ctx
+    f = [synth.faces_tanh(m, 1.7) for m in shape]
+    big = min(shape) > 8
+    meshes = [synth.octa_sphere(2, (0.5, 0.5, 0.5), 0.3)] if big else []
+    g, T, ex, ib, G = classify_both(pkg, c, *f, meshes)
+    e = T.export()
+    b = synth.counter_normal(3, 0, np.arange(ib.size)).reshape(ib.shape) + 5.0
+    p = synth.smooth_field(*f, 4) + 1e-3 * synth.counter_normal(3, 1, np.arange(ib.size)).reshape(ib.shape)
+    p_nan = np.where(ib == 1, np.nan, p)
+    rel, sr, sb = pkg.ibm_residual_norm_noalloc(*f, e["iblank"], e["cell"], e["ref"], e["w"], e["scale"],
+                                                torch.from_numpy(b).cuda(), torch.from_numpy(p_nan).cuda())
+    rf, rg = OY.residual(g, ib, G, b, p, 0.0)
+    want = OY.projected_norm(g, ib, G, rf, rg)
+    base = OY.projected_norm(g, ib, G, np.where(ib == 0, b, 0.0), np.zeros(len(G)))
+    # a residual cell carries about 10 roundings of sum |c| |p| and of the mean of b
+    assert abs(sr - want) <= 1e-12 * want and abs(sb - base) <= 1e-12 * base and abs(rel - want / base) <= 2e-12 * rel
+    T.close()
