@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "dfloat.cuh"
+#include "ghost.cuh"
 #include "ibm_internal.cuh"
 
 namespace ibm {
@@ -125,15 +126,11 @@ __global__ void k_hz_ghost(const long long *src, const long long *dst, const dou
                            long long ng, T *un, const T *u, const T *f) {
   const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (g >= ng) return;
-  T s = 0;
-  for (int c = 0; c < 8; ++c) {
-    const long long q = src[8 * g + c];
-    if (q < 0) continue;
-    const T v = (q & GHOST_CORNER) ? u[q & ~GHOST_CORNER] : un[q];
-    s += (T)gw[8 * g + c] * v;
-  }
-  const T w = (T)ws[g];
-  un[dst[g]] = (f[dst[g]] - ((T)1 - w) * s) / ((T)1 + w);
+  const GhostRow<double> row(src, gw, g);
+  const long long d = dst[g];
+  const T b = f[d], w = (T)ws[g];
+  const T s = row.sum<T>([&](long long q) { return (q & GHOST_CORNER) ? u[q & ~GHOST_CORNER] : un[q]; });
+  un[d] = (b - ((T)1 - w) * s) / ((T)1 + w);
 }
 
 // FP64 residual r = b - H u of the regular fluid rows (coefficients pre-scaled by alpha);
@@ -211,11 +208,7 @@ __global__ void __launch_bounds__(HZ_THREADS) k_hz_resid_rest(
       if (with_b) ab += fi * fi;
     } else {
       const long long g = t - ncut;
-      double s = 0.0;
-      for (int c = 0; c < 8; ++c) {
-        const long long q = src[8 * g + c];
-        if (q >= 0) s += gw[8 * g + c] * x.U(q & ~GHOST_CORNER);
-      }
+      const double s = GhostRow<double>(src, gw, g).sum<double>([&](long long q) { return x.U(q & ~GHOST_CORNER); });
       const long long id = dst[g];
       const double fi = x.F(id);
       const double r = fi - ((1.0 + ws[g]) * x.U(id) + (1.0 - ws[g]) * s);

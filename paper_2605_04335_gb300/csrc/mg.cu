@@ -27,6 +27,7 @@
 
 #include "ibm_internal.cuh"
 #include "dfloat.cuh"
+#include "ghost.cuh"
 #include "scan.cuh"
 #include "zmarch.cuh"
 
@@ -523,12 +524,10 @@ __device__ __forceinline__ void ghost_eval_body(const long long *src, const long
                                                 const long long *ngp, const T *e, const T *rhs, T *gtmp,
                                                 const double *gd, const G &gr) {
   long long g = gr.bx() * (long long)blockDim.x + threadIdx.x;
-  if (g >= (ngp ? *ngp : ng)) return;
-  T s = (T)0;
-  for (int c = 0; c < 8; ++c) {
-    long long q = src[8 * g + c];
-    if (q >= 0) s += (T)w[8 * g + c] * e[q & ~GHOST_CORNER];
-  }
+  if (g >= ng) return;   // the arrays' capacity: a row past the count is loaded, not used
+  const GhostRow<W> row(src, w, g);
+  if (ngp && g >= *ngp) return;
+  T s = row.template sum<T>([&](long long q) { return e[q & ~GHOST_CORNER]; });
   if (rhs) s += rhs[dst[g]];
   if (gd) s += (T)gd[g];     // the row's Neumann datum
   gtmp[g] = s;
@@ -548,17 +547,15 @@ __device__ __forceinline__ void ghost_pp_body(const long long *src, const long l
                                               const long long *ngp, T *enew, const T *eold, const T *rhs,
                                               const double *gd, const G &gr) {
   long long g = gr.bx() * (long long)blockDim.x + threadIdx.x;
-  if (g >= (ngp ? *ngp : ng)) return;
-  T s = (T)0;
-  for (int c = 0; c < 8; ++c) {
-    long long q = src[8 * g + c];
-    if (q < 0) continue;
-    const T v = (q & GHOST_CORNER) ? eold[q & ~GHOST_CORNER] : enew[q];
-    s += (T)w[8 * g + c] * v;
-  }
-  if (rhs) s += rhs[dst[g]];
+  if (g >= ng) return;   // the arrays' capacity: a row past the count is loaded, not used
+  const GhostRow<W> row(src, w, g);
+  const long long d = dst[g];
+  if (ngp && g >= *ngp) return;
+  const T b = rhs ? rhs[d] : (T)0;
+  T s = row.template sum<T>([&](long long q) { return (q & GHOST_CORNER) ? eold[q & ~GHOST_CORNER] : enew[q]; });
+  if (rhs) s += b;
   if (gd) s += (T)gd[g];     // the row's Neumann datum
-  enew[dst[g]] = s;
+  enew[d] = s;
 }
 
 template <typename T, typename W>
@@ -1272,11 +1269,7 @@ __device__ __forceinline__ void ghost_resid64_body(const long long *src, const l
   double a = 0.0;
   const long long ng = *ngp;
   for (long long g = gr.bx() * (long long)blockDim.x + threadIdx.x; g < ng; g += (long long)gr.gx() * blockDim.x) {
-    double s = 0.0;
-    for (int c = 0; c < 8; ++c) {
-      long long q = src[8 * g + c];
-      if (q >= 0) s += w[8 * g + c] * p[q & ~GHOST_CORNER];
-    }
+    const double s = GhostRow<double>(src, w, g).sum<double>([&](long long q) { return p[q & ~GHOST_CORNER]; });
     double rg = s - p[dst[g]];
     if (gd) rg += gd[g];       // r_G = kappa q - (g - sum w v)
     if (r32) r32[dst[g]] = (R)rg;
@@ -1561,14 +1554,10 @@ __device__ __forceinline__ void ghost_resid_df_body(const long long *src, const 
   double a = 0.0;
   const long long ng = *ngp;
   for (long long g = gr.bx() * (long long)blockDim.x + threadIdx.x; g < ng; g += (long long)gr.gx() * blockDim.x) {
-    double s = 0.0;
-    for (int c = 0; c < 8; ++c) {
-      long long q = src[8 * g + c];
-      if (q >= 0) {
-        q &= ~GHOST_CORNER;
-        s += w[8 * g + c] * dfl::join(ph[q], pl[q]);
-      }
-    }
+    const double s = GhostRow<double>(src, w, g).sum<double>([&](long long q) {
+      q &= ~GHOST_CORNER;
+      return dfl::join(ph[q], pl[q]);
+    });
     const long long d = dst[g];
     double rg = s - dfl::join(ph[d], pl[d]);
     if (gd) rg += gd[g];       // r_G = kappa q - (g - sum w v)
@@ -1596,14 +1585,10 @@ __global__ void k_ghost_eval_df(const long long *src, const double *w, long long
                                 const float *pl, double *gtmp, const double *gd) {
   long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (g >= ng) return;
-  double s = 0.0;
-  for (int c = 0; c < 8; ++c) {
-    long long q = src[8 * g + c];
-    if (q >= 0) {
-      q &= ~GHOST_CORNER;
-      s += w[8 * g + c] * dfl::join(ph[q], pl[q]);
-    }
-  }
+  double s = GhostRow<double>(src, w, g).sum<double>([&](long long q) {
+    q &= ~GHOST_CORNER;
+    return dfl::join(ph[q], pl[q]);
+  });
   if (gd) s += gd[g];        // the row's Neumann datum
   gtmp[g] = s;
 }
@@ -2145,11 +2130,7 @@ __global__ void k_gcr_apply_ghost(const long long *src, const long long *dst, co
   T *q = qb + (long long)gs->j * nslot;
   const long long ng = *ngp;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < ng; g += (long long)gridDim.x * blockDim.x) {
-    T s = 0;
-    for (int c = 0; c < 8; ++c) {
-      const long long x = src[8 * g + c];
-      if (x >= 0) s += (T)w[8 * g + c] * z[x & ~GHOST_CORNER];
-    }
+    const T s = GhostRow<W>(src, w, g).template sum<T>([&](long long x) { return z[x & ~GHOST_CORNER]; });
     q[dst[g]] = z[dst[g]] - s;
   }
 }
