@@ -48,6 +48,67 @@ __device__ __forceinline__ void acc_prod(float ah, float al, float bh, float bl,
   acc_l += t + e;
 }
 
+// Two cells' floats side by side: sm_103a's packed FP32 operations, each component rounded as the
+// scalar operation, at half the instructions.
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float x, float y) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void un2(F2 a, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+  F2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 neg2(F2 a) { return F2{a.v ^ 0x8000000080000000ull}; }
+
+// (acc_h, acc_l) -= (c, c_l) * (b_h, b_l): the bits of acc_prod(-c, -c_l, ...); n, nl: -c and -c_l
+__device__ __forceinline__ void acc_prod_neg2(F2 c, F2 n, F2 nl, F2 bh, F2 bl, F2 &acc_h, F2 &acc_l) {
+  const F2 p = mul2(c, bh);
+  F2 e = fma2(n, bh, p);   // -(c b - p)
+  e = fma2(n, bl, e);
+  e = fma2(nl, bh, e);
+  const F2 s = sub2(acc_h, p), bb = sub2(s, acc_h);
+  const F2 t = sub2(sub2(acc_h, sub2(s, bb)), add2(p, bb));
+  acc_h = s;
+  acc_l = add2(acc_l, add2(t, e));
+}
+// (acc_h, acc_l) += (d, d_l) * (b_h, b_l)
+__device__ __forceinline__ void acc_prod2(F2 d, F2 dl, F2 bh, F2 bl, F2 &acc_h, F2 &acc_l) {
+  const F2 p = mul2(d, bh);
+  F2 e = fma2(d, bh, neg2(p));
+  e = fma2(d, bl, e);
+  e = fma2(dl, bh, e);
+  const F2 s = add2(acc_h, p), bb = sub2(s, acc_h);
+  const F2 t = add2(sub2(acc_h, sub2(s, bb)), sub2(p, bb));
+  acc_h = s;
+  acc_l = add2(acc_l, add2(t, e));
+}
+__device__ __forceinline__ void two_sum2(F2 a, F2 b, F2 &s, F2 &e) {
+  s = add2(a, b);
+  const F2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+
 // exact float -> double widening by bit manipulation (keeps the FP64 pipe free); normal
 // floats, zero and inf map exactly, NaN to a NaN; subnormal floats (below 2^-126, far under any
 // low part that matters here) become signed zero

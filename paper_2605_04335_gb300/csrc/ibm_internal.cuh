@@ -101,6 +101,7 @@ struct Hierarchy {
   int *cidx = nullptr;                      // padded index of each coarsest unknown
   int *dncoarse = nullptr;                  // device copy of ncoarse
   double *c64 = nullptr;                    // FP64 fine coefficients cxm cxp cym cyp czm czp
+  float *xq = nullptr;                      // its x parts in aligned rows (DfView::xq)
   float *cdf = nullptr;                     // fine coefficients, diagonal parts and widths split
                                             // into hi (4n floats) and lo (4n) parts
   // solver-side ghost rows: padded source indices (-1 unused), weights (double and float)

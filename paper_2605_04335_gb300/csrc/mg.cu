@@ -433,7 +433,7 @@ inline int relax_gx(const Geom &g) {   // blocks of strips per chunk of planes
 }
 template <typename T, int KZ, class G>
 __device__ __forceinline__ void relax_body(const LV<T> &v, T *e, const T *r, const double *shift, int colour, float om,
-                                           const G &gr) {
+                                           bool sep, const G &gr) {
   static_assert(KZ == 1 || KZ == 2, "the planes of one thread");
   const int groups = (v.nx + 3) >> 2;
   const int strip = gr.bx() * RELAX_THREADS + (int)threadIdx.x;
@@ -485,6 +485,7 @@ __device__ __forceinline__ void relax_body(const LV<T> &v, T *e, const T *r, con
       const int i = min(4 * g + ua + 2 * h, v.nx - 1);
       T cf[6] = {KZ == 1 ? pick(xm, h) : v.cxm[i], KZ == 1 ? pick(xp, h) : v.cxp[i], cym, cyp, czm, czp};
       T D = (KZ == 1 ? pick(xd, h) : v.rdx[i]) + syz;
+      if (!sep) D = ((cf[0] + cf[1]) + (cf[2] + cf[3])) + (cf[4] + cf[5]);
       if (m == zm::IRREGULAR) {   // coefficients scaled by the open fractions, the diagonal their sum
         const long long id = id0 + q * v.sz + ua + 2 * h;
         cf[0] = mul_rn(cf[0], v.fx[id - 1]); cf[1] = mul_rn(cf[1], v.fx[id]);
@@ -492,24 +493,34 @@ __device__ __forceinline__ void relax_body(const LV<T> &v, T *e, const T *r, con
         cf[4] = mul_rn(cf[4], v.fz[id - v.sz]); cf[5] = mul_rn(cf[5], v.fz[id]);
         D = ((cf[0] + cf[1]) + (cf[2] + cf[3])) + (cf[4] + cf[5]);
       }
-      T res = fma_t<T>(-D, c, -(pick(R[q], h) - sh));
-      res = fma_t<T>(cf[0], w, res);
+      const T rhs = pick(R[q], h) - sh;
+      T res = sep ? fma_t<T>(cf[0], w, fma_t<T>(-D, c, -rhs)) : mul_rn(cf[0], w);
       res = fma_t<T>(cf[1], ea, res);
       res = fma_t<T>(cf[2], pick(N[q], h), res);
       res = fma_t<T>(cf[3], pick(S[q], h), res);
       res = fma_t<T>(cf[4], pick(C[q], h), res);
       res = fma_t<T>(cf[5], pick(C[q + 2], h), res);
+      T out;
+      if (sep) out = relax_update(c, res, D, om);
+      else out = c + (T)__fdividef(om * (float)(fma_t<T>(-D, c, res) - rhs), (float)D);
       // a cell with no open face keeps its value
-      if (live && D > (T)0) e[id0 + q * v.sz + ua + 2 * h] = relax_update(c, res, D, om);
+      if (live && D > (T)0) e[id0 + q * v.sz + ua + 2 * h] = out;
     }
   }
 }
 
 template <typename T, int KZ>
 __global__ void __launch_bounds__(RELAX_THREADS) k_relax(LV<T> v, T *e, const T *r, const double *shift, int colour,
-                                                         float om) {
-  relax_body<T, KZ>(v, e, r, shift, colour, om, HwGrid{});
+                                                         float om, bool sep) {
+  relax_body<T, KZ>(v, e, r, shift, colour, om, sep, HwGrid{});
 }
+
+// the order of a level's sums: the fused sweep's (the diagonal's part first, the separable diagonal
+// of regular cells) in FP64 and from 2^18 cells, below it the neighbours' parts first and the
+// diagonal as their sum.  Which of the two is not a question of speed: near the tolerance a
+// Krylov-accelerated solve turns a changed rounding of the coarse levels into one step more or fewer
+template <typename T>
+inline bool relax_sep(const LevelGeom &g) { return sizeof(T) == 8 || (long long)g.nx * g.ny * g.nz >= (1LL << 18); }
 
 // planes per thread of a launch over `cells` cells: two in FP32 where the launch fills the chip
 // several times over (they halve the loads of z-neighbours: 48 against 84 us per colour at 256^3),
@@ -687,6 +698,7 @@ __device__ __forceinline__ void restrict8_body(const LV<T> &f, const SF *e, cons
             const uint8_t m = a ? M[d][b].y : M[d][b].x;
             T c[6] = {cxm[a], cxp[a], cym[b], cyp[b], czm[d], czp[d]};
             T D = (sdx[a] + sdy[b]) + sdz[d];
+            if (!FINEST && sizeof(T) == 4) D = ((c[0] + c[1]) + (c[2] + c[3])) + (c[4] + c[5]);
             if (!FINEST && m == zm::IRREGULAR) {   // coarse levels near a body: face fractions
               const long long id = fb + d * f.sz + b * f.sy + a;
               c[0] = mul_rn(c[0], f.fx[id - 1]); c[1] = mul_rn(c[1], f.fx[id]);
@@ -1172,6 +1184,13 @@ __device__ __forceinline__ void block_partials3(double A0, double A1, double A2,
     for (int q = 0; q < 3; ++q) partials[3 * b + q] = sm[q][0];
 }
 
+// launched as gx blocks, fewer than REDUCE_BLOCKS: the other blocks' slots read zero
+__device__ __forceinline__ void clear_partials3(double *partials, int bx, int gx) {
+  if (threadIdx.x == 0)
+    for (int b = bx + gx; b < REDUCE_BLOCKS; b += gx)
+      for (int q = 0; q < 3; ++q) partials[3 * b + q] = 0.0;
+}
+
 // FP64 fine residual r = b - lambda - A p on fluid rows, stored as R (FP32 for the mixed
 // modes' inner cycles, FP64 for the accelerated FP64 mode; 0 on other cells); block partials
 // (sum V r, sum r, sum r^2, of the FP32 r) at partials[3 b + {0,1,2}].  FP64 arithmetic is
@@ -1433,6 +1452,8 @@ struct DfView {
   long long sy, sz;
   const uint8_t *mask;
   const float *h, *l;
+  const float *xq;     // x parts in rows of nx4 = 4 ceil(nx / 4) floats: cxm cxp -cxm -cxp sdx dx (hi), -cxm -cxp
+                       // sdx (lo)
 };
 
 // split n doubles into hi/lo floats
@@ -1441,83 +1462,124 @@ __global__ void k_split_df(const double *src, int n, float *h, float *l) {
   if (q < n) dfl::split(src[q], h[q], l[q]);
 }
 
+// the x parts of the split fine data (layout of DfView::xq; entries past nx repeat the last)
+constexpr int XQ_ROWS = 9;
+__global__ void k_xq(const float *h, const float *l, int nx, int n, int nx4, float *xq) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nx4) return;
+  const int c = min(i, nx - 1);
+  const float q[XQ_ROWS] = {h[c], h[nx + c], -h[c], -h[nx + c], h[2 * n + c], h[3 * n + c], -l[c], -l[nx + c], l[2 * n + c]};
+  for (int r = 0; r < XQ_ROWS; ++r) xq[r * nx4 + i] = q[r];
+}
+
 // r = b - lambda - A p on fluid rows with pairs of floats (see dfloat.cuh); FP32 copy of r
 // (0 on other cells); block partials (sum V r, sum r, sum r^2) at partials[3 b + {0,1,2}] as
 // k_residual64, for b < REDUCE_BLOCKS whatever the grid.  ph == nullptr: residual of p = 0.
+// Bound by the latency of its loads and about 100 FP32 operations per cell: four cells per thread, the x
+// coefficients of a strip 16-byte loads of aligned rows, and the products and sums packed two cells
+// to an instruction (the same bits as one by one): 150 -> 122 us
+// at 256^3 (0.42 of the copy bandwidth for 21 bytes a cell).  Blocks without a row are not launched: 96
+// problems of edges 16 to 32 took 201 us a launch with 456 blocks each, 20 now.
+// The blocks, their rows and the order of the partial sums are fixed: a z-march with
+// three planes of p in registers takes 98 us at 256^3, but its sums round differently, and near the tolerance
+// a Krylov-accelerated solve turns a changed last bit of the mean into one step more or fewer.
 template <class G>
 __device__ __forceinline__ void residual_df_body(const DfView &v, const float *ph, const float *pl, const float *bh,
                                                  const float *bl, const double *lambda, float *r32, double *partials,
                                                  const G &gr) {
+  using namespace dfl;
   float lh, ll;
-  dfl::split(*lambda, lh, ll);
+  split(*lambda, lh, ll);
   const int nx = v.nx, ny = v.ny, nz = v.nz, n = nx + ny + nz;
   const float *H = v.h, *L = v.l;
   float a0 = 0.f, a1 = 0.f, a2 = 0.f;
   double A0 = 0.0, A1 = 0.0, A2 = 0.0;
   int nrow = 0;
   const RowGroups rg(nx);
-  const int rows = ny * nz;
+  const int rows = ny * nz, nx4 = 4 * rg.G;
+  auto two = [](float x) { return f2(x, x); };
+  auto ld = [](const float *q, F2 (&r)[2]) {   // a strip as two pairs
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(q);
+    r[0].v = a.x;
+    r[1].v = a.y;
+  };
   if (rg.active())
     for (int row = rg.first_row(gr); row < rows; row += rg.row_step(gr)) {
       const int j = row % ny, k = row / ny;
-      const float cymh = H[2 * nx + j], cyml = L[2 * nx + j], cyph = H[2 * nx + ny + j], cypl = L[2 * nx + ny + j];
-      const float czmh = H[2 * nx + 2 * ny + k], czml = L[2 * nx + 2 * ny + k];
-      const float czph = H[2 * nx + 2 * ny + nz + k], czpl = L[2 * nx + 2 * ny + nz + k];
       float syh, syl;   // sdy_j + sdz_k
-      dfl::two_sum(H[2 * n + nx + j], H[2 * n + nx + ny + k], syh, syl);
+      two_sum(H[2 * n + nx + j], H[2 * n + nx + ny + k], syh, syl);
       syl += L[2 * n + nx + j] + L[2 * n + nx + ny + k];
       const float dydz = H[3 * n + nx + j] * H[3 * n + nx + ny + k];
       const long long base = (long long)(k + 1) * v.sz + (long long)(j + 1) * v.sy + OX;
       for (int g = rg.g0; g < rg.G; g += rg.gstep) {
         const long long id = base + 4 * g;
+        const float *xq = v.xq + 4 * g;
         bool fl[4];
         ld_mask4(v.mask + id, fl);
-        float BH[4], BL[4];
-        Vec4<float>::ld(bh + id, BH);
-        Vec4<float>::ld(bl + id, BL);
-        // per cell the terms accumulate in the order b - lambda, diagonal, x-, x+, y-, y+, z-,
-        // z+; the y and z neighbour rows are loaded one pair at a time (fewer live registers)
-        float sh[4], sl[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          dfl::two_sum(BH[u], -lh, sh[u], sl[u]);
-          sl[u] += BL[u] - ll;
-        }
+        F2 BH[2], BL[2], sh[2], sl[2];
+        ld(bh + id, BH);
+        ld(bl + id, BL);
+        // per cell the terms accumulate in the order b - lambda, diagonal, x-, x+, y-, y+, z-, z+
         if (ph) {
-          float PH[4], PL[4];
-          Vec4<float>::ld(ph + id, PH);
-          Vec4<float>::ld(pl + id, PL);
-          const float xlh = ph[id - 1], xll = pl[id - 1], xrh = ph[id + 4], xrl = pl[id + 4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int i = min(4 * g + u, nx - 1);   // coefficients of cells past nx: any valid index
-            float dh, dl;   // diagonal sdx_i + sdy_j + sdz_k
-            dfl::two_sum(H[2 * n + i], syh, dh, dl);
-            dl += L[2 * n + i] + syl;
-            dfl::acc_prod(dh, dl, PH[u], PL[u], sh[u], sl[u]);
-            const float lfh = u == 0 ? xlh : PH[u - 1], lfl = u == 0 ? xll : PL[u - 1];
-            const float rgh = u == 3 ? xrh : PH[u + 1], rgl = u == 3 ? xrl : PL[u + 1];
-            dfl::acc_prod(-H[i], -L[i], lfh, lfl, sh[u], sl[u]);
-            dfl::acc_prod(-H[nx + i], -L[nx + i], rgh, rgl, sh[u], sl[u]);
-          }
+          F2 PH[2], PL[2], NH[4][2], NL[4][2], c[2], cn[2], cl[2];   // rows j - 1, j + 1, planes k - 1, k + 1
+          ld(ph + id, PH);
+          ld(pl + id, PL);
 #pragma unroll
           for (int nb = 0; nb < 4; ++nb) {
             const long long off = nb == 0 ? -v.sy : (nb == 1 ? v.sy : (nb == 2 ? -v.sz : v.sz));
-            const float ch = nb == 0 ? cymh : (nb == 1 ? cyph : (nb == 2 ? czmh : czph));
-            const float cl = nb == 0 ? cyml : (nb == 1 ? cypl : (nb == 2 ? czml : czpl));
-            float NH[4], NL[4];
-            Vec4<float>::ld(ph + id + off, NH);
-            Vec4<float>::ld(pl + id + off, NL);
+            ld(ph + id + off, NH[nb]);
+            ld(pl + id + off, NL[nb]);
+          }
+          const float xlh = ph[id - 1], xll = pl[id - 1], xrh = ph[id + 4], xrl = pl[id + 4];
+          ld(xq + 4 * nx4, c);
+          ld(xq + 8 * nx4, cl);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) dfl::acc_prod(-ch, -cl, NH[u], NL[u], sh[u], sl[u]);
+          for (int u = 0; u < 2; ++u) {
+            two_sum2(BH[u], two(-lh), sh[u], sl[u]);
+            sl[u] = add2(sl[u], sub2(BL[u], two(ll)));
+            F2 dh, dl;   // diagonal sdx_i + sdy_j + sdz_k
+            two_sum2(c[u], two(syh), dh, dl);
+            dl = add2(dl, add2(cl[u], two(syl)));
+            acc_prod2(dh, dl, PH[u], PL[u], sh[u], sl[u]);
+          }
+          float p0, p1, p2, p3, q0, q1, q2, q3;
+          un2(PH[0], p0, p1);
+          un2(PH[1], p2, p3);
+          un2(PL[0], q0, q1);
+          un2(PL[1], q2, q3);
+          ld(xq, c);
+          ld(xq + 2 * nx4, cn);
+          ld(xq + 6 * nx4, cl);
+          acc_prod_neg2(c[0], cn[0], cl[0], f2(xlh, p0), f2(xll, q0), sh[0], sl[0]);
+          acc_prod_neg2(c[1], cn[1], cl[1], f2(p1, p2), f2(q1, q2), sh[1], sl[1]);
+          ld(xq + nx4, c);
+          ld(xq + 3 * nx4, cn);
+          ld(xq + 7 * nx4, cl);
+          acc_prod_neg2(c[0], cn[0], cl[0], f2(p1, p2), f2(q1, q2), sh[0], sl[0]);
+          acc_prod_neg2(c[1], cn[1], cl[1], f2(p3, xrh), f2(q3, xrl), sh[1], sl[1]);
+#pragma unroll
+          for (int nb = 0; nb < 4; ++nb) {
+            const int o = nb < 2 ? 2 * nx + (nb == 0 ? 0 : ny) + j : 2 * nx + 2 * ny + (nb == 2 ? 0 : nz) + k;
+            const float ch = H[o], cL = L[o];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+              acc_prod_neg2(two(ch), two(-ch), two(-cL), NH[nb][u], NL[nb][u], sh[u], sl[u]);
+          }
+        } else {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            two_sum2(BH[u], two(-lh), sh[u], sl[u]);
+            sl[u] = add2(sl[u], sub2(BL[u], two(ll)));
           }
         }
-        float rf[4];
+        float rf[4], dx[4];
+        Vec4<float>::ld(xq + 5 * nx4, dx);
+        un2(add2(sh[0], sl[0]), rf[0], rf[1]);
+        un2(add2(sh[1], sl[1]), rf[2], rf[3]);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int i = min(4 * g + u, nx - 1);
-          rf[u] = fl[u] ? sh[u] + sl[u] : 0.f;
-          a0 = fmaf(H[3 * n + i] * dydz, rf[u], a0);
+          rf[u] = fl[u] ? rf[u] : 0.f;
+          a0 = fmaf(dx[u] * dydz, rf[u], a0);
           a1 += rf[u];
           a2 = fmaf(rf[u], rf[u], a2);
         }
@@ -1532,16 +1594,21 @@ __device__ __forceinline__ void residual_df_body(const DfView &v, const float *p
     }
   A0 += a0; A1 += a1; A2 += a2;
   block_partials3(A0, A1, A2, partials, gr.bx());
-  // launched as one wave of fewer than REDUCE_BLOCKS blocks: the other slots read zero
-  if (threadIdx.x == 0)
-    for (int b = gr.bx() + gr.gx(); b < REDUCE_BLOCKS; b += gr.gx())
-      for (int q = 0; q < 3; ++q) partials[3 * b + q] = 0.0;
+  clear_partials3(partials, gr.bx(), gr.gx());
 }
 
-__global__ void __launch_bounds__(REDUCE_THREADS) k_residual_df(DfView v, const float *ph, const float *pl,
-                                                               const float *bh, const float *bl,
-                                                               const double *lambda, float *r32, double *partials) {
+constexpr int RDF_PER_SM = 3;   // resident blocks per SM (80 registers)
+__global__ void __launch_bounds__(REDUCE_THREADS, RDF_PER_SM) k_residual_df(DfView v, const float *ph, const float *pl,
+                                                                            const float *bh, const float *bl,
+                                                                            const double *lambda, float *r32,
+                                                                            double *partials) {
   residual_df_body(v, ph, pl, bh, bl, lambda, r32, partials, HwGrid{});
+}
+// its blocks: one wave, but none without a row (an idle block's partials read zero either way)
+inline int rdf_blocks(const ibm_ctx *ctx, const LevelGeom &g) {
+  const long long G = (g.nx + 3) / 4, rpi = G >= REDUCE_THREADS ? 1 : REDUCE_THREADS / G;
+  const long long blocks = std::min(REDUCE_BLOCKS, RDF_PER_SM * (ctx->sm_count > 0 ? ctx->sm_count : 152));
+  return (int)std::min<long long>(blocks, ((long long)g.ny * g.nz + rpi - 1) / rpi);
 }
 
 // ghost rows r_G = sum w v - g in FP64 from the split values; block partials of (s_G r_G)^2
@@ -2347,7 +2414,7 @@ void free_hierarchy(Hierarchy *h) {
                  L.zmask, L.ealt, L.zsd};
     ps.insert(ps.end(), q, q + sizeof(q) / sizeof(q[0]));
   }
-  void *q[] = {h->p64, h->b64, h->minv, h->gj, h->cidx, h->dncoarse, h->c64, h->cdf, h->gsrc, h->gdst, h->gw64,
+  void *q[] = {h->p64, h->b64, h->minv, h->gj, h->cidx, h->dncoarse, h->c64, h->cdf, h->xq, h->gsrc, h->gdst, h->gw64,
                h->zcount,
                h->gw32, h->gtmp, h->e_alt, h->tm_base[0], h->tm_base[1], h->d_fvol, h->d_ng,
                h->cut_id, h->cut_nb, h->cut_ijk, h->par_id, h->d_cnt, h->par_flag, h->scan_buf, h->gcr_buf,
@@ -2945,6 +3012,7 @@ void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool
   Level &L = S.h->lv[l];
   LV<T> v = view<T>(L);
   const int kz = relax_kz<T>((long long)L.g.nx * L.g.ny * L.g.nz);
+  const bool sep = relax_sep<T>(L.g);
   const dim3 grid(relax_gx(L.g), (L.g.nz + kz - 1) / kz);
   for (int s = 0; s < sweeps; ++s) {
     const bool timed = fine && S.sweep_events && S.sweep_events->size() >= 2 * (size_t)(s + 1);
@@ -2974,9 +3042,9 @@ void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool
       continue;
     } else {
       for (int colour = 0; colour < 2; ++colour)
-        if (kz == 1) k_relax<T, 1><<<grid, RELAX_THREADS, 0, S.st>>>(v, e, r, shift, colour, (float)S.omega);
+        if (kz == 1) k_relax<T, 1><<<grid, RELAX_THREADS, 0, S.st>>>(v, e, r, shift, colour, (float)S.omega, sep);
         else if constexpr (sizeof(T) == 4)
-          k_relax<T, 2><<<grid, RELAX_THREADS, 0, S.st>>>(v, e, r, shift, colour, (float)S.omega);
+          k_relax<T, 2><<<grid, RELAX_THREADS, 0, S.st>>>(v, e, r, shift, colour, (float)S.omega, sep);
       if (timed) cudaEventRecord((*S.sweep_events)[2 * s + 1], S.st);
       S.ctx->launches += 2;
       if (fine) cut_relax<T>(S, e, e, r, shift);
@@ -3127,6 +3195,7 @@ DfView fine_view_df(Hierarchy *h) {
   const int n = v.nx + v.ny + v.nz;
   v.h = h->cdf;
   v.l = h->cdf + 4 * n;
+  v.xq = h->xq;
   return v;
 }
 
@@ -3145,10 +3214,8 @@ void outer_residual(Solver &S, bool with_p, float *r32, bool update_lambda, cons
   const long long ntot = h->nslot;   // hi/lo split point of the outer arrays
   double *part = S.part;
   float *ph = with_p ? hi_of(h->p64) : nullptr, *pl = lo_of(h->p64, ntot);
-  // 80 registers: three resident blocks per SM, so one wave of 3 x SMs blocks
-  const int rdf_blocks = std::min(REDUCE_BLOCKS, 3 * (S.ctx->sm_count > 0 ? S.ctx->sm_count : 152));
-  k_residual_df<<<rdf_blocks, REDUCE_THREADS, 0, S.st>>>(fine_view_df(h), ph, pl, hi_of(h->b64),
-                                                         lo_of(h->b64, ntot), S.scal + S_LAMBDA, r32, part);
+  k_residual_df<<<rdf_blocks(S.ctx, h->lv[0].g), REDUCE_THREADS, 0, S.st>>>(
+      fine_view_df(h), ph, pl, hi_of(h->b64), lo_of(h->b64, ntot), S.scal + S_LAMBDA, r32, part);
   const long long ng = S.t->nghost;
   const int ngb = FIXED_BLOCKS;
   double *gpart = part + 3 * REDUCE_BLOCKS, *cpart = gpart + ngb;
@@ -3284,6 +3351,9 @@ ibm_status build_hierarchy(ibm_tables *t, int precision, cudaStream_t st, bool c
     h->cdf = cdf;
     k_split_df<<<nblk(3 * n, 128), 128, 0, st>>>(h->c64, 3 * n, cdf, cdf + 4 * n);
     k_split_df<<<nblk(n, 128), 128, 0, st>>>(L0.w1d, n, cdf + 3 * n, cdf + 7 * n);
+    const int nx4 = (nx + 3) / 4 * 4;
+    BTRY(cudaMalloc((void **)&h->xq, sizeof(float) * XQ_ROWS * nx4));
+    k_xq<<<nblk(nx4, 128), 128, 0, st>>>(cdf, cdf + 4 * n, nx, n, nx4, h->xq);
   }
   BTRY(cudaGetLastError());
   BTRY(cudaStreamSynchronize(st));
@@ -3640,6 +3710,7 @@ struct PRelax {
   const float *r;
   const double *shift;
   int gx, gy;
+  bool sep;
 };
 struct PGhost {
   const long long *src, *dst;
@@ -3691,7 +3762,7 @@ static_assert(sizeof(BL<PProlong>) <= 32764 && sizeof(BL<PRestrict>) <= 32764, "
 template <int KZ>
 __global__ void __launch_bounds__(RELAX_THREADS) kb_relax(const __grid_constant__ BL<PRelax> L, int colour, float omega) {
   BL_BLOCK(L)
-  relax_body<float, KZ>(p.v, p.e, p.r, p.shift, colour, omega, vgrid(lb, p.gx, p.gy));
+  relax_body<float, KZ>(p.v, p.e, p.r, p.shift, colour, omega, p.sep, vgrid(lb, p.gx, p.gy));
 }
 __global__ void kb_ghost_pp(const __grid_constant__ BL<PGhost> L) {
   BL_BLOCK(L)
@@ -3785,7 +3856,7 @@ __global__ void __launch_bounds__(REDUCE_THREADS) kb_residual64(const __grid_con
   BL_BLOCK(L)
   residual64_body<float, true>(p.v, p.p, p.b, p.lambda, p.wf, p.r32, p.part, nullptr, vgrid(lb, p.gx, 1));
 }
-__global__ void __launch_bounds__(REDUCE_THREADS) kb_residual_df(const __grid_constant__ BL<PRes> L) {
+__global__ void __launch_bounds__(REDUCE_THREADS, RDF_PER_SM) kb_residual_df(const __grid_constant__ BL<PRes> L) {
   BL_BLOCK(L)
   residual_df_body(p.vd, p.ph, p.pl, p.bh, p.bl, p.lambda, p.r32, p.part, vgrid(lb, p.gx, 1));
 }
@@ -3960,7 +4031,7 @@ void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
                          const Level &L = lk_h(K, i)->lv[l];
                          PRelax p;
                          p.v = view<float>(L); p.e = K.E[l][i]; p.r = lk_r(K, i, l); p.shift = lk_shift(K, i, l);
-                         p.gx = relax_gx(L.g); p.gy = (L.g.nz + kz - 1) / kz;
+                         p.gx = relax_gx(L.g); p.gy = (L.g.nz + kz - 1) / kz; p.sep = relax_sep<float>(L.g);
                          return p;
                        },
                        [&](const BL<PRelax> &L, int b) {
@@ -4086,8 +4157,6 @@ void lk_outer(Lock &K, const std::vector<int> &act) {
   std::vector<Run> &R = *K.R;
   ibm_ctx *ctx = K.ctx;
   const bool dfo = R[act[0]].S.dfo;
-  const int sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
-  const int rdf_blocks = std::min(REDUCE_BLOCKS, 3 * sms);   // as outer_residual's double-FP32 launch
   auto ublocks = [&](int i) {
     return (int)std::min<long long>(nblk(dfo ? R[i].ntot / 4 : R[i].ntot, 256), ctx->wave);
   };
@@ -4112,7 +4181,7 @@ void lk_outer(Lock &K, const std::vector<int> &act) {
                        else kb_update_p<<<b, 256, 0, K.st>>>(L);
                        ctx->launches += 1;
                      });
-  bl_launch<PRes>(act, [&](int) { return dfo ? rdf_blocks : REDUCE_BLOCKS; },
+  bl_launch<PRes>(act, [&](int i) { return dfo ? rdf_blocks(ctx, R[i].h->lv[0].g) : REDUCE_BLOCKS; },
                   [&](int i) {
                     Hierarchy *h = R[i].h;
                     const long long ntot = R[i].ntot;
@@ -4121,7 +4190,7 @@ void lk_outer(Lock &K, const std::vector<int> &act) {
                       p.vd = fine_view_df(h);
                       p.ph = hi_of(h->p64); p.pl = lo_of(h->p64, ntot);
                       p.bh = hi_of(h->b64); p.bl = lo_of(h->b64, ntot);
-                      p.gx = rdf_blocks;
+                      p.gx = rdf_blocks(ctx, h->lv[0].g);
                     } else {
                       p.v = fine_view64(h);
                       p.p = h->p64; p.b = h->b64;
