@@ -1348,14 +1348,27 @@ __device__ __forceinline__ void update_p_body(double *p, const float *e, long lo
 
 __global__ void k_update_p(double *p, const float *e, long long n) { update_p_body(p, e, n, HwGrid{}); }
 
-__global__ void __launch_bounds__(REDUCE_THREADS) k_gauge_sum(LV<double> v, const double *p, double *partials) {
+// blocks of a kernel that takes rows of groups of four cells: one pass per block at most max_blocks
+inline int row_blocks(const LevelGeom &g, int max_blocks) {
+  const long long G = (g.nx + 3) / 4, rpi = G >= REDUCE_THREADS ? 1 : REDUCE_THREADS / G;
+  return (int)std::min<long long>(max_blocks, ((long long)g.ny * g.nz + rpi - 1) / rpi);
+}
+
+// launched as gx blocks: the slots of the others up to REDUCE_BLOCKS read zero
+__device__ __forceinline__ void clear_partials1(double *partials, int bx, int gx) {
+  if (threadIdx.x == 0)
+    for (int b = bx + gx; b < REDUCE_BLOCKS; b += gx) partials[b] = 0.0;
+}
+
+template <class G>
+__device__ __forceinline__ void gauge_sum_body(const LV<double> &v, const double *p, double *partials, const G &gr) {
   __shared__ double sm[REDUCE_THREADS];
   double a = 0.0;
   const int nx = v.nx, ny = v.ny;
   const RowGroups rg(nx);
   const int rows = ny * v.nz;
   if (rg.active())
-    for (int row = rg.first_row(); row < rows; row += rg.row_step()) {
+    for (int row = rg.first_row(gr); row < rows; row += rg.row_step(gr)) {
       const int j = row % ny, k = row / ny;
       const double dydz = v.dy[j] * v.dz[k];
       const long long base = (long long)(k + 1) * v.sz + (long long)(j + 1) * v.sy + OX;
@@ -1380,22 +1393,33 @@ __global__ void __launch_bounds__(REDUCE_THREADS) k_gauge_sum(LV<double> v, cons
     if (threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
     __syncthreads();
   }
-  if (threadIdx.x == 0) partials[blockIdx.x] = sm[0];
+  if (threadIdx.x == 0) partials[gr.bx()] = sm[0];
+  clear_partials1(partials, gr.bx(), gr.gx());
 }
 
-__global__ void k_gauge_finalize(const double *partials, int nb, double *scal) {
+__global__ void __launch_bounds__(REDUCE_THREADS) k_gauge_sum(LV<double> v, const double *p, double *partials) {
+  gauge_sum_body(v, p, partials, HwGrid{});
+}
+
+__device__ __forceinline__ void gauge_finalize_body(const double *partials, int nb, double *scal) {
   double s = block_sum_partials(partials, nb, 1, 0);
   if (threadIdx.x == 0) scal[S_MEANP] = s / scal[S_FLUIDVOL];
 }
 
+__global__ void k_gauge_finalize(const double *partials, int nb, double *scal) {
+  gauge_finalize_body(partials, nb, scal);
+}
+
 // pack a user [k][j][i] array into a padded array (cells past nx in the last group get 0);
 // cells with mask == 1 (plain solid) are set to zero when mask is given
-__global__ void k_pack(const double *src, LevelGeom g, double *dst, const uint8_t *mask, unsigned *nonzero) {
+template <class GR>
+__device__ __forceinline__ void pack_body(const double *src, const LevelGeom &g, double *dst, const uint8_t *mask,
+                                          unsigned *nonzero, const GR &grid) {
   const RowGroups rg(g.nx);
   const int rows = g.ny * g.nz;
   if (!rg.active()) return;
   unsigned long long seen = 0;   // bits of the packed values (nonzero: some value is not +-0)
-  for (int row = rg.first_row(); row < rows; row += rg.row_step()) {
+  for (int row = rg.first_row(grid); row < rows; row += rg.row_step(grid)) {
     const int j = row % g.ny, k = row / g.ny;
     const long long q0 = (long long)row * g.nx;
     const long long base = (long long)(k + 1) * g.sz + (long long)(j + 1) * g.sy + OX;
@@ -1419,13 +1443,19 @@ __global__ void k_pack(const double *src, LevelGeom g, double *dst, const uint8_
     atomicOr(nonzero, 1u);
 }
 
+__global__ void k_pack(const double *src, LevelGeom g, double *dst, const uint8_t *mask, unsigned *nonzero) {
+  pack_body(src, g, dst, mask, nonzero, HwGrid{});
+}
+
 // unpack with the gauge applied: dst = p - mean on active cells, 0 on plain solid cells
-__global__ void k_unpack_gauge(const double *src, const uint8_t *mask, LevelGeom g, const double *scal, double *dst) {
+template <class GR>
+__device__ __forceinline__ void unpack_gauge_body(const double *src, const uint8_t *mask, const LevelGeom &g,
+                                                  const double *scal, double *dst, const GR &grid) {
   const RowGroups rg(g.nx);
   const int rows = g.ny * g.nz;
   if (!rg.active()) return;
   const double mean = scal[S_MEANP];
-  for (int row = rg.first_row(); row < rows; row += rg.row_step()) {
+  for (int row = rg.first_row(grid); row < rows; row += rg.row_step(grid)) {
     const int j = row % g.ny, k = row / g.ny;
     const long long q0 = (long long)row * g.nx;
     const long long base = (long long)(k + 1) * g.sz + (long long)(j + 1) * g.sy + OX;
@@ -1442,6 +1472,9 @@ __global__ void k_unpack_gauge(const double *src, const uint8_t *mask, LevelGeom
   }
 }
 
+__global__ void k_unpack_gauge(const double *src, const uint8_t *mask, LevelGeom g, const double *scal, double *dst) {
+  unpack_gauge_body(src, mask, g, scal, dst, HwGrid{});
+}
 
 // ------------------------------------------------------------------ double-FP32 outer loop
 
@@ -1606,9 +1639,7 @@ __global__ void __launch_bounds__(REDUCE_THREADS, RDF_PER_SM) k_residual_df(DfVi
 }
 // its blocks: one wave, but none without a row (an idle block's partials read zero either way)
 inline int rdf_blocks(const ibm_ctx *ctx, const LevelGeom &g) {
-  const long long G = (g.nx + 3) / 4, rpi = G >= REDUCE_THREADS ? 1 : REDUCE_THREADS / G;
-  const long long blocks = std::min(REDUCE_BLOCKS, RDF_PER_SM * (ctx->sm_count > 0 ? ctx->sm_count : 152));
-  return (int)std::min<long long>(blocks, ((long long)g.ny * g.nz + rpi - 1) / rpi);
+  return row_blocks(g, std::min(REDUCE_BLOCKS, RDF_PER_SM * (ctx->sm_count > 0 ? ctx->sm_count : 152)));
 }
 
 // ghost rows r_G = sum w v - g in FP64 from the split values; block partials of (s_G r_G)^2
@@ -1648,9 +1679,10 @@ __global__ void k_ghost_resid_df(const long long *src, const long long *dst, con
 }
 
 // ghost values g = sum w v from the split values (into gtmp), then stored split (Jacobi)
-__global__ void k_ghost_eval_df(const long long *src, const double *w, long long ng, const float *ph,
-                                const float *pl, double *gtmp, const double *gd) {
-  long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+template <class G>
+__device__ __forceinline__ void ghost_eval_df_body(const long long *src, const double *w, long long ng, const float *ph,
+                                                   const float *pl, double *gtmp, const double *gd, const G &gr) {
+  long long g = gr.bx() * (long long)blockDim.x + threadIdx.x;
   if (g >= ng) return;
   double s = GhostRow<double>(src, w, g).sum<double>([&](long long q) {
     q &= ~GHOST_CORNER;
@@ -1660,9 +1692,20 @@ __global__ void k_ghost_eval_df(const long long *src, const double *w, long long
   gtmp[g] = s;
 }
 
-__global__ void k_ghost_store_df(const long long *dst, long long ng, const double *gtmp, float *ph, float *pl) {
-  long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+__global__ void k_ghost_eval_df(const long long *src, const double *w, long long ng, const float *ph,
+                                const float *pl, double *gtmp, const double *gd) {
+  ghost_eval_df_body(src, w, ng, ph, pl, gtmp, gd, HwGrid{});
+}
+
+template <class G>
+__device__ __forceinline__ void ghost_store_df_body(const long long *dst, long long ng, const double *gtmp, float *ph,
+                                                    float *pl, const G &gr) {
+  long long g = gr.bx() * (long long)blockDim.x + threadIdx.x;
   if (g < ng) dfl::split(gtmp[g], ph[dst[g]], pl[dst[g]]);
+}
+
+__global__ void k_ghost_store_df(const long long *dst, long long ng, const double *gtmp, float *ph, float *pl) {
+  ghost_store_df_body(dst, ng, gtmp, ph, pl, HwGrid{});
 }
 
 // p += e (FP32 correction) on every padded cell, four at a time (n4 = ntot / 4)
@@ -1691,11 +1734,13 @@ __global__ void k_update_df(float4 *ph, float4 *pl, const float4 *e, long long n
 
 // pack a user [k][j][i] array into split padded arrays (cells past nx in the last group
 // get 0); cells with mask == 1 (plain solid) are set to zero when mask is given
-__global__ void k_pack_df(const double *src, LevelGeom g, float *dh, float *dl, const uint8_t *mask) {
+template <class GR>
+__device__ __forceinline__ void pack_df_body(const double *src, const LevelGeom &g, float *dh, float *dl,
+                                             const uint8_t *mask, const GR &grid) {
   const RowGroups rg(g.nx);
   const int rows = g.ny * g.nz;
   if (!rg.active()) return;
-  for (int row = rg.first_row(); row < rows; row += rg.row_step()) {
+  for (int row = rg.first_row(grid); row < rows; row += rg.row_step(grid)) {
     const int j = row % g.ny, k = row / g.ny;
     const long long q0 = (long long)row * g.nx;
     const long long base = (long long)(k + 1) * g.sz + (long long)(j + 1) * g.sy + OX;
@@ -1718,9 +1763,14 @@ __global__ void k_pack_df(const double *src, LevelGeom g, float *dh, float *dl, 
   }
 }
 
+__global__ void k_pack_df(const double *src, LevelGeom g, float *dh, float *dl, const uint8_t *mask) {
+  pack_df_body(src, g, dh, dl, mask, HwGrid{});
+}
+
 // block partials of sum V p over fluid cells; V and the products as pairs of floats
-__global__ void __launch_bounds__(REDUCE_THREADS) k_gauge_sum_df(DfView v, const float *ph, const float *pl,
-                                                                double *partials) {
+template <class G>
+__device__ __forceinline__ void gauge_sum_df_body(const DfView &v, const float *ph, const float *pl, double *partials,
+                                                  const G &gr) {
   __shared__ double sm[REDUCE_THREADS];
   const int nx = v.nx, ny = v.ny, n = nx + ny + v.nz;
   const float *H = v.h + 3 * n, *L = v.l + 3 * n;   // widths
@@ -1728,7 +1778,7 @@ __global__ void __launch_bounds__(REDUCE_THREADS) k_gauge_sum_df(DfView v, const
   const RowGroups rg(nx);
   const int rows = ny * v.nz;
   if (rg.active())
-    for (int row = rg.first_row(); row < rows; row += rg.row_step()) {
+    for (int row = rg.first_row(gr); row < rows; row += rg.row_step(gr)) {
       const int j = row % ny, k = row / ny;
       float ah = 0.f, al = 0.f, yzh, yzl;   // dy_j dz_k
       dfl::acc_prod(H[nx + j], L[nx + j], H[nx + ny + k], L[nx + ny + k], ah, al);
@@ -1757,18 +1807,26 @@ __global__ void __launch_bounds__(REDUCE_THREADS) k_gauge_sum_df(DfView v, const
     if (threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
     __syncthreads();
   }
-  if (threadIdx.x == 0) partials[blockIdx.x] = sm[0];
+  if (threadIdx.x == 0) partials[gr.bx()] = sm[0];
+  clear_partials1(partials, gr.bx(), gr.gx());
+}
+
+__global__ void __launch_bounds__(REDUCE_THREADS) k_gauge_sum_df(DfView v, const float *ph, const float *pl,
+                                                                double *partials) {
+  gauge_sum_df_body(v, ph, pl, partials, HwGrid{});
 }
 
 // unpack with the gauge applied (p - mean in pairs of floats, then one FP64 add per cell)
-__global__ void k_unpack_gauge_df(const float *ph, const float *pl, const uint8_t *mask, LevelGeom g,
-                                  const double *scal, double *dst) {
+template <class GR>
+__device__ __forceinline__ void unpack_gauge_df_body(const float *ph, const float *pl, const uint8_t *mask,
+                                                     const LevelGeom &g, const double *scal, double *dst,
+                                                     const GR &grid) {
   const RowGroups rg(g.nx);
   const int rows = g.ny * g.nz;
   if (!rg.active()) return;
   float mh, ml;
   dfl::split(scal[S_MEANP], mh, ml);
-  for (int row = rg.first_row(); row < rows; row += rg.row_step()) {
+  for (int row = rg.first_row(grid); row < rows; row += rg.row_step(grid)) {
     const int j = row % g.ny, k = row / g.ny;
     const long long q0 = (long long)row * g.nx;
     const long long base = (long long)(k + 1) * g.sz + (long long)(j + 1) * g.sy + OX;
@@ -1789,6 +1847,11 @@ __global__ void k_unpack_gauge_df(const float *ph, const float *pl, const uint8_
       }
     }
   }
+}
+
+__global__ void k_unpack_gauge_df(const float *ph, const float *pl, const uint8_t *mask, LevelGeom g,
+                                  const double *scal, double *dst) {
+  unpack_gauge_df_body(ph, pl, mask, g, scal, dst, HwGrid{});
 }
 
 // ------------------------------------------------------------------ membrane cut cells
@@ -2411,10 +2474,10 @@ void free_hierarchy(Hierarchy *h) {
   std::vector<void *> ps;
   for (Level &L : h->lv) {
     void *q[] = {L.mask, L.inner, L.e, L.r, L.fx, L.fy, L.fz, L.c1d, L.w1d, L.cen, L.poff, L.pt, L.wT, L.sdiag,
-                 L.zmask, L.ealt, L.zsd};
+                 L.ealt};
     ps.insert(ps.end(), q, q + sizeof(q) / sizeof(q[0]));
   }
-  void *q[] = {h->p64, h->b64, h->minv, h->gj, h->cidx, h->dncoarse, h->c64, h->cdf, h->xq, h->gsrc, h->gdst, h->gw64,
+  void *q[] = {h->p64, h->b64, h->minv, h->gj, h->cidx, h->dncoarse, h->c64, h->cdf, h->gsrc, h->gdst, h->gw64,
                h->zcount,
                h->gw32, h->gtmp, h->e_alt, h->tm_base[0], h->tm_base[1], h->d_fvol, h->d_ng,
                h->cut_id, h->cut_nb, h->cut_ijk, h->par_id, h->d_cnt, h->par_flag, h->scan_buf, h->gcr_buf,
@@ -2529,18 +2592,6 @@ static bool setup_zmarch_coarse(Hierarchy *h) {
   return true;
 }
 
-// separable diagonal parts of a level: sd = cm + cp per axis, from its coefficient array
-template <typename T>
-__global__ void k_sdiag(const T *c1d, int nx, int ny, int nz, T *sd) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = nx + ny + nz;
-  if (q >= n) return;
-  const T *cm = q < nx ? c1d : (q < nx + ny ? c1d + 2 * nx : c1d + 2 * nx + 2 * ny);
-  const int o = q < nx ? q : (q < nx + ny ? q - nx : q - nx - ny);
-  const int len = q < nx ? nx : (q < nx + ny ? ny : nz);
-  sd[q] = cm[o] + cm[len + o];
-}
-
 // z-march mask of a coarse level: plain solid (mask != 0) -> 1; fluid -> 8 when a face that
 // carries a coefficient is not fully open, else 0
 template <typename T>
@@ -2607,8 +2658,10 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
     Level L;
     L.g = make_geom((int)F[0][l].size() - 1, (int)F[1][l].size() - 1, (int)F[2][l].size() - 1);
     const int nx = L.g.nx, ny = L.g.ny, nz = L.g.nz;
-    HTRY(cudaMalloc((void **)&L.mask, L.g.ntot));
-    HTRY(cudaMemsetAsync(L.mask, 1, L.g.ntot, st));
+    // coarse levels: the mask of regular and irregular cells after the mask, in the same allocation
+    HTRY(cudaMalloc((void **)&L.mask, (l > 0 ? 2 : 1) * L.g.ntot));
+    if (l > 0) L.zmask = L.mask + L.g.ntot;
+    HTRY(cudaMemsetAsync(L.mask, 1, (l > 0 ? 2 : 1) * L.g.ntot, st));
     // the finest level's arrays end with one slot per membrane ghost entry; coarse levels
     // that the fused sweep takes store e and r in BF16 when asked
     const long long nel = l == 0 ? L.g.ntot + slotcap : L.g.ntot;
@@ -2620,7 +2673,8 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
       HTRY(alloc_zero<T>(&L.e, nel, st));
       HTRY(alloc_zero<T>(&L.r, nel, st));
     }
-    HTRY(cudaMalloc(&L.c1d, sizeof(T) * 2 * (nx + ny + nz)));
+    HTRY(cudaMalloc(&L.c1d, sizeof(T) * 3 * (nx + ny + nz)));
+    if (l > 0) L.zsd = (T *)L.c1d + 2 * (nx + ny + nz);   // separable diagonals, after the coefficients
     HTRY(cudaMalloc((void **)&L.w1d, sizeof(double) * (nx + ny + nz)));
     HTRY(cudaMalloc((void **)&L.cen, sizeof(double) * (nx + ny + nz)));
     HTRY(cudaMalloc(&L.wT, sizeof(T) * (nx + ny + nz)));
@@ -2628,7 +2682,7 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
     h->lv.push_back(L);
     Level &Lr = h->lv.back();
     const double *df = dfaces + foff[l];
-    T *c = (T *)Lr.c1d, *wt = (T *)Lr.wT, *sd = (T *)Lr.sdiag;
+    T *c = (T *)Lr.c1d, *wt = (T *)Lr.wT, *sd = (T *)(l == 0 ? Lr.sdiag : Lr.zsd);
     k_axis_level<T><<<nblk(nx, 128), 128, 0, st>>>(df, nx, c, c + nx, Lr.w1d, Lr.cen, wt, sd);
     k_axis_level<T><<<nblk(ny, 128), 128, 0, st>>>(df + nx + 1, ny, c + 2 * nx, c + 2 * nx + ny, Lr.w1d + nx,
                                                     Lr.cen + nx, wt + nx, sd ? sd + nx : nullptr);
@@ -2639,18 +2693,10 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
   }
   h->nslot = h->lv[0].g.ntot + slotcap;
   HTRY(alloc_zero<int>((void **)&h->zcount, nl, st));
-  // coarse levels: mask of regular and irregular cells, separable diagonals of the regular ones;
-  // the ones swept by the fused sweep: a second e buffer
+  // coarse levels swept by the fused sweep: a second e buffer
   for (int l = 1; l < nl; ++l) {
     Level &L = h->lv[l];
-    HTRY(cudaMalloc((void **)&L.zmask, L.g.ntot));
-    HTRY(cudaMemsetAsync(L.zmask, 1, L.g.ntot, st));
-    HTRY(cudaMalloc(&L.zsd, sizeof(T) * (L.g.nx + L.g.ny + L.g.nz)));
-    k_sdiag<T><<<nblk(L.g.nx + L.g.ny + L.g.nz, 128), 128, 0, st>>>((const T *)L.c1d, L.g.nx, L.g.ny, L.g.nz,
-                                                                    (T *)L.zsd);
-    HTRY(cudaGetLastError());
-    const long long cells = (long long)L.g.nx * L.g.ny * L.g.nz;
-    if (sizeof(T) == 4 && (L.bf16 || cells >= ZM_COARSE_CELLS)) {
+    if (sizeof(T) == 4 && (L.bf16 || (long long)L.g.nx * L.g.ny * L.g.nz >= ZM_COARSE_CELLS)) {
       if (L.bf16) HTRY(alloc_zero<bf16>(&L.ealt, L.g.ntot, st));
       else HTRY(alloc_zero<T>(&L.ealt, L.g.ntot, st));
       L.zm = true;
@@ -3347,12 +3393,12 @@ ibm_status build_hierarchy(ibm_tables *t, int precision, cudaStream_t st, bool c
     // split coefficients, diagonal parts (3n doubles of c64) and widths (n of w1d); the FP64
     // residual uses the high parts of the widths as FP32 volume weights
     float *cdf = nullptr;
-    BTRY(cudaMalloc((void **)&cdf, sizeof(float) * 8 * n));
+    const int nx4 = (nx + 3) / 4 * 4;
+    BTRY(cudaMalloc((void **)&cdf, sizeof(float) * (8 * n + XQ_ROWS * nx4)));
     h->cdf = cdf;
+    h->xq = cdf + 8 * n;   // in the same allocation, 16-byte aligned rows
     k_split_df<<<nblk(3 * n, 128), 128, 0, st>>>(h->c64, 3 * n, cdf, cdf + 4 * n);
     k_split_df<<<nblk(n, 128), 128, 0, st>>>(L0.w1d, n, cdf + 3 * n, cdf + 7 * n);
-    const int nx4 = (nx + 3) / 4 * 4;
-    BTRY(cudaMalloc((void **)&h->xq, sizeof(float) * XQ_ROWS * nx4));
     k_xq<<<nblk(nx4, 128), 128, 0, st>>>(cdf, cdf + 4 * n, nx, n, nx4, h->xq);
   }
   BTRY(cudaGetLastError());
@@ -3396,10 +3442,9 @@ struct Run {
   ibm_status result = IBM_ERR_NOT_CONVERGED;
 };
 
-// phase 1: hierarchy, packed inputs, and the residual of p = 0 (its norm is ||S P b||)
-ibm_status run_start(Run &R, ibm_ctx *ctx, ibm_tables *t, const double *rhs, const double *p_user,
-                     const ibm_solve_opts *opts, double *scal, double *part, double *hs, bool batched,
-                     cudaStream_t st) {
+// phase 1: the hierarchy, the solver's fields and the scalars' host copy
+ibm_status run_prepare(Run &R, ibm_ctx *ctx, ibm_tables *t, const ibm_solve_opts *opts, double *scal, double *part,
+                       double *hs, bool batched, cudaStream_t st) {
   R.ctx = ctx; R.t = t; R.opts = opts; R.prec = opts->precision; R.hs = hs;
   const bool cb = opts->coarse_bf16 != 0;
   ibm_status s = build_hierarchy(t, R.prec, st, cb);
@@ -3417,7 +3462,19 @@ ibm_status run_start(Run &R, ibm_ctx *ctx, ibm_tables *t, const double *rhs, con
   for (int q = 0; q < NSCAL; ++q) hs[q] = 0.0;
   hs[S_FLUIDVOL] = L0.fluid_vol;
   hs[S_NF] = (double)L0.nfluid;
-  IBM_TRY(cudaMemcpyAsync(scal, hs, sizeof(double) * NSCAL, cudaMemcpyHostToDevice, st));
+  R.r32 = R.prec != 0 ? (float *)L0.r : nullptr;
+  R.gcr_m = opts->krylov < 0 ? (t->membrane ? GCR_MAX : 0) : std::min(opts->krylov, GCR_MAX);
+  return IBM_OK;
+}
+
+// packed inputs, and the residual of p = 0 (its norm is ||S P b||)
+ibm_status run_pack(Run &R, const double *rhs, const double *p_user, cudaStream_t st) {
+  ibm_ctx *ctx = R.ctx;
+  ibm_tables *t = R.t;
+  Hierarchy *h = R.h;
+  Level &L0 = h->lv[0];
+  double *scal = R.S.scal;
+  IBM_TRY(cudaMemcpyAsync(scal, R.hs, sizeof(double) * NSCAL, cudaMemcpyHostToDevice, st));
   if (R.S.dfo) {
     k_pack_df<<<R.ctx->wave, 256, 0, st>>>(rhs, L0.g, hi_of(h->b64), lo_of(h->b64, R.ntot), nullptr);
     k_pack_df<<<R.ctx->wave, 256, 0, st>>>(p_user, L0.g, hi_of(h->p64), lo_of(h->p64, R.ntot), L0.mask);
@@ -3428,7 +3485,6 @@ ibm_status run_start(Run &R, ibm_ctx *ctx, ibm_tables *t, const double *rhs, con
   ctx->launches += 2;
   // the residual of p = 0 (its norm is ||S P b||); in mode 1 on closed bodies it also writes the
   // FP32 right-hand side b - lambda, which is the initial residual when the guess is zero
-  R.r32 = R.prec != 0 ? (float *)L0.r : nullptr;
   outer_residual(R.S, false, R.prec == 1 && !t->membrane ? R.r32 : nullptr, false);
   IBM_TRY(cudaGetLastError());
   return IBM_OK;
@@ -3436,16 +3492,30 @@ ibm_status run_start(Run &R, ibm_ctx *ctx, ibm_tables *t, const double *rhs, con
 
 // phase 2 (hs holds the norm of b): ghost values consistent with p, the Krylov state, and
 // the initial residual
-ibm_status run_begin(Run &R, cudaStream_t st) {
+void run_denom(Run &R) {
   const double bnorm = std::sqrt(R.hs[S_NORM2]);
   R.finite_b = std::isfinite(bnorm);
   R.denom = bnorm > 0 ? bnorm : 1.0;
+  R.ng = R.t->nghost;
+}
+
+// mode 1, zero guess (as packed, no ghost datum): the residual of p = 0 already computed the
+// initial residual's partial sums and wrote r = b - lambda (lambda still 0), and its ghost rows are zero;
+// finalising those sums with the lambda update gives the initial residual's scalars bit for bit
+bool run_zero_guess(const Run &R) {
+  uint64_t pnz_bits = 0;
+  std::memcpy(&pnz_bits, &R.hs[S_PNZ], sizeof pnz_bits);
+  return R.prec == 1 && !R.t->membrane && !R.t->has_datum && pnz_bits == 0;
+}
+
+ibm_status run_begin(Run &R, cudaStream_t st) {
+  run_denom(R);
   Hierarchy *h = R.h;
   ibm_tables *t = R.t;
   ibm_ctx *ctx = R.ctx;
   Level &L0 = h->lv[0];
   R.S.st = st;
-  const long long ntot = R.ntot, ng = R.ng = t->nghost;
+  const long long ntot = R.ntot, ng = R.ng;
   if (ng > 0 && R.S.dfo) {
     k_ghost_eval_df<<<nblk(ng, 128), 128, 0, st>>>(h->gsrc, t->gw, ng, hi_of(h->p64), lo_of(h->p64, ntot), h->gtmp,
                                                    t->has_datum ? t->gd : nullptr);
@@ -3459,8 +3529,6 @@ ibm_status run_begin(Run &R, cudaStream_t st) {
   }
   // Krylov acceleration of the refinement loop: directions (of the cycle's type), state,
   // partials.  Mode 0 with it runs in correction form like the mixed modes, in FP64.
-  const ibm_solve_opts *opts = R.opts;
-  R.gcr_m = opts->krylov < 0 ? (t->membrane ? GCR_MAX : 0) : std::min(opts->krylov, GCR_MAX);
   if (R.gcr_m > 0) {
     if (h->gcr_m < R.gcr_m) {
       if (h->gcr_buf) cudaFree(h->gcr_buf);
@@ -3480,12 +3548,7 @@ ibm_status run_begin(Run &R, cudaStream_t st) {
   R.S.gd = R.prec == 0 && R.gcr_m == 0 && t->has_datum ? t->gd : nullptr;
   // a zero initial guess (as packed) gives A p = 0 unless ghost rows carry a datum
   const unsigned *pnz = t->has_datum ? nullptr : reinterpret_cast<const unsigned *>(R.S.scal + S_PNZ);
-  uint64_t pnz_bits = 0;
-  std::memcpy(&pnz_bits, &R.hs[S_PNZ], sizeof pnz_bits);
-  if (R.prec == 1 && !t->membrane && !t->has_datum && pnz_bits == 0) {
-    // mode 1, zero guess: the residual of p = 0 already computed its partial sums and wrote
-    // r = b - lambda (lambda still 0), and its ghost rows are zero; finalising those sums with
-    // the lambda update gives the initial residual's scalars bit for bit
+  if (run_zero_guess(R)) {
     k_finalize_resid<<<1, 256, 0, st>>>(R.S.part, REDUCE_BLOCKS, nullptr, 0, R.S.scal, 1, nullptr, 0);
     ctx->launches += 1;
   } else if (R.r64) {
@@ -3580,10 +3643,10 @@ void run_finish(Run &R, double *p_user, cudaStream_t st) {
   const long long ntot = R.ntot;
   double *scal = R.S.scal, *part = R.S.part;
   if (R.S.dfo)
-    k_gauge_sum_df<<<REDUCE_BLOCKS, REDUCE_THREADS, 0, st>>>(fine_view_df(h), hi_of(h->p64), lo_of(h->p64, ntot),
+    k_gauge_sum_df<<<row_blocks(L0.g, REDUCE_BLOCKS), REDUCE_THREADS, 0, st>>>(fine_view_df(h), hi_of(h->p64), lo_of(h->p64, ntot),
                                                              part);
   else
-    k_gauge_sum<<<REDUCE_BLOCKS, REDUCE_THREADS, 0, st>>>(fine_view64(h), h->p64, part);
+    k_gauge_sum<<<row_blocks(L0.g, REDUCE_BLOCKS), REDUCE_THREADS, 0, st>>>(fine_view64(h), h->p64, part);
   k_gauge_finalize<<<1, 256, 0, st>>>(part, REDUCE_BLOCKS, scal);
   if (R.S.dfo)
     k_unpack_gauge_df<<<R.ctx->wave, 256, 0, st>>>(hi_of(h->p64), lo_of(h->p64, ntot), L0.mask, L0.g, scal, p_user);
@@ -3840,7 +3903,40 @@ struct PGres {
 struct PFin {
   const double *part, *gpart;
   double *scal;
-  int ngb;
+  int ngb, update;
+};
+// set-up and finish of the solves: packing, ghost values of p, gauge
+struct PPack {
+  const double *src;
+  LevelGeom g;
+  double *d64;        // FP64 destination, or the hi and lo parts
+  float *dh, *dl;
+  const uint8_t *mask;
+  unsigned *nonzero;
+  int gx;
+};
+struct PGhostP {
+  const long long *src, *dst;
+  const double *w, *gd;
+  long long ng;
+  double *p, *gtmp;   // FP64 p, or its parts
+  float *ph, *pl;
+};
+struct PGauge {
+  LV<double> v;
+  DfView vd;
+  const double *p;
+  const float *ph, *pl;
+  double *part, *scal;
+  int gx;
+};
+struct PUnpack {
+  const double *p, *scal;
+  const float *ph, *pl;
+  const uint8_t *mask;
+  LevelGeom g;
+  double *dst;
+  int gx;
 };
 static_assert(sizeof(BL<PRes>) <= 32764, "kernel parameters of at most 32764 bytes");
 
@@ -3871,7 +3967,40 @@ __global__ void kb_ghost_resid_df(const __grid_constant__ BL<PGres> L) {
 __global__ void kb_finalize_resid(const __grid_constant__ BL<PFin> L) {
   BL_BLOCK(L)
   (void)lb;
-  finalize_resid_body(p.part, REDUCE_BLOCKS, p.gpart, p.ngb, p.scal, 1, nullptr, 0);
+  finalize_resid_body(p.part, REDUCE_BLOCKS, p.gpart, p.ngb, p.scal, p.update, nullptr, 0);
+}
+__global__ void kb_pack(const __grid_constant__ BL<PPack> L) {
+  BL_BLOCK(L)
+  if (p.d64) pack_body(p.src, p.g, p.d64, p.mask, p.nonzero, vgrid(lb, p.gx, 1));
+  else pack_df_body(p.src, p.g, p.dh, p.dl, p.mask, vgrid(lb, p.gx, 1));
+}
+__global__ void kb_ghost_eval_p(const __grid_constant__ BL<PGhostP> L) {
+  BL_BLOCK(L)
+  if (p.p) ghost_eval_body<double, double>(p.src, p.dst, p.w, p.ng, nullptr, p.p, nullptr, p.gtmp, p.gd, vgrid(lb, 1 << 30, 1));
+  else ghost_eval_df_body(p.src, p.w, p.ng, p.ph, p.pl, p.gtmp, p.gd, vgrid(lb, 1 << 30, 1));
+}
+__global__ void kb_ghost_store_p(const __grid_constant__ BL<PGhostP> L) {
+  BL_BLOCK(L)
+  if (p.p) ghost_store_body<double>(p.dst, p.ng, nullptr, p.gtmp, p.p, vgrid(lb, 1 << 30, 1));
+  else ghost_store_df_body(p.dst, p.ng, p.gtmp, p.ph, p.pl, vgrid(lb, 1 << 30, 1));
+}
+__global__ void __launch_bounds__(REDUCE_THREADS) kb_gauge_sum(const __grid_constant__ BL<PGauge> L) {
+  BL_BLOCK(L)
+  gauge_sum_body(p.v, p.p, p.part, vgrid(lb, p.gx, 1));
+}
+__global__ void __launch_bounds__(REDUCE_THREADS) kb_gauge_sum_df(const __grid_constant__ BL<PGauge> L) {
+  BL_BLOCK(L)
+  gauge_sum_df_body(p.vd, p.ph, p.pl, p.part, vgrid(lb, p.gx, 1));
+}
+__global__ void kb_gauge_finalize(const __grid_constant__ BL<PGauge> L) {
+  BL_BLOCK(L)
+  (void)lb;
+  gauge_finalize_body(p.part, REDUCE_BLOCKS, p.scal);
+}
+__global__ void kb_unpack_gauge(const __grid_constant__ BL<PUnpack> L) {
+  BL_BLOCK(L)
+  if (p.p) unpack_gauge_body(p.p, p.mask, p.g, p.scal, p.dst, vgrid(lb, p.gx, 1));
+  else unpack_gauge_df_body(p.ph, p.pl, p.mask, p.g, p.scal, p.dst, vgrid(lb, p.gx, 1));
 }
 #undef BL_BLOCK
 static_assert(sizeof(TailArgs<float>) % 8 == 0, "tail arguments are copied as 8-byte words");
@@ -4150,10 +4279,8 @@ void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
   lk_smooth(K, l, mid, K.nu2);
 }
 
-// the outer step of every problem in act, as the single-problem run_outer takes it: p += e,
-// then the fine residual (FP64 in mode 1, double-FP32 in mode 2), its ghost rows and norms,
-// with lambda updated; one launch per kernel over all problems
-void lk_outer(Lock &K, const std::vector<int> &act) {
+// the outer update of every problem in act, p += e
+void lk_update(Lock &K, const std::vector<int> &act) {
   std::vector<Run> &R = *K.R;
   ibm_ctx *ctx = K.ctx;
   const bool dfo = R[act[0]].S.dfo;
@@ -4181,6 +4308,16 @@ void lk_outer(Lock &K, const std::vector<int> &act) {
                        else kb_update_p<<<b, 256, 0, K.st>>>(L);
                        ctx->launches += 1;
                      });
+}
+
+// the fine residual of every problem in act (FP64 in mode 1, double-FP32 in mode 2), its ghost rows
+// and norms, as the single-problem outer_residual takes it, with lambda updated when asked; without p the
+// residual of p = 0
+void lk_residual(Lock &K, const std::vector<int> &act, bool with_p, bool update) {
+  if (act.empty()) return;
+  std::vector<Run> &R = *K.R;
+  ibm_ctx *ctx = K.ctx;
+  const bool dfo = R[act[0]].S.dfo;
   bl_launch<PRes>(act, [&](int i) { return dfo ? rdf_blocks(ctx, R[i].h->lv[0].g) : REDUCE_BLOCKS; },
                   [&](int i) {
                     Hierarchy *h = R[i].h;
@@ -4197,8 +4334,9 @@ void lk_outer(Lock &K, const std::vector<int> &act) {
                       p.wf = h->cdf + 3 * (p.v.nx + p.v.ny + p.v.nz);
                       p.gx = REDUCE_BLOCKS;
                     }
+                    if (!with_p) p.ph = nullptr, p.p = nullptr;
                     p.lambda = R[i].S.scal + S_LAMBDA;
-                    p.r32 = R[i].r32;
+                    p.r32 = with_p || !dfo ? R[i].r32 : nullptr;
                     p.part = R[i].S.part;
                     return p;
                   },
@@ -4207,6 +4345,7 @@ void lk_outer(Lock &K, const std::vector<int> &act) {
                     else kb_residual64<<<b, REDUCE_THREADS, 0, K.st>>>(L);
                     ctx->launches += 1;
                   });
+  if (with_p)
   bl_launch<PGres>(act, [&](int i) { return R[i].t->nghost > 0 ? FIXED_BLOCKS : 0; },
                    [&](int i) {
                      Hierarchy *h = R[i].h;
@@ -4231,13 +4370,114 @@ void lk_outer(Lock &K, const std::vector<int> &act) {
                     p.part = R[i].S.part;
                     p.gpart = R[i].S.part + 3 * REDUCE_BLOCKS;
                     p.scal = R[i].S.scal;
-                    p.ngb = R[i].t->nghost > 0 ? FIXED_BLOCKS : 0;
+                    p.ngb = with_p && R[i].t->nghost > 0 ? FIXED_BLOCKS : 0;
+                    p.update = update;
                     return p;
                   },
                   [&](const BL<PFin> &L, int b) {
                     kb_finalize_resid<<<b, 256, 0, K.st>>>(L);
                     ctx->launches += 1;
                   });
+}
+
+// the outer step of every problem in act, as the single-problem run_outer takes it
+void lk_outer(Lock &K, const std::vector<int> &act) {
+  lk_update(K, act);
+  lk_residual(K, act, true, true);
+}
+
+// The set-up and finish of every problem in lockstep, the single-problem phases' kernels with one launch
+// over all problems each: run_pack, run_begin and run_finish launch about 15 kernels per problem,
+// which for 96 problems of edges 16 to 32 took 5.4 of 13.5 ms and as many launches as the host could issue.
+void lk_pack(Lock &K, const std::vector<int> &all, const double *const *rhs, double *const *p_user) {
+  std::vector<Run> &R = *K.R;
+  for (int what = 0; what < 2; ++what)   // the right-hand sides, then the initial guesses
+    bl_launch<PPack>(all, [&](int i) { return row_blocks(R[i].h->lv[0].g, K.ctx->wave); },
+                     [&](int i) {
+                       Hierarchy *h = R[i].h;
+                       double *a = what == 0 ? h->b64 : h->p64;
+                       PPack p{};
+                       p.src = what == 0 ? rhs[i] : p_user[i];
+                       p.g = h->lv[0].g;
+                       if (R[i].S.dfo) { p.dh = hi_of(a); p.dl = lo_of(a, R[i].ntot); }
+                       else p.d64 = a;
+                       p.mask = what == 0 ? nullptr : h->lv[0].mask;
+                       p.nonzero = what == 0 || R[i].S.dfo ? nullptr : reinterpret_cast<unsigned *>(R[i].S.scal + S_PNZ);
+                       p.gx = row_blocks(p.g, K.ctx->wave);
+                       return p;
+                     },
+                     [&](const BL<PPack> &L, int b) { kb_pack<<<b, 256, 0, K.st>>>(L); K.ctx->launches += 1; });
+  lk_residual(K, all, false, false);
+}
+
+void lk_begin(Lock &K, const std::vector<int> &all) {
+  std::vector<Run> &R = *K.R;
+  for (int i : all) run_denom(R[i]);
+  auto blocks = [&](int i) { return R[i].ng > 0 ? (int)nblk(R[i].ng, 128) : 0; };
+  auto fill = [&](int i) {
+    Hierarchy *h = R[i].h;
+    const ibm_tables *t = R[i].t;
+    PGhostP p{};
+    p.src = h->gsrc; p.dst = h->gdst; p.w = t->gw; p.gd = t->has_datum ? t->gd : nullptr;
+    p.ng = R[i].ng;
+    p.gtmp = h->gtmp;
+    if (R[i].S.dfo) { p.ph = hi_of(h->p64); p.pl = lo_of(h->p64, R[i].ntot); }
+    else p.p = h->p64;
+    return p;
+  };
+  bl_launch<PGhostP>(all, blocks, fill,
+                     [&](const BL<PGhostP> &L, int b) { kb_ghost_eval_p<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
+  bl_launch<PGhostP>(all, blocks, fill,
+                     [&](const BL<PGhostP> &L, int b) { kb_ghost_store_p<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
+  std::vector<int> zero, rest;
+  for (int i : all) (run_zero_guess(R[i]) ? zero : rest).push_back(i);
+  bl_launch<PFin>(zero, [](int) { return 1; },
+                  [&](int i) {
+                    PFin p{};
+                    p.part = R[i].S.part;
+                    p.scal = R[i].S.scal;
+                    p.update = 1;
+                    return p;
+                  },
+                  [&](const BL<PFin> &L, int b) { kb_finalize_resid<<<b, 256, 0, K.st>>>(L); K.ctx->launches += 1; });
+  lk_residual(K, rest, true, true);
+}
+
+void lk_finish(Lock &K, const std::vector<int> &all, double *const *p_user) {
+  std::vector<Run> &R = *K.R;
+  const bool dfo = R[all[0]].S.dfo;
+  auto fill = [&](int i) {
+    Hierarchy *h = R[i].h;
+    PGauge p{};
+    if (dfo) { p.vd = fine_view_df(h); p.ph = hi_of(h->p64); p.pl = lo_of(h->p64, R[i].ntot); }
+    else { p.v = fine_view64(h); p.p = h->p64; }
+    p.part = R[i].S.part;
+    p.scal = R[i].S.scal;
+    p.gx = row_blocks(h->lv[0].g, REDUCE_BLOCKS);
+    return p;
+  };
+  bl_launch<PGauge>(all, [&](int i) { return row_blocks(R[i].h->lv[0].g, REDUCE_BLOCKS); }, fill,
+                    [&](const BL<PGauge> &L, int b) {
+                      if (dfo) kb_gauge_sum_df<<<b, REDUCE_THREADS, 0, K.st>>>(L);
+                      else kb_gauge_sum<<<b, REDUCE_THREADS, 0, K.st>>>(L);
+                      K.ctx->launches += 1;
+                    });
+  bl_launch<PGauge>(all, [](int) { return 1; }, fill,
+                    [&](const BL<PGauge> &L, int b) { kb_gauge_finalize<<<b, 256, 0, K.st>>>(L); K.ctx->launches += 1; });
+  bl_launch<PUnpack>(all, [&](int i) { return row_blocks(R[i].h->lv[0].g, K.ctx->wave); },
+                     [&](int i) {
+                       Hierarchy *h = R[i].h;
+                       PUnpack p{};
+                       if (dfo) { p.ph = hi_of(h->p64); p.pl = lo_of(h->p64, R[i].ntot); }
+                       else p.p = h->p64;
+                       p.mask = h->lv[0].mask;
+                       p.g = h->lv[0].g;
+                       p.scal = R[i].S.scal;
+                       p.dst = p_user[i];
+                       p.gx = row_blocks(p.g, K.ctx->wave);
+                       return p;
+                     },
+                     [&](const BL<PUnpack> &L, int b) { kb_unpack_gauge<<<b, 256, 0, K.st>>>(L); K.ctx->launches += 1; });
 }
 
 // can the batch advance in lockstep: mixed precision, closed bodies, no Krylov acceleration,
@@ -4358,8 +4598,9 @@ ibm_status solve_impl(ibm_ctx *ctx, ibm_tables *t, const double *rhs, double tol
                       const ibm_solve_opts *opts, ibm_solve_info *info, cudaStream_t st) {
   if (opts->method == 1) return solve_bicgstab_impl(ctx, t, rhs, tol, p_user, opts, info, st);
   Run R;
-  ibm_status s = run_start(R, ctx, t, rhs, p_user, opts, ctx->scal, ctx->partials, ctx->hscal, false, st);
+  ibm_status s = run_prepare(R, ctx, t, opts, ctx->scal, ctx->partials, ctx->hscal, false, st);
   if (s != IBM_OK) return s;
+  if ((s = run_pack(R, rhs, p_user, st)) != IBM_OK) return s;
   auto readback = [&]() -> ibm_status {
     IBM_TRY(cudaMemcpyAsync(ctx->hscal, ctx->scal, sizeof(double) * NSCAL, cudaMemcpyDeviceToHost, st));
     IBM_TRY(cudaStreamSynchronize(st));
@@ -4429,21 +4670,13 @@ ibm_status solve_batched_impl(ibm_ctx *ctx, int n, ibm_tables *const *ts, const 
   };
   ibm_status s;
   for (int p = 0; p < n; ++p)
-    if ((s = run_start(R[p], ctx, ts[p], rhs[p], p_user[p], opts, ctx->bscal + (size_t)p * NSCAL,
-                       ctx->bpart + part_n * p, ctx->bhscal + (size_t)p * NSCAL, true, st)) != IBM_OK)
+    if ((s = run_prepare(R[p], ctx, ts[p], opts, ctx->bscal + (size_t)p * NSCAL, ctx->bpart + part_n * p,
+                         ctx->bhscal + (size_t)p * NSCAL, true, st)) != IBM_OK)
       return s;
-  if ((s = readback()) != IBM_OK) return s;
-  for (int p = 0; p < n; ++p)
-    if ((s = run_begin(R[p], st)) != IBM_OK) return s;
-  if ((s = readback()) != IBM_OK) return s;
-  int active = 0;
-  for (int p = 0; p < n; ++p) {
-    run_initial(R[p], tol);
-    active += R[p].active;
-  }
   const bool lock = lockstep_ok(R, opts);
   Lock K;
-  std::vector<char> graph(n, 0);
+  std::vector<int> all(n);
+  for (int p = 0; p < n; ++p) all[p] = p;
   if (lock) {
     K.ctx = ctx;
     K.st = st;
@@ -4452,12 +4685,33 @@ ibm_status solve_batched_impl(ibm_ctx *ctx, int n, ibm_tables *const *ts, const 
     K.nu2 = opts->nu2;
     K.omega = (float)opts->omega;
     if ((s = lockstep_setup(K, R)) != IBM_OK) return s;
+    IBM_TRY(cudaMemcpyAsync(ctx->bscal, ctx->bhscal, sizeof(double) * NSCAL * n, cudaMemcpyHostToDevice, st));
+    lk_pack(K, all, rhs, p_user);
   } else {
+    for (int p = 0; p < n; ++p)
+      if ((s = run_pack(R[p], rhs[p], p_user[p], st)) != IBM_OK) return s;
+  }
+  IBM_TRY(cudaGetLastError());
+  if ((s = readback()) != IBM_OK) return s;
+  if (lock) {
+    lk_begin(K, all);
+  } else {
+    for (int p = 0; p < n; ++p)
+      if ((s = run_begin(R[p], st)) != IBM_OK) return s;
+  }
+  IBM_TRY(cudaGetLastError());
+  if ((s = readback()) != IBM_OK) return s;
+  int active = 0;
+  for (int p = 0; p < n; ++p) {
+    run_initial(R[p], tol);
+    active += R[p].active;
+  }
+  std::vector<char> graph(n, 0);
+  if (!lock)
     for (int p = 0; p < n; ++p) {
       graph[p] = run_graphable(R[p]);
       if (graph[p] && (s = run_capture(R[p])) != IBM_OK) return s;
     }
-  }
   const int ns = std::min(n, (int)ibm_ctx::NBSTREAM);
   int it = 0;
   std::vector<int> act;
@@ -4487,7 +4741,9 @@ ibm_status solve_batched_impl(ibm_ctx *ctx, int n, ibm_tables *const *ts, const 
       active += R[p].active;
     }
   }
-  for (int p = 0; p < n; ++p) run_finish(R[p], p_user[p], st);
+  if (lock) lk_finish(K, all, p_user);
+  else
+    for (int p = 0; p < n; ++p) run_finish(R[p], p_user[p], st);
   IBM_TRY(cudaGetLastError());
   IBM_TRY(cudaMemcpyAsync(ctx->bhscal, ctx->bscal, sizeof(double) * NSCAL * n, cudaMemcpyDeviceToHost, st));
   ibm_status result = IBM_OK;
@@ -4691,8 +4947,9 @@ void bc_precond(Solver &S, Bicg &B, const double *x, double *y, int K, cudaStrea
 ibm_status solve_bicgstab_impl(ibm_ctx *ctx, ibm_tables *t, const double *rhs, double tol, double *p_user,
                                const ibm_solve_opts *opts, ibm_solve_info *info, cudaStream_t st) {
   Run R;
-  ibm_status s = run_start(R, ctx, t, rhs, p_user, opts, ctx->scal, ctx->partials, ctx->hscal, false, st);
+  ibm_status s = run_prepare(R, ctx, t, opts, ctx->scal, ctx->partials, ctx->hscal, false, st);
   if (s != IBM_OK) return s;
+  if ((s = run_pack(R, rhs, p_user, st)) != IBM_OK) return s;
   IBM_TRY(cudaMemcpyAsync(ctx->hscal, ctx->scal, sizeof(double) * NSCAL, cudaMemcpyDeviceToHost, st));
   IBM_TRY(cudaStreamSynchronize(st));
   const double bnorm = std::sqrt(ctx->hscal[S_NORM2]);
