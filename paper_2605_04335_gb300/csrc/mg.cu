@@ -1279,6 +1279,14 @@ __global__ void __launch_bounds__(REDUCE_THREADS) k_residual64(LV<double> v, con
   residual64_body<R, WP>(v, p, b, lambda, wf, r32, partials, p_nonzero, HwGrid{});
 }
 
+// launched as gx blocks: the slots of the others up to FIXED_BLOCKS read zero
+__device__ __forceinline__ void clear_ghost_partials(double *gpart, int bx, int gx) {
+  if (threadIdx.x == 0)
+    for (int b = bx + gx; b < FIXED_BLOCKS; b += gx) gpart[b] = 0.0;
+}
+// blocks of the ghost residual over ng rows (a launch for a count read on the device takes FIXED_BLOCKS)
+inline int ghost_resid_blocks(long long ng) { return (int)std::max<long long>(1, std::min<long long>(FIXED_BLOCKS, nblk(ng, REDUCE_THREADS))); }
+
 // ghost rows r_G = sum w v - g; block partials of (s_G r_G)^2 at gpart[b]
 template <typename R, class G>
 __device__ __forceinline__ void ghost_resid64_body(const long long *src, const long long *dst, const double *w,
@@ -1302,6 +1310,7 @@ __device__ __forceinline__ void ghost_resid64_body(const long long *src, const l
     __syncthreads();
   }
   if (threadIdx.x == 0) gpart[gr.bx()] = sm[0];
+  clear_ghost_partials(gpart, gr.bx(), gr.gx());
 }
 
 template <typename R>
@@ -1670,6 +1679,7 @@ __device__ __forceinline__ void ghost_resid_df_body(const long long *src, const 
     __syncthreads();
   }
   if (threadIdx.x == 0) gpart[gr.bx()] = sm[0];
+  clear_ghost_partials(gpart, gr.bx(), gr.gx());
 }
 
 __global__ void k_ghost_resid_df(const long long *src, const long long *dst, const double *w, const double *scale,
@@ -2516,6 +2526,12 @@ static bool make_map(CUtensorMap *m, void *base, CUtensorMapDataType dt, int ele
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Finest levels of fewer cells are relaxed strip by strip.  FP32: 96 problems of edges 16 to 32 take 5.0
+// against 5.9 ms, single solves of 24^3 to 64^3 the same either way within 2 %, 24 problems of edges 64
+// to 96 10.2 against 11.3 ms for the fused sweep (a batch that mixes both forms pays two launches per stage,
+// so the line lies at 32^3).  FP64: 24^3 1.39 against 1.70 ms, 64^3 2.44 against 2.93, 80^3 3.25 against 3.64.
+template <typename T>
+constexpr long long fused_cells() { return sizeof(T) == 4 ? (1LL << 15) + 1 : 1LL << 19; }
 template <typename T>
 static void setup_zmarch(Hierarchy *h, void *e0, void *r0) {
   Level &L0 = h->lv[0];
@@ -2537,6 +2553,9 @@ static void setup_zmarch(Hierarchy *h, void *e0, void *r0) {
     h->zm_per_sm = per_sm;
   else
     h->zmarch = false;
+  // small grids: tiles of 128 x 14 leave most lanes idle, and the strip relaxation (the same bits)
+  // with its ghost rows in two launches takes less
+  if ((long long)L0.g.nx * L0.g.ny * L0.g.nz < fused_cells<T>()) h->zmarch = false;
 }
 
 // Coarse levels swept by the fused z-march: levels >= 1 of at least ZM_COARSE_CELLS cells in
@@ -3058,7 +3077,7 @@ void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool
   Level &L = S.h->lv[l];
   LV<T> v = view<T>(L);
   const int kz = relax_kz<T>((long long)L.g.nx * L.g.ny * L.g.nz);
-  const bool sep = relax_sep<T>(L.g);
+  const bool sep = fine || relax_sep<T>(L.g);   // the finest level as its fused sweep
   const dim3 grid(relax_gx(L.g), (L.g.nz + kz - 1) / kz);
   for (int s = 0; s < sweeps; ++s) {
     const bool timed = fine && S.sweep_events && S.sweep_events->size() >= 2 * (size_t)(s + 1);
@@ -3899,6 +3918,7 @@ struct PGres {
   const float *ph, *pl;
   float *r32;
   double *gpart;
+  int gx;
 };
 struct PFin {
   const double *part, *gpart;
@@ -3958,11 +3978,11 @@ __global__ void __launch_bounds__(REDUCE_THREADS, RDF_PER_SM) kb_residual_df(con
 }
 __global__ void kb_ghost_resid64(const __grid_constant__ BL<PGres> L) {
   BL_BLOCK(L)
-  ghost_resid64_body<float>(p.src, p.dst, p.w, p.scale, p.ngp, p.p, p.r32, p.gpart, p.gd, vgrid(lb, FIXED_BLOCKS, 1));
+  ghost_resid64_body<float>(p.src, p.dst, p.w, p.scale, p.ngp, p.p, p.r32, p.gpart, p.gd, vgrid(lb, p.gx, 1));
 }
 __global__ void kb_ghost_resid_df(const __grid_constant__ BL<PGres> L) {
   BL_BLOCK(L)
-  ghost_resid_df_body(p.src, p.dst, p.w, p.scale, p.ngp, p.ph, p.pl, p.r32, p.gpart, p.gd, vgrid(lb, FIXED_BLOCKS, 1));
+  ghost_resid_df_body(p.src, p.dst, p.w, p.scale, p.ngp, p.ph, p.pl, p.r32, p.gpart, p.gd, vgrid(lb, p.gx, 1));
 }
 __global__ void kb_finalize_resid(const __grid_constant__ BL<PFin> L) {
   BL_BLOCK(L)
@@ -4131,19 +4151,28 @@ int lk_ghost_blocks(Lock &K, int i) {
   return (*K.R)[i].t->nghost > 0 ? (int)nblk(lk_h(K, i)->gcap, 128) : 0;
 }
 
+// the finest level's ghost rows from its current values (Jacobi: all rows evaluated, then stored)
+void lk_ghost_update(Lock &K, const std::vector<int> &grp) {
+  bl_launch<PGhost>(grp, [&](int i) { return lk_ghost_blocks(K, i); },
+                    [&](int i) { return lk_ghost(K, i, K.E[0][i], nullptr); },
+                    [&](const BL<PGhost> &L, int b) { kb_ghost_eval<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
+  bl_launch<PGhost>(grp, [&](int i) { return lk_ghost_blocks(K, i); },
+                    [&](int i) { return lk_ghost(K, i, K.E[0][i], nullptr); },
+                    [&](const BL<PGhost> &L, int b) { kb_ghost_store<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
+}
+
 void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
   for (int s = 0; s < sweeps; ++s) {
-    if (l == 0) {
-      std::vector<float *> old(K.E[0]);
-      lk_zmarch(K, 0, grp);
-      bl_launch<PGhost>(grp, [&](int i) { return lk_ghost_blocks(K, i); },
-                        [&](int i) { return lk_ghost(K, i, K.E[0][i], old[i]); },
-                        [&](const BL<PGhost> &L, int b) { kb_ghost_pp<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
-      continue;
-    }
     std::vector<int> zg, rg;
-    for (int i : grp) (lk_h(K, i)->lv[l].zm ? zg : rg).push_back(i);
-    if (!zg.empty()) lk_zmarch(K, l, zg);
+    for (int i : grp) ((l == 0 ? lk_h(K, i)->zmarch : lk_h(K, i)->lv[l].zm) ? zg : rg).push_back(i);
+    if (!zg.empty()) {
+      std::vector<float *> old(K.E[l]);
+      lk_zmarch(K, l, zg);
+      if (l == 0)
+        bl_launch<PGhost>(zg, [&](int i) { return lk_ghost_blocks(K, i); },
+                          [&](int i) { return lk_ghost(K, i, K.E[0][i], old[i]); },
+                          [&](const BL<PGhost> &L, int b) { kb_ghost_pp<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
+    }
     long long cells = 0;
     for (int i : rg) {
       const LevelGeom &g = lk_h(K, i)->lv[l].g;
@@ -4160,7 +4189,7 @@ void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
                          const Level &L = lk_h(K, i)->lv[l];
                          PRelax p;
                          p.v = view<float>(L); p.e = K.E[l][i]; p.r = lk_r(K, i, l); p.shift = lk_shift(K, i, l);
-                         p.gx = relax_gx(L.g); p.gy = (L.g.nz + kz - 1) / kz; p.sep = relax_sep<float>(L.g);
+                         p.gx = relax_gx(L.g); p.gy = (L.g.nz + kz - 1) / kz; p.sep = l == 0 || relax_sep<float>(L.g);
                          return p;
                        },
                        [&](const BL<PRelax> &L, int b) {
@@ -4168,6 +4197,7 @@ void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
                          else kb_relax<1><<<b, RELAX_THREADS, 0, K.st>>>(L, colour, K.omega);
                          K.ctx->launches += 1;
                        });
+    if (l == 0) lk_ghost_update(K, rg);
   }
 }
 
@@ -4268,14 +4298,7 @@ void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
                         kb_prolong8<<<b, 128, 0, K.st>>>(L);
                         K.ctx->launches += 1;
                       });
-  if (l == 0) {   // the corrected fluid values make the ghost rows stale
-    bl_launch<PGhost>(mid, [&](int i) { return lk_ghost_blocks(K, i); },
-                      [&](int i) { return lk_ghost(K, i, K.E[0][i], nullptr); },
-                      [&](const BL<PGhost> &L, int b) { kb_ghost_eval<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
-    bl_launch<PGhost>(mid, [&](int i) { return lk_ghost_blocks(K, i); },
-                      [&](int i) { return lk_ghost(K, i, K.E[0][i], nullptr); },
-                      [&](const BL<PGhost> &L, int b) { kb_ghost_store<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
-  }
+  if (l == 0) lk_ghost_update(K, mid);   // the corrected fluid values make the ghost rows stale
   lk_smooth(K, l, mid, K.nu2);
 }
 
@@ -4346,7 +4369,7 @@ void lk_residual(Lock &K, const std::vector<int> &act, bool with_p, bool update)
                     ctx->launches += 1;
                   });
   if (with_p)
-  bl_launch<PGres>(act, [&](int i) { return R[i].t->nghost > 0 ? FIXED_BLOCKS : 0; },
+  bl_launch<PGres>(act, [&](int i) { return R[i].t->nghost > 0 ? ghost_resid_blocks(R[i].t->nghost) : 0; },
                    [&](int i) {
                      Hierarchy *h = R[i].h;
                      const ibm_tables *t = R[i].t;
@@ -4357,6 +4380,7 @@ void lk_residual(Lock &K, const std::vector<int> &act, bool with_p, bool update)
                      else p.p = h->p64;
                      p.r32 = R[i].r32;
                      p.gpart = R[i].S.part + 3 * REDUCE_BLOCKS;
+                     p.gx = ghost_resid_blocks(R[i].t->nghost);
                      return p;
                    },
                    [&](const BL<PGres> &L, int b) {
@@ -4481,14 +4505,14 @@ void lk_finish(Lock &K, const std::vector<int> &all, double *const *p_user) {
 }
 
 // can the batch advance in lockstep: mixed precision, closed bodies, no Krylov acceleration,
-// FP32 coarse storage, and every finest level swept by the fused z-march on its own e and r
+// FP32 coarse storage, and every fused sweep of a finest level on its own e and r
 bool lockstep_ok(const std::vector<Run> &R, const ibm_solve_opts *opts) {
   if (R.empty() || opts->batch_schedule != 0 || opts->precision == 0 || opts->coarse_bf16) return false;
   for (const Run &r : R) {
     const Hierarchy *h = r.h;
-    if (r.t->membrane || r.gcr_m > 0 || h->hcnt[1] > 0 || h->hcnt[2] > 0 || !h->zmarch || h->elem != 4) return false;
+    if (r.t->membrane || r.gcr_m > 0 || h->hcnt[1] > 0 || h->hcnt[2] > 0 || h->elem != 4) return false;
     const void *e0 = h->lv[0].e;
-    if ((e0 != h->tm_base[0] && e0 != h->tm_base[1]) || (const void *)r.r32 != h->tm_rbase) return false;
+    if (h->zmarch && ((e0 != h->tm_base[0] && e0 != h->tm_base[1]) || (const void *)r.r32 != h->tm_rbase)) return false;
     if ((int)h->lv.size() > 1 && h->lv[1].bf16) return false;
   }
   return true;
