@@ -102,6 +102,94 @@ __global__ void __launch_bounds__(TX *TY) k_hz_sweep(HzView<T> v, const T *u, T 
   }
 }
 
+// The same step in FP32 (the correction cycles): a strip of four cells and KZ planes per thread, strips
+// numbered along x then y, every load of a thread before the arithmetic, and the strip's x
+// coefficients (xq: cxm, cxp, sdx in rows of nx4 floats) in 16-byte loads.  FIRST: the field is zero
+// (it is neither read nor cleared first).  HBM-bound, 13 bytes per cell (FIRST: 9): 42 us and 21 us at
+// 256^3, the one-cell-per-thread form 59 us for either
+constexpr int SW_THREADS = 128, SW_KZ = 2;
+template <bool FIRST>
+__global__ void __launch_bounds__(SW_THREADS) k_hz_sweep4(HzView<float> v, const float *xq, const float *u, float *un,
+                                                          const float *f, float w) {
+  const int groups = (v.nx + 3) >> 2, nx4 = 4 * groups;
+  const int strip = blockIdx.x * SW_THREADS + threadIdx.x, j = strip / groups, g = strip - j * groups;
+  const int k0 = blockIdx.y * SW_KZ;
+  if (j >= v.ny) return;
+  auto ld = [](const float *p, float (&a)[4]) {
+    const float4 q = *reinterpret_cast<const float4 *>(p);
+    a[0] = q.x; a[1] = q.y; a[2] = q.z; a[3] = q.w;
+  };
+  const long long id0 = ((long long)(k0 + 1) * (v.ny + 2) + (j + 1)) * v.sy + OX + 4 * g;
+  float C[SW_KZ + 2][4], N[SW_KZ][4], S[SW_KZ][4], F[SW_KZ][4], xl[SW_KZ], xr[SW_KZ];
+  unsigned m[SW_KZ];
+#pragma unroll
+  for (int q = 0; q < SW_KZ; ++q) {
+    const long long id = id0 + q * v.sz;
+    const bool in = k0 + q < v.nz;   // plane nz of an odd grid's last pair is the halo
+    m[q] = in ? *reinterpret_cast<const unsigned *>(v.mask + id) : 0xffffffffu;
+    ld(f + id, F[q]);
+    if (!FIRST) {
+      ld(u + id, C[q + 1]);
+      if (in) {
+        ld(u + id - v.sy, N[q]);
+        ld(u + id + v.sy, S[q]);
+        xl[q] = u[id - 1];
+        xr[q] = u[id + 4];
+      }
+    }
+  }
+  if (!FIRST) {
+    ld(u + id0 - v.sz, C[0]);
+    if (k0 + SW_KZ <= v.nz) ld(u + id0 + SW_KZ * v.sz, C[SW_KZ + 1]);
+  }
+  float cm[4], cp[4], sd[4];
+  ld(xq + 4 * g, cm);
+  ld(xq + nx4 + 4 * g, cp);
+  ld(xq + 2 * nx4 + 4 * g, sd);
+  const float cym = v.cym[j], cyp = v.cyp[j], sdy = v.sdy[j];
+#pragma unroll
+  for (int q = 0; q < SW_KZ; ++q) {
+    const int k = min(k0 + q, v.nz - 1);
+    const float czm = v.czm[k], czp = v.czp[k], sdz = v.sdz[k];
+    float out[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const float D = (1.0f + (sd[a] + sdy)) + sdz, rr = w * relax_rcp(D);
+      if (FIRST) {
+        out[a] = rr * F[q][a];
+      } else {
+        float s = cm[a] * (a == 0 ? xl[q] : C[q + 1][a > 0 ? a - 1 : 0]);
+        s = fmaf(cp[a], a == 3 ? xr[q] : C[q + 1][a < 3 ? a + 1 : 3], s);
+        s = fmaf(cym, N[q][a], s);
+        s = fmaf(cyp, S[q][a], s);
+        s = fmaf(czm, C[q][a], s);
+        s = fmaf(czp, C[q + 2][a], s);
+        const float c = C[q + 1][a], res = fmaf(-D, c, F[q][a]) + s;
+        out[a] = fmaf(rr, res, c);
+      }
+    }
+    float *o = un + id0 + q * v.sz;
+    if (m[q] == 0u) {
+      *reinterpret_cast<float4 *>(o) = make_float4(out[0], out[1], out[2], out[3]);
+    } else {
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        if (((m[q] >> (8 * a)) & 0xffu) == 0u) o[a] = out[a];
+    }
+  }
+}
+
+// x coefficients in rows of nx4 floats (entries past nx repeat the last): alpha x cxm, cxp, sdx (hi
+// parts, the FP32 sweep's), then their lo parts
+constexpr int HZ_XQ = 6;
+__global__ void k_hz_xq(const float *h, const float *l, int nx, int na, int nx4, float *xq) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nx4) return;
+  const int c = min(i, nx - 1);
+  const float q[HZ_XQ] = {h[c], h[nx + c], h[2 * na + c], l[c], l[nx + c], l[2 * na + c]};
+  for (int r = 0; r < HZ_XQ; ++r) xq[r * nx4 + i] = q[r];
+}
+
 // the same step at the membrane cut cells (their links read the entries through cut_nb)
 template <typename T>
 __global__ void k_hz_sweep_cut(HzView<T> v, const long long *cut_id, const long long *cut_nb, const int *cut_ijk,
@@ -119,7 +207,7 @@ __global__ void k_hz_sweep_cut(HzView<T> v, const long long *cut_id, const long 
   }
 }
 
-// ghost rows from the new fluid values and the previous ghost values:
+// ghost rows from the new fluid values and the previous ghost values (u null: they are zero):
 // u_G = (b_G - (1 - w_s) sum w v) / (1 + w_s), b_G = f at the ghost's slot
 template <typename T>
 __global__ void k_hz_ghost(const long long *src, const long long *dst, const double *gw, const double *ws,
@@ -129,7 +217,9 @@ __global__ void k_hz_ghost(const long long *src, const long long *dst, const dou
   const GhostRow<double> row(src, gw, g);
   const long long d = dst[g];
   const T b = f[d], w = (T)ws[g];
-  const T s = row.sum<T>([&](long long q) { return (q & GHOST_CORNER) ? u[q & ~GHOST_CORNER] : un[q]; });
+  const T s = row.sum<T>([&](long long q) {
+    return (q & GHOST_CORNER) ? (u ? u[q & ~GHOST_CORNER] : (T)0) : un[q];
+  });
   un[d] = (b - ((T)1 - w) * s) / ((T)1 + w);
 }
 
@@ -263,78 +353,138 @@ __device__ __forceinline__ void df_add(float ah, float al, float bh, float bl, f
   dfl::fast_two_sum(s, e, sh, sl);
 }
 
-__global__ void __launch_bounds__(HZ_THREADS) k_hz_resid_df(HzView<double> v, HzDf c, const float *uh,
-                                                            const float *ul, const float *fh, const float *fl,
-                                                            float *r32, double *part, bool with_b) {
+// Bound by the latency of its loads: a thread marches a strip of four cells through kz planes with three
+// planes of u in registers and the next plane's u, f and mask loaded one plane ahead; products and
+// sums are packed two cells to an instruction.  One warp per row, each lane four cells with the
+// neighbour planes reloaded, took 135 us at 256^3; this takes 106
+__global__ void __launch_bounds__(HZ_THREADS, 2) k_hz_resid_df(HzView<double> v, HzDf c, const float *xq, const float *uh,
+                                                               const float *ul, const float *fh, const float *fl,
+                                                               float *r32, double *part, bool with_b, int kz) {
+  using namespace dfl;
   __shared__ double sr[HZ_THREADS], sb[HZ_THREADS];
-  const int nx = v.nx, ny = v.ny, nz = v.nz, na = nx + ny + nz;
+  const int nx = v.nx, ny = v.ny, nz = v.nz, na = nx + ny + nz, groups = (nx + 3) >> 2, nx4 = 4 * groups;
   const long long sy = v.sy, sz = v.sz;
   // coefficient offsets in the layout cxm cxp cym cyp czm czp (2 na) then sdx sdy sdz (na)
-  const float *cxmh = c.ch, *cxml = c.cl, *cxph = c.ch + nx, *cxpl = c.cl + nx;
   const float *cyh = c.ch + 2 * nx, *cyl = c.cl + 2 * nx, *czh = c.ch + 2 * nx + 2 * ny, *czl = c.cl + 2 * nx + 2 * ny;
   const float *sdh = c.ch + 2 * na, *sdl = c.cl + 2 * na;
   double dr = 0.0, db = 0.0;
-  // one warp per row, each lane four consecutive cells (16-byte loads: rows start at OX = 4 of
-  // a 16-float pitch, so every group is aligned); the halo and padding masks are non-zero
-  const int lane = threadIdx.x & 31;
-  const long long rows = (long long)ny * nz, wstep = (long long)gridDim.x * (HZ_THREADS / 32);
-  const int ngroups = (nx + 3) / 4;
-  for (long long row = blockIdx.x * (long long)(HZ_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += wstep) {
-    const int j = (int)(row % ny), k = (int)(row / ny);
-    const long long base = ((long long)(k + 1) * (ny + 2) + (j + 1)) * sy + OX;
-    const float cymh = cyh[j], cyml = cyl[j], cyph = cyh[ny + j], cypl = cyl[ny + j];
-    const float czmh = czh[k], czml = czl[k], czph = czh[nz + k], czpl = czl[nz + k];
-    float dyzh, dyzl, t1h, t1l;
+  auto two = [](float x) { return f2(x, x); };
+  auto ld = [](const float *q, F2 (&r)[2]) {   // a strip as two pairs
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(q);
+    r[0].v = a.x;
+    r[1].v = a.y;
+  };
+  const int sblocks = (groups * ny + HZ_THREADS - 1) / HZ_THREADS;
+  const int items = sblocks * ((nz + kz - 1) / kz);
+  for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    const int chunk = item / sblocks, strip = (item - chunk * sblocks) * HZ_THREADS + (int)threadIdx.x;
+    const int j = strip / groups, g = strip - j * groups;
+    if (j >= ny) continue;
+    const int k0 = chunk * kz, k1 = min(nz, k0 + kz);
+    const float *x = xq + 4 * g;
+    const F2 ymh = two(cyh[j]), yml = two(cyl[j]), yph = two(cyh[ny + j]), ypl = two(cyl[ny + j]);
+    float t1h, t1l;
     df_add(1.0f, 0.0f, sdh[nx + j], sdl[nx + j], t1h, t1l);
-    df_add(t1h, t1l, sdh[nx + ny + k], sdl[nx + ny + k], dyzh, dyzl);
+    long long id = ((long long)(k0 + 1) * (ny + 2) + (j + 1)) * sy + OX + 4 * g;
+    F2 MH[2], ML[2], PH[2], PL[2], UH[2], UL[2], FH[2], FL[2];   // u in planes k - 1, k, k + 1; f in plane k
+    ld(uh + id - sz, MH);
+    ld(ul + id - sz, ML);
+    ld(uh + id, PH);
+    ld(ul + id, PL);
+    ld(uh + id + sz, UH);
+    ld(ul + id + sz, UL);
+    ld(fh + id, FH);
+    ld(fl + id, FL);
+    unsigned mn = *reinterpret_cast<const unsigned *>(v.mask + id);
     float ar = 0.f, ab = 0.f;
-    for (int g = lane; g < ngroups; g += 32) {
-      const long long id = base + 4 * g;
-      const uchar4 m4 = *reinterpret_cast<const uchar4 *>(v.mask + id);
-      const uint8_t mk[4] = {m4.x, m4.y, m4.z, m4.w};
-      if (mk[0] && mk[1] && mk[2] && mk[3]) continue;
-      const float4 ch4 = *reinterpret_cast<const float4 *>(uh + id), cl4 = *reinterpret_cast<const float4 *>(ul + id);
-      const float4 f4h = *reinterpret_cast<const float4 *>(fh + id), f4l = *reinterpret_cast<const float4 *>(fl + id);
-      const float Ch[6] = {uh[id - 1], ch4.x, ch4.y, ch4.z, ch4.w, uh[id + 4]};
-      const float Cl[6] = {ul[id - 1], cl4.x, cl4.y, cl4.z, cl4.w, ul[id + 4]};
-      const float Fh[4] = {f4h.x, f4h.y, f4h.z, f4h.w}, Fl[4] = {f4l.x, f4l.y, f4l.z, f4l.w};
-      float R[4];
-      // neighbours in y and z, one pair of 16-byte loads each, consumed one at a time
-      float acc_h[4], acc_l[4];
+    int nplane = 0;
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k, id += sz) {
+      const unsigned m = mn;
+      F2 NH[2][2], NL[2][2], cc[2], cl[2], sh[2], sl[2], b[2], wh[2], wl[2], gh[2], gl[2];
+      ld(uh + id - sy, NH[0]);
+      ld(ul + id - sy, NL[0]);
+      ld(uh + id + sy, NH[1]);
+      ld(ul + id + sy, NL[1]);
+      const float xlh = uh[id - 1], xll = ul[id - 1], xrh = uh[id + 4], xrl = ul[id + 4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { acc_h[q] = Fh[q]; acc_l[q] = Fl[q]; }
-#pragma unroll
-      for (int nb = 0; nb < 4; ++nb) {
-        const long long off = nb == 0 ? -sy : (nb == 1 ? sy : (nb == 2 ? -sz : sz));
-        const float4 h4 = *reinterpret_cast<const float4 *>(uh + id + off);
-        const float4 l4 = *reinterpret_cast<const float4 *>(ul + id + off);
-        const float H[4] = {h4.x, h4.y, h4.z, h4.w}, L[4] = {l4.x, l4.y, l4.z, l4.w};
-        const float cH = nb == 0 ? cymh : (nb == 1 ? cyph : (nb == 2 ? czmh : czph));
-        const float cL = nb == 0 ? cyml : (nb == 1 ? cypl : (nb == 2 ? czml : czpl));
-#pragma unroll
-        for (int q = 0; q < 4; ++q) dfl::acc_prod(cH, cL, H[q], L[q], acc_h[q], acc_l[q]);
+      for (int q = 0; q < 2; ++q) {
+        sh[q] = FH[q];
+        sl[q] = FL[q];
+        b[q] = add2(FH[q], FL[q]);
+        wh[q] = UH[q];
+        wl[q] = UL[q];
+        gh[q] = FH[q];
+        gl[q] = FL[q];
       }
+      if (k + 1 < k1) {
+        mn = *reinterpret_cast<const unsigned *>(v.mask + id + sz);
+        ld(uh + id + 2 * sz, wh);
+        ld(ul + id + 2 * sz, wl);
+        ld(fh + id + sz, gh);
+        ld(fl + id + sz, gl);
+      }
+      float dyzh, dyzl;
+      df_add(t1h, t1l, sdh[nx + ny + k], sdl[nx + ny + k], dyzh, dyzl);
+      const F2 zmh = two(czh[k]), zml = two(czl[k]), zph = two(czh[nz + k]), zpl = two(czl[nz + k]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = min(4 * g + q, nx - 1);
-        float Dh, Dl;
-        df_add(dyzh, dyzl, sdh[i], sdl[i], Dh, Dl);
-        dfl::acc_prod(-Dh, -Dl, Ch[q + 1], Cl[q + 1], acc_h[q], acc_l[q]);
-        dfl::acc_prod(cxmh[i], cxml[i], Ch[q], Cl[q], acc_h[q], acc_l[q]);
-        dfl::acc_prod(cxph[i], cxpl[i], Ch[q + 2], Cl[q + 2], acc_h[q], acc_l[q]);
-        R[q] = acc_h[q] + acc_l[q];
-        if (mk[q] == 0) {
+      for (int q = 0; q < 2; ++q) {
+        acc_prod2(ymh, yml, NH[0][q], NL[0][q], sh[q], sl[q]);
+        acc_prod2(yph, ypl, NH[1][q], NL[1][q], sh[q], sl[q]);
+        acc_prod2(zmh, zml, MH[q], ML[q], sh[q], sl[q]);
+        acc_prod2(zph, zpl, UH[q], UL[q], sh[q], sl[q]);
+      }
+      ld(x + 2 * nx4, cc);
+      ld(x + 5 * nx4, cl);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        // D = (1 + sdy + sdz) + sdx as a renormalised pair, then -D u
+        F2 t, e;
+        two_sum2(two(dyzh), cc[q], t, e);
+        e = add2(e, add2(two(dyzl), cl[q]));
+        const F2 Dh = add2(t, e), Dl = sub2(e, sub2(Dh, t));
+        acc_prod_neg2(Dh, neg2(Dh), neg2(Dl), PH[q], PL[q], sh[q], sl[q]);
+      }
+      float p0, p1, p2, p3, q0, q1, q2, q3;
+      un2(PH[0], p0, p1);
+      un2(PH[1], p2, p3);
+      un2(PL[0], q0, q1);
+      un2(PL[1], q2, q3);
+      ld(x, cc);
+      ld(x + 3 * nx4, cl);
+      acc_prod2(cc[0], cl[0], f2(xlh, p0), f2(xll, q0), sh[0], sl[0]);
+      acc_prod2(cc[1], cl[1], f2(p1, p2), f2(q1, q2), sh[1], sl[1]);
+      ld(x + nx4, cc);
+      ld(x + 4 * nx4, cl);
+      acc_prod2(cc[0], cl[0], f2(p1, p2), f2(q1, q2), sh[0], sl[0]);
+      acc_prod2(cc[1], cl[1], f2(p3, xrh), f2(q3, xrl), sh[1], sl[1]);
+      float R[4], B[4];
+      un2(add2(sh[0], sl[0]), R[0], R[1]);
+      un2(add2(sh[1], sl[1]), R[2], R[3]);
+      un2(b[0], B[0], B[1]);
+      un2(b[1], B[2], B[3]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (((m >> (8 * q)) & 0xffu) == 0u) {
           ar = fmaf(R[q], R[q], ar);
-          if (with_b) { const float b = Fh[q] + Fl[q]; ab = fmaf(b, b, ab); }
+          if (with_b) ab = fmaf(B[q], B[q], ab);
+          if (r32 && m != 0u) r32[id + q] = R[q];
         }
+      if (r32 && m == 0u) *reinterpret_cast<float4 *>(r32 + id) = make_float4(R[0], R[1], R[2], R[3]);
+      if (++nplane == 2 || k + 1 == k1) {   // the float sums of a few cells into FP64
+        dr += widen(ar);
+        if (with_b) db += widen(ab);
+        ar = ab = 0.f;
+        nplane = 0;
       }
-      if (r32)
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (mk[q] == 0) r32[id + q] = R[q];
+      for (int q = 0; q < 2; ++q) {
+        MH[q] = PH[q]; ML[q] = PL[q];
+        PH[q] = UH[q]; PL[q] = UL[q];
+        UH[q] = wh[q]; UL[q] = wl[q];
+        FH[q] = gh[q]; FL[q] = gl[q];
+      }
     }
-    dr += dfl::widen(ar);   // per row: the float sums of a lane's few groups
-    if (with_b) db += dfl::widen(ab);
   }
   sr[threadIdx.x] = dr;
   sb[threadIdx.x] = db;
@@ -356,16 +506,35 @@ __global__ void k_hz_update_df(float *uh, float *ul, const float *e, long long n
   }
 }
 
-__global__ void k_hz_pack_df(const double *f, const double *u, long long ncell, int nx, int ny, LevelGeom g,
-                             const uint8_t *mask, float *fh, float *fl, float *uh, float *ul) {
-  // grid: (x blocks, ny, nz); no divisions
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
+// Packs and unpacks stream 33 and 17 bytes per cell: a thread takes one cell of four rows of a plane,
+// all loads before the stores (one row per thread keeps a quarter of the bytes in flight: 180 and 97 us at 256^3, this 103 and 57);
+// the split into pairs runs on the integer pipe (dfloat.cuh)
+constexpr int HZ_PK = 128, HZ_PKR = 4;   // grid: (x blocks, row groups, nz)
+template <class LD, class ST>
+__device__ __forceinline__ void hz_rows(int nx, int ny, LevelGeom g, const uint8_t *mask, LD ld, ST st) {
+  const int i = blockIdx.x * HZ_PK + threadIdx.x, j0 = blockIdx.y * HZ_PKR, k = blockIdx.z;
   if (i >= nx) return;
-  const long long l = ((long long)k * ny + j) * nx + i;
-  const long long id = pidx(g, i, j, k);
-  const uint8_t m = mask[id];
-  dfl::split(fluid_row(m) ? f[l] : 0.0, fh[id], fl[id]);
-  dfl::split((fluid_row(m) || m == 3) ? u[l] : 0.0, uh[id], ul[id]);
+  const long long l0 = ((long long)k * ny + j0) * nx + i, id0 = pidx(g, i, j0, k);
+  double2 x[HZ_PKR];
+  uint8_t m[HZ_PKR];
+#pragma unroll
+  for (int q = 0; q < HZ_PKR; ++q)
+    if (j0 + q < ny) {
+      m[q] = mask[id0 + q * g.sy];
+      x[q] = ld(l0 + (long long)q * nx, id0 + q * g.sy);
+    }
+#pragma unroll
+  for (int q = 0; q < HZ_PKR; ++q)
+    if (j0 + q < ny) st(l0 + (long long)q * nx, id0 + q * g.sy, fluid_row(m[q]), fluid_row(m[q]) || m[q] == 3, x[q]);
+}
+
+__global__ void __launch_bounds__(HZ_PK) k_hz_pack_df(const double *f, const double *u, int nx, int ny, LevelGeom g,
+                                                      const uint8_t *mask, float *fh, float *fl, float *uh, float *ul) {
+  hz_rows(nx, ny, g, mask, [&](long long l, long long) { return make_double2(f[l], u[l]); },
+          [&](long long, long long id, bool fluid, bool active, double2 x) {
+            dfl::split(fluid ? x.x : 0.0, fh[id], fl[id]);
+            dfl::split(active ? x.y : 0.0, uh[id], ul[id]);
+          });
 }
 
 __global__ void k_hz_ghost_rhs_df(const long long *dst, const double *ub, long long ng, float *fh, float *fl) {
@@ -373,28 +542,20 @@ __global__ void k_hz_ghost_rhs_df(const long long *dst, const double *ub, long l
   if (g < ng) dfl::split(ub ? 2.0 * ub[g] : 0.0, fh[dst[g]], fl[dst[g]]);
 }
 
-__global__ void k_hz_unpack_df(const float *uh, const float *ul, long long ncell, int nx, int ny, LevelGeom g,
-                               const uint8_t *mask, double *u) {
-  // grid: (x blocks, ny, nz); no divisions
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
-  if (i >= nx) return;
-  const long long l = ((long long)k * ny + j) * nx + i;
-  const long long id = pidx(g, i, j, k);
-  const uint8_t m = mask[id];
-  u[l] = (fluid_row(m) || m == 3) ? dfl::join(uh[id], ul[id]) : 0.0;
+__global__ void __launch_bounds__(HZ_PK) k_hz_unpack_df(const float *uh, const float *ul, int nx, int ny, LevelGeom g,
+                                                        const uint8_t *mask, double *u) {
+  hz_rows(nx, ny, g, mask, [&](long long, long long id) { return make_double2(dfl::join(uh[id], ul[id]), 0.0); },
+          [&](long long l, long long, bool, bool active, double2 x) { u[l] = active ? x.x : 0.0; });
 }
 
 // user layout -> padded: f on fluid rows (0 elsewhere), u on fluid and ghost cells
-__global__ void k_hz_pack(const double *f, const double *u, long long ncell, int nx, int ny, LevelGeom g,
-                          const uint8_t *mask, double *fp, double *up) {
-  // grid: (x blocks, ny, nz); no divisions
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
-  if (i >= nx) return;
-  const long long l = ((long long)k * ny + j) * nx + i;
-  const long long id = pidx(g, i, j, k);
-  const uint8_t m = mask[id];
-  fp[id] = fluid_row(m) ? f[l] : 0.0;
-  up[id] = (fluid_row(m) || m == 3) ? u[l] : 0.0;
+__global__ void __launch_bounds__(HZ_PK) k_hz_pack(const double *f, const double *u, int nx, int ny, LevelGeom g,
+                                                   const uint8_t *mask, double *fp, double *up) {
+  hz_rows(nx, ny, g, mask, [&](long long l, long long) { return make_double2(f[l], u[l]); },
+          [&](long long, long long id, bool fluid, bool active, double2 x) {
+            fp[id] = fluid ? x.x : 0.0;
+            up[id] = active ? x.y : 0.0;
+          });
 }
 
 // ghost-row right-hand sides 2 u_b at the ghosts' slots
@@ -403,15 +564,10 @@ __global__ void k_hz_ghost_rhs(const long long *dst, const double *ub, long long
   if (g < ng) fp[dst[g]] = ub ? 2.0 * ub[g] : 0.0;
 }
 
-__global__ void k_hz_unpack(const double *up, long long ncell, int nx, int ny, LevelGeom g, const uint8_t *mask,
-                            double *u) {
-  // grid: (x blocks, ny, nz); no divisions
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
-  if (i >= nx) return;
-  const long long l = ((long long)k * ny + j) * nx + i;
-  const long long id = pidx(g, i, j, k);
-  const uint8_t m = mask[id];
-  u[l] = (fluid_row(m) || m == 3) ? up[id] : 0.0;
+__global__ void __launch_bounds__(HZ_PK) k_hz_unpack(const double *up, int nx, int ny, LevelGeom g, const uint8_t *mask,
+                                                     double *u) {
+  hz_rows(nx, ny, g, mask, [&](long long, long long id) { return make_double2(up[id], 0.0); },
+          [&](long long l, long long, bool, bool active, double2 x) { u[l] = active ? x.x : 0.0; });
 }
 
 // u += e on every slot (e is zero off the active rows)
@@ -470,7 +626,7 @@ double axis_max_sum(const std::vector<double> &f) {
 
 struct HzWork {
   double *u[2], *f, *ac64;   // ac: alpha x coefficients and sums
-  float *e[2], *r32, *ac32, *ac32lo;
+  float *e[2], *r32, *ac32, *ac32lo, *xq;
   double *part, *norms;
 };
 
@@ -494,13 +650,13 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
   Hierarchy *h = t->hier[0];
   Level &L0 = h->lv[0];
   const LevelGeom &G = L0.g;
-  const long long nslot = h->nslot, ncell = t->ncell, ng = t->nghost;
+  const long long nslot = h->nslot, ng = t->nghost;
   const int nx = G.nx, ny = G.ny, nz = G.nz, na = nx + ny + nz;
   // workspace: u (2), f in FP64; e (2), r in FP32; FP32 coefficients; partials; norms
   const long long want = nslot;
   const size_t na3 = ((3 * (size_t)na + 31) / 32) * 32;   // keeps the FP32 arrays 256-byte aligned
   const size_t bytes = sizeof(double) * (3 * (size_t)want + 2 * (size_t)HZ_BLOCKS * 2 + 8 + na3) +
-                       sizeof(float) * (3 * (size_t)want + 2 * na3 + 64);
+                       sizeof(float) * (3 * (size_t)want + 2 * na3 + 64 + HZ_XQ * (((size_t)nx + 3) / 4 * 4));
   if (!h->helm_buf || h->helm_n != want + na) {
     if (h->helm_buf) { IBM_TRY(cudaStreamSynchronize(st)); cudaFree(h->helm_buf); }
     h->helm_buf = nullptr;
@@ -520,11 +676,14 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
     float *fl = (float *)(W.ac64 + na3);
     W.e[0] = fl; W.e[1] = fl + want; W.r32 = fl + 2 * want; W.ac32 = fl + 3 * want;
     W.ac32lo = W.ac32 + na3;
+    W.xq = W.ac32lo + na3;
   }
   // views of the finest level: alpha x the hierarchy's FP64 coefficients, and FP32 copies
   long long launches = 0;
   k_scale_coefs<<<nb_of(3 * na, 256), 256, 0, st>>>(h->c64, 3 * na, alpha, W.ac64, W.ac32, W.ac32lo);
-  ++launches;
+  const int nx4 = (nx + 3) / 4 * 4;
+  k_hz_xq<<<nb_of(nx4, 256), 256, 0, st>>>(W.ac32, W.ac32lo, nx, na, nx4, W.xq);
+  launches += 2;
   HzView<double> v64;
   {
     const double *c = W.ac64;
@@ -546,16 +705,16 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
   // The packs write the cells only; halo and padding slots must read 0 in either view, so
   // the arrays are cleared whenever the layout changes.
   const bool df = o.precision == 2;
-  const dim3 cell_grid(nb_of(nx, 256), ny, nz);   // pack / unpack: one thread per cell of a row
+  const dim3 cell_grid(nb_of(nx, HZ_PK), nb_of(ny, HZ_PKR), nz);   // pack / unpack
   float *uh = (float *)W.u[0], *ul = uh + want, *fh = (float *)W.f, *fl = fh + want;
   if (h->helm_layout != (df ? 1 : 0)) {
     IBM_TRY(cudaMemsetAsync(W.u[0], 0, sizeof(double) * 3 * (size_t)want, st));   // u[0], u[1], f
     h->helm_layout = df ? 1 : 0;
   }
   if (df)
-    k_hz_pack_df<<<cell_grid, 256, 0, st>>>(f_user, u_user, ncell, nx, ny, G, L0.mask, fh, fl, uh, ul);
+    k_hz_pack_df<<<cell_grid, HZ_PK, 0, st>>>(f_user, u_user, nx, ny, G, L0.mask, fh, fl, uh, ul);
   else
-    k_hz_pack<<<cell_grid, 256, 0, st>>>(f_user, u_user, ncell, nx, ny, G, L0.mask, W.f, W.u[0]);
+    k_hz_pack<<<cell_grid, HZ_PK, 0, st>>>(f_user, u_user, nx, ny, G, L0.mask, W.f, W.u[0]);
   ++launches;
   if (ng > 0) {
     if (df) k_hz_ghost_rhs_df<<<nb_of(ng, 128), 128, 0, st>>>(h->gdst, ub, ng, fh, fl);
@@ -572,14 +731,28 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
   for (int k = 0; k < K; ++k) om[k] = 1.0 / (1.0 + rho * std::cos(3.141592653589793 * (2.0 * k + 1.0) / (2.0 * K)));
   const dim3 sweep_grid(nb_of(nx, TX), nb_of(ny, TY), nb_of(nz, KCH)), sweep_block(TX, TY);
   const int rest_blocks = (int)std::max<long long>(1, std::min<long long>(HZ_BLOCKS, nb_of((cuts ? h->cutcap : 0) + ng, HZ_THREADS)));
-  // the double-FP32 residual keeps 80 registers: three resident blocks per SM, one wave
-  const int df_blocks = std::max(1, std::min(HZ_BLOCKS, 3 * std::max(1, ctx->sm_count)));
+  // the FP32 sweep's grid; the double-FP32 residual's: one wave of two blocks per SM, and the planes per
+  // march that give the fewest plane steps
+  const long long strips = (long long)(nx4 / 4) * ny;
+  const dim3 sweep4_grid(nb_of(strips, SW_THREADS), nb_of(nz, SW_KZ));
+  const int df_max = std::max(1, std::min(HZ_BLOCKS, 2 * std::max(1, ctx->sm_count)));
+  int df_kz = 1;
+  {
+    const long long sblocks = nb_of(strips, HZ_THREADS);
+    long long best = -1;
+    for (int q = std::min(16, nz); q >= 1; --q) {
+      const long long cost = (sblocks * ((nz + q - 1) / q) + df_max - 1) / df_max * (q + 1);
+      if (best < 0 || cost < best) { best = cost; df_kz = q; }
+    }
+  }
+  const int df_blocks = (int)std::min<long long>(df_max, (long long)nb_of(strips, HZ_THREADS) * ((nz + df_kz - 1) / df_kz));
   // residual r = b - H u (FP64) with its norm, and the norm of b on the first call
   auto residual = [&](const double *u, float *r32, bool with_b) -> ibm_status {
     const long long *cnt = cuts ? h->d_cnt : nullptr;
     if (df) {
       const float *xh = (const float *)u, *xl = xh + want;
-      k_hz_resid_df<<<df_blocks, HZ_THREADS, 0, st>>>(v64, HzDf{W.ac32, W.ac32lo}, xh, xl, fh, fl, r32, W.part, with_b);
+      k_hz_resid_df<<<df_blocks, HZ_THREADS, 0, st>>>(v64, HzDf{W.ac32, W.ac32lo}, W.xq, xh, xl, fh, fl, r32, W.part,
+                                                      with_b, df_kz);
       k_hz_resid_rest<DfVals><<<rest_blocks, HZ_THREADS, 0, st>>>(
           v64, h->cut_id, h->cut_nb, h->cut_ijk, cnt, h->gsrc, h->gdst, t->gw, t->gwself, t->gscale, ng,
           DfVals{xh, xl, fh, fl}, alpha, r32, W.part + 2 * HZ_BLOCKS, with_b);
@@ -595,13 +768,20 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
     IBM_TRY(cudaStreamSynchronize(st));
     return IBM_OK;
   };
-  // one SRJ cycle of K relaxed Jacobi steps on (u, rhs); returns the index of the current buffer
-  auto srj_cycle = [&](auto *buf0, auto *buf1, const auto *rhs, auto view, int cur) -> int {
+  // one SRJ cycle of K relaxed Jacobi steps on (u, rhs); returns the index of the current buffer.
+  // zero: the field is zero, whatever its buffer holds (the first step does not read it)
+  auto srj_cycle = [&](auto *buf0, auto *buf1, const auto *rhs, auto view, int cur, bool zero) -> int {
     using T = std::remove_const_t<std::remove_pointer_t<decltype(buf0)>>;
     T *b[2] = {buf0, buf1};
     for (int k = 0; k < K; ++k) {
       T *u = b[cur], *un = b[1 - cur];
-      k_hz_sweep<T><<<sweep_grid, sweep_block, 0, st>>>(view, u, un, rhs, (T)om[k]);
+      const bool first = zero && k == 0;
+      if constexpr (sizeof(T) == 4) {
+        if (first) k_hz_sweep4<true><<<sweep4_grid, SW_THREADS, 0, st>>>(view, W.xq, u, un, rhs, (T)om[k]);
+        else k_hz_sweep4<false><<<sweep4_grid, SW_THREADS, 0, st>>>(view, W.xq, u, un, rhs, (T)om[k]);
+      } else {
+        k_hz_sweep<T><<<sweep_grid, sweep_block, 0, st>>>(view, u, un, rhs, (T)om[k]);
+      }
       ++launches;
       if (cuts) {
         k_hz_sweep_cut<T><<<cut_blocks, 256, 0, st>>>(view, h->cut_id, h->cut_nb, h->cut_ijk, h->d_cnt, u, un, rhs,
@@ -609,7 +789,8 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
         ++launches;
       }
       if (ng > 0) {
-        k_hz_ghost<T><<<nb_of(ng, 128), 128, 0, st>>>(h->gsrc, h->gdst, t->gw, t->gwself, ng, un, u, rhs);
+        k_hz_ghost<T><<<nb_of(ng, 128), 128, 0, st>>>(h->gsrc, h->gdst, t->gw, t->gwself, ng, un,
+                                                      first ? nullptr : (const T *)u, rhs);
         ++launches;
       }
       cur = 1 - cur;
@@ -624,8 +805,8 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
       if (o.precision == 0)
         k_hz_sweep<double><<<sweep_grid, sweep_block, 0, st>>>(v64, W.u[q & 1], W.u[1 - (q & 1)], W.f, om[0]);
       else
-        k_hz_sweep<float><<<sweep_grid, sweep_block, 0, st>>>(v32, W.e[q & 1], W.e[1 - (q & 1)], W.r32,
-                                                              (float)om[0]);
+        k_hz_sweep4<false><<<sweep4_grid, SW_THREADS, 0, st>>>(v32, W.xq, W.e[q & 1], W.e[1 - (q & 1)], W.r32,
+                                                               (float)om[0]);
       IBM_TRY(cudaEventRecord(ev[2 * q + 1], st));
     }
     IBM_TRY(cudaGetLastError());
@@ -659,11 +840,12 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
     while (rel > tol) {
       if (cycles >= o.max_cycles) { ret = IBM_ERR_NOT_CONVERGED; break; }
       if (o.precision == 0) {
-        cur = srj_cycle(W.u[0], W.u[1], (const double *)W.f, v64, cur);
+        cur = srj_cycle(W.u[0], W.u[1], (const double *)W.f, v64, cur, false);
         if ((s = residual(W.u[cur], nullptr, false)) != IBM_OK) return s;
       } else {
-        IBM_TRY(cudaMemsetAsync(W.e[0], 0, sizeof(float) * want, st));
-        const int ec = srj_cycle(W.e[0], W.e[1], (const float *)W.r32, v32, 0);
+        // the correction starts from zero; the membranes' cut cells read it, so there it is cleared
+        if (cuts) IBM_TRY(cudaMemsetAsync(W.e[0], 0, sizeof(float) * want, st));
+        const int ec = srj_cycle(W.e[0], W.e[1], (const float *)W.r32, v32, 0, !cuts);
         if (df) k_hz_update_df<<<ctx->wave, 256, 0, st>>>(uh, ul, W.e[ec], want);
         else k_hz_update<<<ctx->wave, 256, 0, st>>>(W.u[cur], W.e[ec], want);
         ++launches;
@@ -676,8 +858,8 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
       if (!std::isfinite(rel) || rn > 1e6 * std::max(r0, bnorm)) { ret = IBM_ERR_DIVERGED; break; }
     }
   }
-  if (df) k_hz_unpack_df<<<cell_grid, 256, 0, st>>>(uh, ul, ncell, nx, ny, G, L0.mask, u_user);
-  else k_hz_unpack<<<cell_grid, 256, 0, st>>>(W.u[cur], ncell, nx, ny, G, L0.mask, u_user);
+  if (df) k_hz_unpack_df<<<cell_grid, HZ_PK, 0, st>>>(uh, ul, nx, ny, G, L0.mask, u_user);
+  else k_hz_unpack<<<cell_grid, HZ_PK, 0, st>>>(W.u[cur], nx, ny, G, L0.mask, u_user);
   ++launches;
   IBM_TRY(cudaGetLastError());
   IBM_TRY(cudaStreamSynchronize(st));

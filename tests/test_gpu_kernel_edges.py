@@ -143,3 +143,30 @@ def test_noalloc_residual_at_march_edges(ctx, shape):
     # a residual cell carries about 10 roundings of sum |c| |p| and of the mean of b
     assert abs(sr - want) <= 1e-12 * want and abs(sb - base) <= 1e-12 * base and abs(rel - want / base) <= 2e-12 * rel
     T.close()
+
+
+@pytest.mark.parametrize("shape", [(33, 18, 21), (34, 19, 20), (35, 17, 18), (64, 16, 32), (130, 13, 15), (9, 24, 70)])
+def test_velocity_solve_at_odd_sizes(ctx, shape):
+    """The FP32 strip sweep (4 cells, 2 planes), the marched double-FP32 residual and the packs of 4 rows
+    against the oracle's direct solve; a second solve starts from correction arrays in use."""
+    from oracle import helmholtz as OH
+    pkg, c = ctx
+    n = max(shape)
+    f = [m / n * synth.faces_tanh(m, 1.5) for m in shape]
+    size = min(shape) / n
+    mesh = synth.ellipsoid(3, (0.33 * size, 0.26 * size, 0.29 * size), 25.0, [0.5 * m / n for m in shape])
+    g, T, _, ib, G = classify_both(pkg, c, *f, [mesh])
+    S = (np.max(g.cxm + g.cxp) + np.max(g.cym + g.cyp)) + np.max(g.czm + g.czp)
+    rhs = synth.smooth_field(*f, 3) + 0.1 * synth.counter_normal(6, 0, np.arange(ib.size)).reshape(ib.shape)
+    ub = synth.counter_normal(7, 0, np.arange(len(G)))
+    fd, ubd = torch.from_numpy(rhs).cuda(), torch.from_numpy(ub).cuda()
+    for aS in (0.7, 2.5):
+        u_o = OH.solve_closed(g, ib, G, aS / S, rhs, ub)
+        for prec in (0, 1, 2):
+            u = torch.zeros_like(fd)
+            rep = T.helmholtz_solve(aS / S, fd, u, ubd, 1e-11, pkg.HelmholtzOpts(precision=prec))
+            got = u.cpu().numpy()
+            err = np.linalg.norm((got - u_o)[ib != 1]) / np.linalg.norm(u_o[ib != 1])
+            assert rep["status"] == "IBM_OK" and err <= 1e-8, (aS, prec, err)
+            assert np.all(got[ib == 1] == 0.0)
+    T.close()
