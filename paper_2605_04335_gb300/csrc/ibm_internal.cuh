@@ -145,6 +145,7 @@ struct Hierarchy {
   long long *scan_buf = nullptr;            // compaction scratch: block counts and offsets
   long long scan_cap = 0;
   int tail_level = -1;                      // first level of the one-block coarse tail (-1: none)
+  int tail_smem = 0;                        // and its shared memory in bytes
   bool zmarch = false;
   int zm_per_sm = 1;                        // resident CTAs per SM of the fused sweep
   int zmc_per_sm = 1;                       // the same for its coarse-level form

@@ -925,27 +925,49 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 5)
 
 // ------------------------------------------------------------------ coarse tail
 
-// The V-cycle below the first level of at most TAIL_CELLS cells in one block of
-// TAIL_THREADS threads: the same smoothing, restriction (with the projection shift),
-// coarsest solve and prolongation as the per-level kernels, one pass after another with
-// block barriers instead of kernel launches.  Small levels are latency-bound, so the
-// launches and grid-wide ramps they save dominate.
-constexpr int TAIL_CELLS = 512;
+// The V-cycle below the first small level in one block: smoothing, restriction (with the projection
+// shift), coarsest solve and prolongation of the per-level kernels, with block barriers instead of
+// launches, and everything but the first level's right-hand side and correction in shared memory.
+// Latency-bound: a pass over a level is one dependent chain, so the coefficients (open fractions and
+// dead cells applied) are laid out once per call, and a barrier and a few shared loads remain per
+// colour.  Cells are kept by colour: a pass reads its own colour's coefficients and the other colour's
+// values without bank conflicts.  31 us per call from a 16^3 level on (two sweeps before and after); the same
+// levels took 22 us from 8^3 on in global memory and 11 launches of 2 to 4 us above
+constexpr int TAIL_CELLS = 512;       // up to here a level's correction is interpolated corner by corner
+// FP32 tails start at a level of up to 4096 cells: a launch costs more than such a level's pass in one
+// block (64^3 solves: 1291 us from 512 cells on, 1135 us from 4096).  FP64 stays at 512 cells: one SM's FP64 pipe takes 1.8 us per pass over 1300 cells
+template <typename T>
+constexpr int tail_cells() { return sizeof(T) == 4 ? 4096 : TAIL_CELLS; }
 constexpr int TAIL_THREADS = 1024;
 constexpr int TAIL_MAX_LEVELS = 8;
+constexpr int TAIL_SMEM = 220 * 1024;   // of 227 KB, which also hold the arguments and the reductions
+constexpr int TAIL_RHS = 7, TAIL_ARRAYS = 8;   // six coefficients, the diagonal, the right-hand side
 
+// A level in shared memory.  Pairs (2 p, 2 p + 1) along x hold one cell of each colour; pair
+// l = (k ny + j) hx + p; values by colour at pad + l.  There are no halos: a coefficient across the domain's
+// boundary is zero, and so is an interpolation weight, whatever value it multiplies.  The x-neighbours of a
+// cell are l - 1 + odd and l + odd of the other colour, odd = i & 1.  Rows without halos keep the
+// eight neighbours' loads free of bank conflicts.
 template <typename T>
 struct TailLevel {
   LV<T> v;
   T *e, *r;
   const int8_t *poff;    // prolongation tables of this level as the fine level (x, y, z)
   const float *pt;
+  const uint8_t *inner;  // of this level as the coarse level
+  int hx, np, plane, pad, ne;                 // pairs per row, in all and per plane; values per colour
+  int o_co, o_e, o_c, o_w, o_t, o_off, o_lv;   // byte offsets in shared memory
+  unsigned d_hx, d_ny, d_nx;                   // ceil(2^32 / divisor), 0 for 1 (tail_div)
+  int big;               // more than TAIL_CELLS cells
 };
 
 template <typename T>
 struct TailArgs {
   TailLevel<T> lv[TAIL_MAX_LEVELS];
   int nl;                 // levels in the tail (the last one is the coarsest)
+  int o_res;              // offset of a level's residuals, later of the coarsest inverse's copy
+  int minv_here;          // (0: the inverse is read where it is)
+  int bytes, threads;
   const double *shift0;   // projection shift of the tail's first level
   const double *fvol;     // fluid volume of each tail level
   const T *minv;
@@ -954,149 +976,439 @@ struct TailArgs {
   T omega;
 };
 
-// one colour of red-black relaxation of level v, all threads of the block
+// x / d for x d < 2^32 by its multiplier: three instructions, where a division by a kernel argument takes
+// about thirty and every pass decodes its cells
+__host__ __device__ __forceinline__ unsigned tail_magic(int d) {
+  return d > 1 ? (unsigned)((0xffffffffull + d) / d) : 0u;
+}
+__device__ __forceinline__ int tail_div(int x, unsigned m) { return m ? (int)__umulhi((unsigned)x, m) : x; }
+
+// shared-memory layout; returns its bytes
 template <typename T>
-__device__ void tail_relax(const LV<T> &v, T *e, const T *r, T sh, int colour, T omega) {
-  const int hx = (v.nx + 1) >> 1;
-  const int rows = v.ny * v.nz;
-  const int rstep = hx >= (int)blockDim.x ? 1 : (int)blockDim.x / hx;
-  const int r0 = hx >= (int)blockDim.x ? 0 : (int)threadIdx.x / hx;
-  const int t0 = hx >= (int)blockDim.x ? (int)threadIdx.x : (int)threadIdx.x - r0 * hx;
-  const int tstep = hx >= (int)blockDim.x ? (int)blockDim.x : hx;
-  if (r0 >= rstep) return;
-  for (int row = r0; row < rows; row += rstep) {
-    const int j = row % v.ny, k = row / v.ny;
-    for (int ti = t0; ti < hx; ti += tstep) {
-      const int i = 2 * ti + ((j + k + colour) & 1);
-      if (i >= v.nx) continue;
+int tail_layout(TailArgs<T> &A, const Level *lv, int nl) {
+  long long at = 0;
+  auto take = [&](long long n) {
+    const long long o = at;
+    at += (n + 15) / 16 * 16;
+    return (int)std::min<long long>(o, 1 << 30);
+  };
+  A.nl = nl;
+  long long cells0 = 0;
+  for (int q = 0; q < nl; ++q) {
+    TailLevel<T> &t = A.lv[q];
+    const LevelGeom &g = lv[q].g;
+    const long long n = (long long)g.nx + g.ny + g.nz, cells = (long long)g.nx * g.ny * g.nz;
+    if (cells > 4096) return 1 << 30;
+    if (q == 0) cells0 = cells;
+    t.hx = (g.nx + 1) / 2;
+    t.np = t.hx * g.ny * g.nz;
+    t.plane = t.hx * g.ny;
+    t.pad = (t.plane + t.hx + 2 + 31) / 32 * 32;
+    t.ne = t.np + 2 * t.pad;
+    t.big = cells > TAIL_CELLS;
+    t.d_hx = tail_magic(t.hx);
+    t.d_ny = tail_magic(g.ny);
+    t.d_nx = tail_magic(g.nx);
+    t.o_co = take((long long)TAIL_ARRAYS * 2 * t.np * sizeof(T));
+    t.o_e = take(2LL * t.ne * sizeof(T));
+    t.o_w = take(n * sizeof(T));
+    t.o_c = take(2 * n * sizeof(T));
+    t.o_t = take(n * 4);
+    t.o_off = take(n);
+    t.o_lv = take(2LL * t.ne);
+  }
+  const long long nc = (long long)lv[nl - 1].g.nx * lv[nl - 1].g.ny * lv[nl - 1].g.nz, minv = nc * (nc + 1) * sizeof(T);
+  const long long res = 2LL * A.lv[0].np * sizeof(T);
+  A.minv_here = minv <= res || at + minv <= TAIL_SMEM;
+  A.o_res = take(A.minv_here ? std::max(minv, res) : res);
+  A.bytes = (int)std::min<long long>(at, 1 << 30);
+  A.threads = (int)std::min<long long>(TAIL_THREADS, std::max<long long>(128, (cells0 / 2 + 31) / 32 * 32));
+  return A.bytes;
+}
+
+template <typename T>
+struct TailView {
+  int nx, ny, nz, hx, np, plane, pad, ne;
+  unsigned d_hx, d_ny, d_nx;
+  T *co, *e, *w, *c1;   // c1: cxm cxp cym cyp czm czp
+  float *t;
+  int8_t *off;
+  uint8_t *live;   // bit 0: a fluid cell; bit 1: its 26 neighbours too
+  __device__ __forceinline__ TailView(const TailLevel<T> &L, unsigned char *sm)
+      : nx(L.v.nx), ny(L.v.ny), nz(L.v.nz), hx(L.hx), np(L.np), plane(L.plane), pad(L.pad), ne(L.ne), d_hx(L.d_hx),
+        d_ny(L.d_ny), d_nx(L.d_nx), co(reinterpret_cast<T *>(sm + L.o_co)), e(reinterpret_cast<T *>(sm + L.o_e)),
+        w(reinterpret_cast<T *>(sm + L.o_w)), c1(reinterpret_cast<T *>(sm + L.o_c)),
+        t(reinterpret_cast<float *>(sm + L.o_t)), off(reinterpret_cast<int8_t *>(sm + L.o_off)), live(sm + L.o_lv) {}
+  // pair l -> its first cell; returns (j + k) & 1, the colour of that cell
+  __device__ __forceinline__ int pair(int l, int &i, int &j, int &k) const {
+    const int row = tail_div(l, d_hx);
+    k = tail_div(row, d_ny);
+    j = row - k * ny;
+    i = 2 * (l - row * hx);
+    return (j + k) & 1;
+  }
+  // colour-major position of a cell, or of one beside it
+  __device__ __forceinline__ int pos(int i, int j, int k) const {
+    return ((i + j + k) & 1) * ne + pad + k * plane + j * hx + (i >> 1);
+  }
+  // sum of c e over the six neighbours of the cell of colour c, pair l: stencil_sum's order
+  __device__ __forceinline__ T sum(int c, int l, int odd) const {
+    const T *cf = co + c * np + l, *en = e + (c ? 0 : ne) + pad + l;
+    const int n2 = 2 * np;
+    T s = mul_rn(cf[0], en[odd - 1]);
+    s = fma_t<T>(cf[n2], en[odd], s);
+    s = fma_t<T>(cf[2 * n2], en[-hx], s);
+    s = fma_t<T>(cf[3 * n2], en[hx], s);
+    s = fma_t<T>(cf[4 * n2], en[-plane], s);
+    return fma_t<T>(cf[5 * n2], en[plane], s);
+  }
+};
+
+template <typename T> struct TailPair;
+template <> struct TailPair<float> { using type = float2; };
+template <> struct TailPair<double> { using type = double2; };
+
+// a level's 1-D data into shared memory, its values and live flags cleared
+template <typename T>
+__device__ __forceinline__ void tail_clear(const TailLevel<T> &L, unsigned char *sm, bool last) {
+  const TailView<T> V(L, sm);
+  const LV<T> &v = L.v;
+  const int n = V.nx + V.ny + V.nz;
+  for (int q = threadIdx.x; q < n; q += blockDim.x) {
+    V.w[q] = q < V.nx ? v.wx[q] : q < V.nx + V.ny ? v.wy[q - V.nx] : v.wz[q - V.nx - V.ny];
+    V.c1[q] = v.cxm[q];           // the six rows are one array
+    V.c1[n + q] = v.cxm[n + q];
+    if (!last) {
+      V.t[q] = L.pt[q];
+      V.off[q] = L.poff[q];
+    }
+  }
+  const uint4 z = make_uint4(0u, 0u, 0u, 0u);   // both arrays end on 16 bytes
+  for (int q = threadIdx.x; q < (2 * L.ne * (int)sizeof(T) + 15) / 16; q += blockDim.x) reinterpret_cast<uint4 *>(V.e)[q] = z;
+  for (int q = threadIdx.x; q < (2 * L.ne + 15) / 16; q += blockDim.x) reinterpret_cast<uint4 *>(V.live)[q] = z;
+}
+
+// one level's live flags and, per cell, its coefficients and right-hand side (r - sh where r is given, else 0;
+// dead cells have zeros throughout), by thread t of the block
+template <typename T>
+__device__ __forceinline__ void tail_load(const TailLevel<T> &L, unsigned char *sm, const T *r, T sh, bool last, int t) {
+  const TailView<T> V(L, sm);
+  const LV<T> &v = L.v;
+  // a pair of cells in one load each, and two pairs before the arithmetic (the fractions of regular cells
+  // too); the cell past an odd level's end is a halo cell
+  constexpr int U = sizeof(T) == 4 ? 2 : 1;
+  using P = typename TailPair<T>::type;
+  auto ld2p = [](const T *p) { return *reinterpret_cast<const P *>(p); };
+  for (int l0 = t; l0 < V.np; l0 += U * blockDim.x) {
+    P R[U], X[U], Y0[U], Y1[U], Z0[U], Z1[U];
+    T xl[U];
+    uchar2 M[U], Q[U], I[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int l = l0 + u * blockDim.x;
+      if (l >= V.np) continue;
+      int i, j, k;
+      V.pair(l, i, j, k);
       const long long id = vidx(v, i, j, k);
-      if (v.mask[id] != 0) continue;
-      T c[6];
-      coefs(v, i, j, k, id, c);
-      const T D = v.sdx ? (v.sdx[i] + v.sdy[j]) + v.sdz[k] : ((c[0] + c[1]) + (c[2] + c[3])) + (c[4] + c[5]);
-      if (D == (T)0) continue;
-      const T res = stencil_sum(v, e, id, c) - D * e[id] - (r[id] - sh);
-      e[id] += (T)__fdividef((float)omega * (float)res, (float)D);
+      M[u] = *reinterpret_cast<const uchar2 *>(v.mask + id);
+      Q[u] = *reinterpret_cast<const uchar2 *>(v.zmask + id);
+      I[u] = *reinterpret_cast<const uchar2 *>(L.inner + id);
+      R[u].x = R[u].y = (T)0;
+      if (r) R[u] = ld2p(r + id);
+      xl[u] = v.fx[id - 1];
+      X[u] = ld2p(v.fx + id);
+      Y0[u] = ld2p(v.fy + id - v.sy);
+      Y1[u] = ld2p(v.fy + id);
+      Z0[u] = ld2p(v.fz + id - v.sz);
+      Z1[u] = ld2p(v.fz + id);
     }
-  }
-}
-
-// restriction of level f to level c (rc, ec = 0); returns sum V_c rc on thread 0
-template <typename T>
-__device__ double tail_restrict(const LV<T> &f, const T *e, const T *r, T sh, const LV<T> &cv, T *rc, T *ec) {
-  __shared__ double red[TAIL_THREADS / 32];
-  double acc_all = 0.0;
-  const int nc = cv.nx * cv.ny * cv.nz;
-  for (int l = threadIdx.x; l < nc; l += blockDim.x) {
-    const int I = l % cv.nx, q = l / cv.nx, J = q % cv.ny, K = q / cv.ny;
-    const long long ic = vidx(cv, I, J, K);
-    ec[ic] = (T)0;
-    if (cv.mask[ic] != 0) { rc[ic] = (T)0; continue; }
-    T acc = (T)0;
-    for (int c = 0; c < 8; ++c) {
-      const int i = 2 * I + (c & 1), j = 2 * J + ((c >> 1) & 1), k = 2 * K + ((c >> 2) & 1);
-      if (i >= f.nx || j >= f.ny || k >= f.nz) continue;
-      const long long id = vidx(f, i, j, k);
-      if (f.mask[id] != 0) continue;
-      T cf[6];
-      coefs(f, i, j, k, id, cf);
-      const T D = f.sdx ? (f.sdx[i] + f.sdy[j]) + f.sdz[k] : ((cf[0] + cf[1]) + (cf[2] + cf[3])) + (cf[4] + cf[5]);
-      const T res = (r[id] - sh) - (stencil_sum(f, e, id, cf) - D * e[id]);
-      acc += (f.wx[i] * f.wy[j]) * f.wz[k] * res;
-    }
-    rc[ic] = acc / ((cv.wx[I] * cv.wy[J]) * cv.wz[K]);
-    acc_all += (double)acc;
-  }
-  for (int o = 16; o > 0; o >>= 1) acc_all += __shfl_down_sync(0xffffffffu, acc_all, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc_all;
-  __syncthreads();
-  double sum = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
-  __syncthreads();
-  return sum;
-}
-
-// prolongation e_f += P e_c on the fluid cells of level f (per fine cell)
-template <typename T>
-__device__ void tail_prolong(const LV<T> &cv, const T *ec, const LV<T> &f, T *ef, const int8_t *poff,
-                             const float *pt) {
-  const int nf = f.nx * f.ny * f.nz;
-  const int8_t *offx = poff, *offy = poff + f.nx, *offz = poff + f.nx + f.ny;
-  const float *tx = pt, *ty = pt + f.nx, *tz = pt + f.nx + f.ny;
-  for (int l = threadIdx.x; l < nf; l += blockDim.x) {
-    const int i = l % f.nx, q = l / f.nx, j = q % f.ny, k = q / f.ny;
-    const long long id = vidx(f, i, j, k);
-    if (f.mask[id] != 0) continue;
-    const int I = i >> 1, J = j >> 1, K = k >> 1;
-    const float wx[2] = {1.0f - tx[i], tx[i]}, wy[2] = {1.0f - ty[j], ty[j]}, wz[2] = {1.0f - tz[k], tz[k]};
-    const int ox = offx[i], oy = offy[j], oz = offz[k];
-    T s = (T)0;
-    float ws = 0.0f;
-    for (int c = 0; c < 8; ++c) {
-      const int a = c & 1, b = (c >> 1) & 1, d = (c >> 2) & 1;
-      const float w = (wx[a] * wy[b]) * wz[d];
-      if (w == 0.0f) continue;
-      const long long ic = vidx(cv, I + a * ox, J + b * oy, K + d * oz);
-      if (cv.mask[ic] != 0) continue;
-      s += (T)w * ec[ic];
-      ws += w;
-    }
-    if (ws > 0.0f) ef[id] += s * (T)(1.0f / ws);
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void tail_body(const TailArgs<T> &A) {
-  __shared__ double shift_s[TAIL_MAX_LEVELS];
-  __shared__ T rs[MAX_COARSE + 1];
-  if (threadIdx.x == 0) shift_s[0] = *A.shift0;
-  __syncthreads();
-  const int last = A.nl - 1;
-  // down: pre-smooth, restrict
-  for (int l = 0; l < last; ++l) {
-    const TailLevel<T> &F = A.lv[l];
-    const T sh = (T)shift_s[l];
-    for (int s = 0; s < A.nu1; ++s)
-      for (int colour = 0; colour < 2; ++colour) {
-        tail_relax(F.v, F.e, F.r, sh, colour, A.omega);
-        __syncthreads();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int l = l0 + u * blockDim.x;
+      if (l >= V.np) continue;
+      int i0, j, k;
+      const int par = V.pair(l, i0, j, k);
+      const T *cy = V.c1 + 2 * V.nx, *cz = cy + 2 * V.ny;
+      const T cym = cy[j], cyp = cy[V.ny + j], czm = cz[k], czp = cz[V.nz + k];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = i0 + h, c = par ^ h, q = c * V.np + l;
+        const bool live = i < V.nx && (h ? M[u].y : M[u].x) == 0;
+        if (live) V.live[c * V.ne + V.pad + l] = (uint8_t)(1 + 2 * ((h ? I[u].y : I[u].x) != 0));
+        T cf[TAIL_ARRAYS];
+#pragma unroll
+        for (int a = 0; a < TAIL_ARRAYS; ++a) cf[a] = (T)0;
+        if (live && !last) {
+          if (r) cf[TAIL_RHS] = (h ? R[u].y : R[u].x) - sh;
+          cf[0] = V.c1[i]; cf[1] = V.c1[V.nx + i]; cf[2] = cym; cf[3] = cyp; cf[4] = czm; cf[5] = czp;
+          if ((h ? Q[u].y : Q[u].x) == zm::IRREGULAR) {
+            cf[0] = mul_rn(cf[0], h ? X[u].x : xl[u]); cf[1] = mul_rn(cf[1], h ? X[u].y : X[u].x);
+            cf[2] = mul_rn(cf[2], h ? Y0[u].y : Y0[u].x); cf[3] = mul_rn(cf[3], h ? Y1[u].y : Y1[u].x);
+            cf[4] = mul_rn(cf[4], h ? Z0[u].y : Z0[u].x); cf[5] = mul_rn(cf[5], h ? Z1[u].y : Z1[u].x);
+          }
+          cf[6] = ((cf[0] + cf[1]) + (cf[2] + cf[3])) + (cf[4] + cf[5]);
+        }
+        if (last) {
+          V.co[2 * TAIL_RHS * V.np + q] = (T)0;
+        } else {
+#pragma unroll
+          for (int a = 0; a < TAIL_ARRAYS; ++a) V.co[2 * a * V.np + q] = cf[a];
+        }
       }
-    const TailLevel<T> &C = A.lv[l + 1];
-    const double sum = tail_restrict(F.v, F.e, F.r, sh, C.v, C.r, C.e);
-    if (threadIdx.x == 0) shift_s[l + 1] = A.fvol[l + 1] > 0 ? sum / A.fvol[l + 1] : 0.0;
+    }
+  }
+}
+
+// nu red-black sweeps, all threads of the block
+template <typename T>
+__device__ __forceinline__ void tail_relax(const TailView<T> &V, int nu, float omega) {
+  const int n2 = 2 * V.np;
+  int odd[2];   // of the thread's first two pairs: the colour of their first cell
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    int i, j, k;
+    odd[u] = V.pair(threadIdx.x + u * blockDim.x, i, j, k);
+  }
+  for (int s = 0; s < 2 * nu; ++s) {
+    const int c = s & 1;
+    T *e = V.e + (c ? V.ne : 0) + V.pad;
+    const T *cf = V.co + c * V.np;
+    for (int l0 = threadIdx.x; l0 < V.np; l0 += 2 * blockDim.x) {   // two cells of the colour in flight
+      T D[2], ce[2], res[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int l = l0 + u * blockDim.x;
+        D[u] = (T)0;
+        if (l >= V.np) continue;
+        int par = odd[u];
+        if (l0 != threadIdx.x) {
+          int i, j, k;
+          par = V.pair(l, i, j, k);
+        }
+        D[u] = cf[6 * n2 + l];
+        ce[u] = e[l];
+        res[u] = fma_t<T>(-D[u], ce[u], V.sum(c, l, par ^ c)) - cf[TAIL_RHS * n2 + l];
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)   // a cell with no open face keeps its value
+        if (D[u] > (T)0) e[l0 + u * blockDim.x] = ce[u] + (T)__fdividef(omega * (float)res[u], (float)D[u]);
+    }
     __syncthreads();
+  }
+}
+
+// restriction of level f: the residual's sums into the right-hand side of c, less its projection
+// shift.  Residuals by colour first (eight children gathered at once put four lanes on a bank: 22000
+// of a tail's 85000 cycles at 16^3), then one thread per coarse cell sums its children in order.
+template <typename T>
+__device__ __forceinline__ void tail_restrict(const TailView<T> &f, const TailView<T> &c, double fvol, bool last, T *res,
+                                              double *red) {
+  const int nc = c.nx * c.ny * c.nz, n2 = 2 * f.np, lane = threadIdx.x & 31;
+  for (int l = threadIdx.x; l < f.np; l += blockDim.x) {
+    int i, j, k;
+    const int par = f.pair(l, i, j, k);
+    T s[2];
+#pragma unroll
+    for (int col = 0; col < 2; ++col) {
+      const T *cf = f.co + col * f.np + l;
+      s[col] = cf[TAIL_RHS * n2] - fma_t<T>(-cf[6 * n2], f.e[(col ? f.ne : 0) + f.pad + l], f.sum(col, l, par ^ col));
+    }
+    res[l] = s[0];
+    res[f.np + l] = s[1];
+  }
+  __syncthreads();
+  double all = 0.0;
+  for (int cell = threadIdx.x; cell < nc; cell += blockDim.x) {
+    const int q = tail_div(cell, c.d_nx), K = tail_div(q, c.d_ny), J = q - K * c.ny, I = cell - q * c.nx;
+    const int cc = (I + J + K) & 1;
+    const int cl = K * c.plane + J * c.hx + (I >> 1);
+    if (!(c.live[cc * c.ne + c.pad + cl] & 1)) continue;
+    T acc = (T)0;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int i = 2 * I + (a & 1), j = 2 * J + ((a >> 1) & 1), k = 2 * K + (a >> 2);
+      if (i >= f.nx || j >= f.ny || k >= f.nz) continue;
+      acc = fma_t<T>((f.w[i] * f.w[f.nx + j]) * f.w[f.nx + f.ny + k], res[((i + j + k) & 1) * f.np + (k * f.ny + j) * f.hx + I],
+                     acc);
+    }
+    c.co[(2 * TAIL_RHS + cc) * c.np + cl] = acc / ((c.w[I] * c.w[c.nx + J]) * c.w[c.nx + c.ny + K]);
+    if constexpr (sizeof(T) == 4) all += dfl::widen(acc);
+    else all += acc;
+  }
+  if (last) {   // the bordered solve takes r itself
+    __syncthreads();
+    return;
+  }
+  // FP64 operations only in the warps that have something to add: 20 cycles of the SM's pipe each
+  const int first = (int)threadIdx.x & ~31;
+  if (first < nc)
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+  if (lane == 0) red[threadIdx.x >> 5] = all;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double t = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    __syncwarp();
+    if (lane == 0) red[0] = fvol > 0 ? t / fvol : 0.0;
+  }
+  __syncthreads();
+  const T sh = (T)red[0];
+  for (int q = threadIdx.x; q < 2 * c.np; q += blockDim.x) {
+    const int col = q >= c.np;
+    if (c.live[c.pad + q + col * (c.ne - c.np)] & 1) c.co[2 * TAIL_RHS * c.np + q] -= sh;
+  }
+  __syncthreads();
+}
+
+// prolongation e_f += P e_c on the fluid cells of level f, corner by corner (big levels: a pair of cells per
+// thread, contracted axis by axis, as the per-level kernel does)
+template <typename T>
+__device__ __forceinline__ void tail_prolong(const TailView<T> &c, const TailView<T> &f, bool big) {
+  if (!big) {
+    for (int q = threadIdx.x; q < 2 * f.np; q += blockDim.x) {
+      const int col = q >= f.np, l = q - col * f.np, b = col * f.ne + f.pad + l;
+      int i, j, k;
+      const int par = f.pair(l, i, j, k);
+      i += par ^ col;
+      if (i >= f.nx || !(f.live[b] & 1)) continue;
+      const int I = i >> 1, J = j >> 1, K = k >> 1;
+      const float tx = f.t[i], ty = f.t[f.nx + j], tz = f.t[f.nx + f.ny + k];
+      const int ox = f.off[i], oy = f.off[f.nx + j], oz = f.off[f.nx + f.ny + k];
+      const float wx[2] = {1.0f - tx, tx}, wy[2] = {1.0f - ty, ty}, wz[2] = {1.0f - tz, tz};
+      T s = (T)0;
+      float ws = 0.0f;
+#pragma unroll
+      for (int a8 = 0; a8 < 8; ++a8) {
+        const int a = a8 & 1, bb = (a8 >> 1) & 1, d = (a8 >> 2) & 1;
+        const float w = (wx[a] * wy[bb]) * wz[d];
+        const int ic = c.pos(I + a * ox, J + bb * oy, K + d * oz);
+        if (w == 0.0f || !(c.live[ic] & 1)) continue;
+        s += (T)w * c.e[ic];
+        ws += w;
+      }
+      if (ws > 0.0f) f.e[b] += s * (T)(1.0f / ws);
+    }
+  } else {
+    // along an axis the first child weighs the lower neighbour and the parent, the second the
+    // parent and the upper neighbour, in this order
+    auto axis = [](int odd, int o, float t, T (&w)[2]) {
+      w[0] = odd ? (T)(1.f - t) : (T)(o < 0 ? t : 0.f);
+      w[1] = odd ? (T)(o > 0 ? t : 0.f) : (T)(1.f - t);
+    };
+    for (int l = threadIdx.x; l < f.np; l += blockDim.x) {
+      int i, j, k;
+      const int par = f.pair(l, i, j, k), b0 = par * f.ne + f.pad + l, b1 = (1 - par) * f.ne + f.pad + l;
+      const int I = i >> 1, J = j >> 1, K = k >> 1, i1 = min(2 * I + 1, f.nx - 1);
+      const bool u0 = f.live[b0] & 1, u1 = 2 * I + 1 < f.nx && (f.live[b1] & 1);
+      if (!u0 && !u1) continue;
+      T wx0[2], wx1[2], wy[2], wz[2];
+      axis(0, f.off[2 * I], f.t[2 * I], wx0);
+      axis(1, f.off[i1], f.t[i1], wx1);
+      axis(j & 1, f.off[f.nx + j], f.t[f.nx + j], wy);
+      axis(k & 1, f.off[f.nx + f.ny + k], f.t[f.nx + f.ny + k], wz);
+      const int Jl = J - 1 + (j & 1), Kl = K - 1 + (k & 1);
+      // coarse cells (I - 1, I, I + 1) of a row: I in one colour, its neighbours in the other
+      auto contract = [&](auto val, T &o0, T &o1) {
+        T n0[2], n1[2];
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+          T r0[2], r1[2];
+#pragma unroll
+          for (int y = 0; y < 2; ++y) {
+            const int Jr = Jl + y, Kr = Kl + d, rowp = c.pad + Kr * c.plane + Jr * c.hx;
+            const int ci = (I + Jr + Kr) & 1, mine = ci * c.ne + rowp + (I >> 1);
+            const int left = (1 - ci) * c.ne + rowp + ((I - 1) >> 1);
+            const T v0 = val(left), v1 = val(mine), v2 = val(left + 1);
+            r0[y] = fma_t<T>(wx0[1], v1, wx0[0] * v0);
+            r1[y] = fma_t<T>(wx1[1], v2, wx1[0] * v1);
+          }
+          n0[d] = fma_t<T>(wy[1], r0[1], wy[0] * r0[0]);
+          n1[d] = fma_t<T>(wy[1], r1[1], wy[0] * r1[0]);
+        }
+        o0 = fma_t<T>(wz[1], n0[1], wz[0] * n0[0]);
+        o1 = fma_t<T>(wz[1], n1[1], wz[0] * n1[0]);
+      };
+      T a0, a1;
+      contract([&](int q) { return c.e[q]; }, a0, a1);
+      if (!(c.live[c.pos(I, J, K)] & 2)) {   // not a fully fluid block: by the sum of the fluid corners' weights
+        T d0, d1;
+        contract([&](int q) { return (c.live[q] & 1) ? (T)1 : (T)0; }, d0, d1);
+        a0 = d0 > (T)0 ? a0 / d0 : (T)0;
+        a1 = d1 > (T)0 ? a1 / d1 : (T)0;
+      }
+      if (u0) f.e[b0] += a0;
+      if (u1) f.e[b1] += a1;
+    }
+  }
+  __syncthreads();
+}
+
+template <typename T>
+__device__ __forceinline__ void tail_body(const TailArgs<T> &A, unsigned char *sm) {
+  __shared__ T rs[MAX_COARSE + 1];
+  __shared__ int2 map[MAX_COARSE + 1];   // coarsest unknowns: right-hand side slot, position
+  __shared__ double red[TAIL_THREADS / 32];
+  const int last = A.nl - 1, n = *A.ncoarse, m = n + 1;
+  for (int l = 0; l <= last; ++l) tail_clear(A.lv[l], sm, l == last);
+  __syncthreads();
+  // the levels' loads overlap: the second level's by the first warps, the third's by the last ones
+  for (int l = 0; l <= last; ++l)
+    tail_load(A.lv[l], sm, l == 0 ? (const T *)A.lv[0].r : nullptr, l == 0 ? (T)*A.shift0 : (T)0, l == last,
+              l & 1 ? (int)threadIdx.x : (int)(blockDim.x - 1 - threadIdx.x));
+  const TailView<T> Lc(A.lv[last], sm);
+  T *const res = reinterpret_cast<T *>(sm + A.o_res);
+  {
+    const LV<T> &v = A.lv[last].v;
+    const long long base = vidx(v, 0, 0, 0);
+    for (int q = threadIdx.x; q < n; q += blockDim.x) {
+      const long long d = A.cidx[q] - base;
+      const int k = (int)(d / v.sz), j = (int)((d - k * v.sz) / v.sy), i = (int)(d - k * v.sz - j * v.sy);
+      map[q] = make_int2((2 * TAIL_RHS + ((i + j + k) & 1)) * Lc.np + (k * v.ny + j) * Lc.hx + (i >> 1), Lc.pos(i, j, k));
+    }
+  }
+  __syncthreads();
+  const float om = (float)A.omega;
+  for (int l = 0; l < last; ++l) {
+    const TailView<T> F(A.lv[l], sm), C(A.lv[l + 1], sm);
+    tail_relax(F, A.nu1, om);
+    tail_restrict(F, C, A.fvol[l + 1], l + 1 == last, res, red);
   }
   // coarsest: e = Minv r (the bordered row's right-hand side is 0)
-  {
-    const TailLevel<T> &Lc = A.lv[last];
-    const int n = *A.ncoarse, m = n + 1;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) rs[q] = Lc.r[A.cidx[q]];
-    __syncthreads();
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-      T acc = (T)0;
+  for (int q = threadIdx.x; q < n; q += blockDim.x) rs[q] = Lc.co[map[q].x];
+  if (A.minv_here)
+    for (int q = threadIdx.x; q < n * m; q += blockDim.x) res[q] = A.minv[q];
+  __syncthreads();
+  for (int q = threadIdx.x; q < n; q += blockDim.x) {
+    T acc = (T)0;
+    if (A.minv_here)
+      for (int c = 0; c < n; ++c) acc += res[q * m + c] * rs[c];
+    else
       for (int c = 0; c < n; ++c) acc += A.minv[q * m + c] * rs[c];
-      Lc.e[A.cidx[q]] = acc;
-    }
-    __syncthreads();
+    Lc.e[map[q].y] = acc;
   }
-  // up: prolong, post-smooth
+  __syncthreads();
   for (int l = last - 1; l >= 0; --l) {
-    const TailLevel<T> &F = A.lv[l], &C = A.lv[l + 1];
-    tail_prolong(C.v, C.e, F.v, F.e, F.poff, F.pt);
-    __syncthreads();
-    const T sh = (T)shift_s[l];
-    for (int s = 0; s < A.nu2; ++s)
-      for (int colour = 0; colour < 2; ++colour) {
-        tail_relax(F.v, F.e, F.r, sh, colour, A.omega);
-        __syncthreads();
-      }
+    const TailView<T> F(A.lv[l], sm), C(A.lv[l + 1], sm);
+    tail_prolong(C, F, A.lv[l].big != 0);
+    tail_relax(F, A.nu2, om);
+  }
+  // dead cells and the one past an odd level's end are zero there already
+  const TailLevel<T> &L = A.lv[0];
+  const TailView<T> V(L, sm);
+  for (int l = threadIdx.x; l < V.np; l += blockDim.x) {
+    int i, j, k;
+    const int par = V.pair(l, i, j, k);
+    typename TailPair<T>::type x;
+    x.x = V.e[par * V.ne + V.pad + l];
+    x.y = V.e[(1 - par) * V.ne + V.pad + l];
+    *reinterpret_cast<typename TailPair<T>::type *>(L.e + vidx(L.v, i, j, k)) = x;
   }
 }
 
+extern __shared__ __align__(16) unsigned char tail_smem[];
 template <typename T>
 __global__ void __launch_bounds__(TAIL_THREADS) k_tail(const __grid_constant__ TailArgs<T> A) {
-  tail_body(A);
+  tail_body(A, tail_smem);
 }
 
 // bordered coarsest solve: [e; lambda] = Minv [r; 0]
@@ -2773,7 +3085,17 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
   h->tail_level = -1;
   for (int l = 1; l < nl; ++l) {
     const Level &L = h->lv[l];
-    if ((long long)L.g.nx * L.g.ny * L.g.nz <= TAIL_CELLS && nl - l <= TAIL_MAX_LEVELS) { h->tail_level = l; break; }
+    TailArgs<T> A;
+    if ((long long)L.g.nx * L.g.ny * L.g.nz <= tail_cells<T>() && nl - l <= TAIL_MAX_LEVELS &&
+        tail_layout(A, &h->lv[l], nl - l) <= TAIL_SMEM) {
+      h->tail_level = l;
+      h->tail_smem = A.bytes;
+      break;
+    }
+  }
+  if (cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_SMEM) != cudaSuccess) {
+    cudaGetLastError();
+    h->tail_level = -1;
   }
   // one wave of the row-strided restriction
   {
@@ -3137,6 +3459,29 @@ int prolong_grid(const ibm_ctx *ctx, const LevelGeom &C, int problems, int &gx, 
   return (int)std::max(1LL, std::min<long long>(PROLONG_KC, (long long)gx * gy * C.nz * problems / (PROLONG_BPS * sms)));
 }
 
+// the arguments of the tail from level l on (e of level l was zeroed by the restriction into it)
+template <typename T>
+void tail_fill(TailArgs<T> &A, Hierarchy *h, int l, const double *shift, const int *ncoarse, int nu1, int nu2, T omega) {
+  tail_layout(A, &h->lv[l], (int)h->lv.size() - l);
+  for (int q = 0; q < A.nl; ++q) {
+    Level &L = h->lv[l + q];
+    A.lv[q].v = view<T>(L);
+    A.lv[q].e = (T *)L.e;
+    A.lv[q].r = (T *)L.r;
+    A.lv[q].poff = L.poff;
+    A.lv[q].pt = L.pt;
+    A.lv[q].inner = L.inner;
+  }
+  A.shift0 = shift;
+  A.fvol = h->d_fvol + l;
+  A.minv = (const T *)h->minv;
+  A.cidx = h->cidx;
+  A.ncoarse = ncoarse;
+  A.nu1 = nu1;
+  A.nu2 = nu2;
+  A.omega = omega;
+}
+
 // V-cycle for level l: e_l (in/out) approximately solves A_l e_l = r_l - shift_l.  On the
 // finest level e is the hierarchy's own pointer: the fused sweep swaps it between two buffers.
 template <typename T>
@@ -3146,24 +3491,8 @@ void vcycle(Solver &S, int l, T *&e, const T *r, const double *shift, const T *g
   if (l > 0 && l == h->tail_level && nl - l >= 2) {
     // levels l .. nl-1 in one block (e of level l was zeroed by the restriction into it)
     TailArgs<T> A;
-    A.nl = nl - l;
-    for (int q = 0; q < A.nl; ++q) {
-      Level &L = h->lv[l + q];
-      A.lv[q].v = view<T>(L);
-      A.lv[q].e = (T *)L.e;
-      A.lv[q].r = (T *)L.r;
-      A.lv[q].poff = L.poff;
-      A.lv[q].pt = L.pt;
-    }
-    A.shift0 = shift;
-    A.fvol = h->d_fvol + l;
-    A.minv = (const T *)h->minv;
-    A.cidx = h->cidx;
-    A.ncoarse = S.d_ncoarse;
-    A.nu1 = S.nu1;
-    A.nu2 = S.nu2;
-    A.omega = (T)S.omega;
-    k_tail<T><<<1, TAIL_THREADS, 0, S.st>>>(A);
+    tail_fill(A, h, l, shift, S.d_ncoarse, S.nu1, S.nu2, (T)S.omega);
+    k_tail<T><<<1, A.threads, A.bytes, S.st>>>(A);
     S.ctx->launches += 1;
     return;
   }
@@ -3893,7 +4222,7 @@ __global__ void __launch_bounds__(TAIL_THREADS) kb_tail(const TailArgs<float> *A
   unsigned long long *dst = reinterpret_cast<unsigned long long *>(&As);
   for (int w = threadIdx.x; w < (int)(sizeof(TailArgs<float>) / 8); w += blockDim.x) dst[w] = src[w];
   __syncthreads();
-  tail_body<float>(As);
+  tail_body<float>(As, tail_smem);
 }
 // the outer step: p += e, the fine residual with its ghost rows and norms (lambda updated)
 struct PUpdate {
@@ -4214,9 +4543,11 @@ void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
     else mid.push_back(i);
   }
   if (!tail.empty()) {
+    int tail_bytes = 0;
+    for (int i : tail) tail_bytes = std::max(tail_bytes, lk_h(K, i)->tail_smem);
     bl_launch<int>(tail, [](int) { return 1; }, [](int i) { return i; },
                    [&](const BL<int> &L, int b) {
-                     kb_tail<<<b, TAIL_THREADS, 0, K.st>>>((const TailArgs<float> *)K.ctx->lk_tail, L);
+                     kb_tail<<<b, TAIL_THREADS, tail_bytes, K.st>>>((const TailArgs<float> *)K.ctx->lk_tail, L);
                      K.ctx->launches += 1;
                    });
   }
@@ -4522,6 +4853,7 @@ bool lockstep_ok(const std::vector<Run> &R, const ibm_solve_opts *opts) {
 ibm_status lockstep_setup(Lock &K, std::vector<Run> &R) {
   ibm_ctx *ctx = K.ctx;
   const int n = (int)R.size();
+  IBM_TRY(cudaFuncSetAttribute(kb_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_SMEM));
   if (!ctx->lk_count) IBM_TRY(cudaMalloc((void **)&ctx->lk_count, sizeof(int) * LK_COUNTERS));
   if (ctx->lk_tail_cap < n) {
     if (ctx->lk_tail) cudaFree(ctx->lk_tail);
@@ -4538,25 +4870,8 @@ ibm_status lockstep_setup(Lock &K, std::vector<Run> &R) {
     const int nl = (int)h->lv.size(), l = h->tail_level;
     TailArgs<float> &A = ta[i];
     A = TailArgs<float>{};
-    if (l > 0 && nl - l >= 2) {
-      A.nl = nl - l;
-      for (int q = 0; q < A.nl; ++q) {
-        Level &L = h->lv[l + q];
-        A.lv[q].v = view<float>(L);
-        A.lv[q].e = (float *)L.e;
-        A.lv[q].r = (float *)L.r;
-        A.lv[q].poff = L.poff;
-        A.lv[q].pt = L.pt;
-      }
-      A.shift0 = R[i].S.scal + S_LEVEL_SHIFT + l;
-      A.fvol = h->d_fvol + l;
-      A.minv = (const float *)h->minv;
-      A.cidx = h->cidx;
-      A.ncoarse = h->dncoarse;
-      A.nu1 = K.nu1;
-      A.nu2 = K.nu2;
-      A.omega = K.omega;
-    }
+    if (l > 0 && nl - l >= 2)
+      tail_fill(A, h, l, R[i].S.scal + S_LEVEL_SHIFT + l, h->dncoarse, K.nu1, K.nu2, K.omega);
   }
   IBM_TRY(cudaMemcpyAsync(ctx->lk_tail, ta.data(), sizeof(TailArgs<float>) * n, cudaMemcpyHostToDevice, K.st));
   K.E.assign(nl_max, std::vector<float *>(n, nullptr));

@@ -170,3 +170,25 @@ def test_velocity_solve_at_odd_sizes(ctx, shape):
             assert rep["status"] == "IBM_OK" and err <= 1e-8, (aS, prec, err)
             assert np.all(got[ib == 1] == 0.0)
     T.close()
+
+
+@pytest.mark.parametrize("shape", [(32, 32, 32), (33, 32, 31), (34, 32, 32), (16, 16, 16), (130, 40, 9), (12, 9, 150), (20, 24, 17)])
+def test_coarse_tail_edges(ctx, shape):
+    """The one-block coarse tail at its largest level (16^3 cells), just past it, at the corner-by-corner
+    limit (8^3) and on long levels: every precision against the oracle's direct solve."""
+    from oracle import solve as OS
+    pkg, c = ctx
+    n = max(shape)
+    f = [m / n * synth.faces_tanh(m, 1.4) for m in shape]
+    size = min(shape) / n
+    mesh = synth.ellipsoid(3, (0.31 * size, 0.27 * size, 0.24 * size), 25.0, [0.5 * m / n for m in shape])
+    g, T, _, ib, G = classify_both(pkg, c, *f, [mesh])
+    b = synth.rhs_divergence(*f, 3)
+    p_o, _ = OS.solve_sparse(g, ib, G, b)
+    fl = ib == 0
+    for prec in (0, 1, 2):
+        p = torch.zeros(b.shape, dtype=torch.float64, device="cuda")
+        T.solve(torch.from_numpy(b).cuda(), p, 1e-11, pkg.SolveOpts(precision=prec))
+        err = np.linalg.norm((p.cpu().numpy() - p_o)[fl]) / np.linalg.norm(p_o[fl])
+        assert err < 1e-8, (prec, err)
+    T.close()
