@@ -552,7 +552,8 @@ __global__ void k_ghost_eval(const long long *src, const long long *dst, const W
 
 // ghost rows right after a ping-pong sweep, in one launch: fluid sources from the new
 // array, ghost sources from the previous one (whose ghost values the sweep copied
-// unchanged), so no thread reads a value another thread writes (Jacobi among ghosts)
+// unchanged), so no thread reads a value another thread writes (Jacobi among ghosts); eold null:
+// the previous values are zero
 template <typename T, typename W, class G>
 __device__ __forceinline__ void ghost_pp_body(const long long *src, const long long *dst, const W *w, long long ng,
                                               const long long *ngp, T *enew, const T *eold, const T *rhs,
@@ -563,7 +564,7 @@ __device__ __forceinline__ void ghost_pp_body(const long long *src, const long l
   const long long d = dst[g];
   if (ngp && g >= *ngp) return;
   const T b = rhs ? rhs[d] : (T)0;
-  T s = row.template sum<T>([&](long long q) { return (q & GHOST_CORNER) ? eold[q & ~GHOST_CORNER] : enew[q]; });
+  T s = row.template sum<T>([&](long long q) { return (q & GHOST_CORNER) ? (eold ? eold[q & ~GHOST_CORNER] : (T)0) : enew[q]; });
   if (rhs) s += b;
   if (gd) s += (T)gd[g];     // the row's Neumann datum
   enew[d] = s;
@@ -935,7 +936,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 5)
 // levels took 22 us from 8^3 on in global memory and 11 launches of 2 to 4 us above
 constexpr int TAIL_CELLS = 512;       // up to here a level's correction is interpolated corner by corner
 // FP32 tails start at a level of up to 4096 cells: a launch costs more than such a level's pass in one
-// block (64^3 solves: 1291 us from 512 cells on, 1135 us from 4096).  FP64 stays at 512 cells: one SM's FP64 pipe takes 1.8 us per pass over 1300 cells
+// block (64^3 solves: 1291 us from 512 cells on, 1135 us from 4096).  FP64 stays at 512 cells: one SM's
+// FP64 pipe takes 1.8 us per pass over 1300 cells
 template <typename T>
 constexpr int tail_cells() { return sizeof(T) == 4 ? 4096 : TAIL_CELLS; }
 constexpr int TAIL_THREADS = 1024;
@@ -3300,11 +3302,21 @@ void ghost_update(Solver &S, T *e, const T *ghost_rhs) {
   S.ctx->launches += 2;
 }
 
+// plane offset that puts every plane a sweep loads past the last one
+inline int sweep_zero_plane(int nz) { return 2 * nz + 64; }
+
+// The first sweep of a correction cycle starts from e = 0.  The fused sweep then neither reads e nor
+// needs it cleared (at 1024^3 the clearing took 0.65 ms of a step's 85, at 256^3 12.7 us of 1240); the membranes' cut
+// cells read e, and small grids are relaxed in place, so these clear it.
+inline bool sweep_from_zero(const Hierarchy *h, const ibm_tables *t, const void *e, const void *r, int nu1) {
+  return h->zmarch && !t->membrane && nu1 > 0 && (e == h->tm_base[0] || e == h->tm_base[1]) && r == h->tm_rbase;
+}
+
 // One fused red-black sweep of level l: the finest level (tensor maps of the hierarchy, ghost
 // values read as neighbours) or a coarse level (its own maps, face fractions on irregular
-// cells).  e is swapped to the output buffer.
+// cells).  e is swapped to the output buffer.  zero: the field is zero, whatever e holds.
 template <typename T>
-void sweep_zmarch(Solver &S, int l, T *&e, const double *shift) {
+void sweep_zmarch(Solver &S, int l, T *&e, const double *shift, bool zero = false) {
   Hierarchy *h = S.h;
   Level &L0 = h->lv[l];
   const bool coarse = l > 0;
@@ -3326,6 +3338,7 @@ void sweep_zmarch(Solver &S, int l, T *&e, const double *shift) {
   a.shift = shift;
   a.omega = (float)S.omega;
   a.out = other;
+  a.ez = zero ? sweep_zero_plane(a.nz) : 0;
   a.err = S.ctx->errflag;
   const int gx = (a.nx + zm::TX - 1) / zm::TX, gy = (a.ny + zm::TY - 1) / zm::TY;
   const long long tiles = (long long)gx * gy;
@@ -3395,7 +3408,8 @@ void cut_relax(Solver &S, T *e, const T *eg, const T *r, const double *shift) {
 }
 
 template <typename T>
-void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool fine, const T *ghost_rhs, int sweeps) {
+void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool fine, const T *ghost_rhs, int sweeps,
+                  bool zero = false) {
   Level &L = S.h->lv[l];
   LV<T> v = view<T>(L);
   const int kz = relax_kz<T>((long long)L.g.nx * L.g.ny * L.g.nz);
@@ -3412,8 +3426,8 @@ void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool
     // the finest level's fused sweep, when e and r are the arrays its tensor maps cover (in
     // FP64 the solution and right-hand side of the V-cycle on p)
     if (fine && S.h->zmarch && (e == S.h->tm_base[0] || e == S.h->tm_base[1]) && (const void *)r == S.h->tm_rbase) {
-      T *old = e;
-      sweep_zmarch<T>(S, 0, e, shift);
+      T *old = zero && s == 0 ? nullptr : e;
+      sweep_zmarch<T>(S, 0, e, shift, zero && s == 0);
       if (timed) cudaEventRecord((*S.sweep_events)[2 * s + 1], S.st);
       cut_relax<T>(S, e, old, r, shift);
       const long long ng = S.t->nghost;
@@ -3484,8 +3498,9 @@ void tail_fill(TailArgs<T> &A, Hierarchy *h, int l, const double *shift, const i
 
 // V-cycle for level l: e_l (in/out) approximately solves A_l e_l = r_l - shift_l.  On the
 // finest level e is the hierarchy's own pointer: the fused sweep swaps it between two buffers.
+// zero: e is zero, whatever its buffer holds (only where sweep_from_zero)
 template <typename T>
-void vcycle(Solver &S, int l, T *&e, const T *r, const double *shift, const T *ghost_rhs) {
+void vcycle(Solver &S, int l, T *&e, const T *r, const double *shift, const T *ghost_rhs, bool zero = false) {
   Hierarchy *h = S.h;
   const int nl = (int)h->lv.size();
   if (l > 0 && l == h->tail_level && nl - l >= 2) {
@@ -3502,7 +3517,7 @@ void vcycle(Solver &S, int l, T *&e, const T *r, const double *shift, const T *g
     return;
   }
   const bool fine = (l == 0);
-  smooth_level<T>(S, l, e, r, shift, fine, ghost_rhs, S.nu1);
+  smooth_level<T>(S, l, e, r, shift, fine, ghost_rhs, S.nu1, zero);
   Level &F = h->lv[l], &C = h->lv[l + 1];
   T *ec = (T *)C.e, *rc = (T *)C.r;
   const int lg = row_lg(C.g.nx);
@@ -3957,8 +3972,9 @@ void run_step(Run &R, cudaStream_t bs) {
   } else {
     float *&e32 = reinterpret_cast<float *&>(L0.e);
     for (int q = 0; q < std::max(1, opts->inner_cycles); ++q) {
-      if (q == 0) cudaMemsetAsync(e32, 0, sizeof(float) * ntot, bs);
-      vcycle<float>(S, 0, e32, R.r32, S.scal + S_MU, R.r32);
+      const bool zero = q == 0 && sweep_from_zero(h, R.t, e32, R.r32, S.nu1);
+      if (q == 0 && !zero) cudaMemsetAsync(e32, 0, sizeof(float) * ntot, bs);
+      vcycle<float>(S, 0, e32, R.r32, S.scal + S_MU, R.r32, zero);
     }
     if (R.gcr_m > 0) {
       gcr_step<float>(S, e32, R.r32, R.gcr_m);
@@ -4396,8 +4412,14 @@ const double *lk_shift(Lock &K, int i, int l) {
   return l == 0 ? scal + S_MU : scal + S_LEVEL_SHIFT + l;
 }
 
-// one fused sweep of level l of every problem in grp (all swept by the z-march on that level)
-void lk_zmarch(Lock &K, int l, const std::vector<int> &grp) {
+// can a cycle's first sweep of problem i's finest level start from zero without clearing e
+bool lk_from_zero(Lock &K, int i) {
+  return sweep_from_zero(lk_h(K, i), (*K.R)[i].t, K.E[0][i], (*K.R)[i].r32, K.nu1);
+}
+
+// one fused sweep of level l of every problem in grp (all swept by the z-march on that level); zero: e
+// is zero where lk_from_zero
+void lk_zmarch(Lock &K, int l, const std::vector<int> &grp, bool zero) {
   const bool coarse = l > 0;
   const long long resident = coarse ? K.zmc_resident : K.zm_resident;
   // one chunk length for the launch: the fewest rounds x steps over every problem's items, as
@@ -4445,6 +4467,7 @@ void lk_zmarch(Lock &K, int l, const std::vector<int> &grp) {
       a.shift = lk_shift(K, i, l);
       a.omega = K.omega;
       a.out = other;
+      a.ez = zero && lk_from_zero(K, i) ? sweep_zero_plane(a.nz) : 0;
       a.err = K.ctx->errflag;
       a.kz = std::min(best_kz, a.nz);
       a.tiles_x = (a.nx + zm::TX - 1) / zm::TX;
@@ -4490,13 +4513,17 @@ void lk_ghost_update(Lock &K, const std::vector<int> &grp) {
                     [&](const BL<PGhost> &L, int b) { kb_ghost_store<<<b, 128, 0, K.st>>>(L); K.ctx->launches += 1; });
 }
 
-void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
+void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps, bool zero = false) {
   for (int s = 0; s < sweeps; ++s) {
     std::vector<int> zg, rg;
     for (int i : grp) ((l == 0 ? lk_h(K, i)->zmarch : lk_h(K, i)->lv[l].zm) ? zg : rg).push_back(i);
     if (!zg.empty()) {
       std::vector<float *> old(K.E[l]);
-      lk_zmarch(K, l, zg);
+      const bool z = zero && s == 0;
+      if (z)
+        for (int i : zg)
+          if (lk_from_zero(K, i)) old[i] = nullptr;
+      lk_zmarch(K, l, zg, z);
       if (l == 0)
         bl_launch<PGhost>(zg, [&](int i) { return lk_ghost_blocks(K, i); },
                           [&](int i) { return lk_ghost(K, i, K.E[0][i], old[i]); },
@@ -4533,7 +4560,7 @@ void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps) {
 // the restriction's grid of level l -> l + 1, as the single-problem V-cycle takes it
 void lk_restrict_grid(Hierarchy *h, int l, int &gx, int &gy) { restrict_grid(h, l, gx, gy); }
 
-void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
+void lk_vcycle(Lock &K, int l, const std::vector<int> &grp, bool zero = false) {
   std::vector<int> tail, coarsest, mid;
   for (int i : grp) {
     Hierarchy *h = lk_h(K, i);
@@ -4566,7 +4593,7 @@ void lk_vcycle(Lock &K, int l, const std::vector<int> &grp) {
                          });
   }
   if (mid.empty()) return;
-  lk_smooth(K, l, mid, K.nu1);
+  lk_smooth(K, l, mid, K.nu1, zero);
   bl_launch<PRestrict>(mid,
                        [&](int i) {
                          int gx, gy;
@@ -4899,16 +4926,18 @@ ibm_status lockstep_step(Lock &K, const std::vector<int> &act, int inner) {
   IBM_TRY(cudaMemsetAsync(ctx->lk_count, 0, sizeof(int) * LK_COUNTERS, K.st));
   K.ncount = 0;
   for (int q = 0; q < std::max(1, inner); ++q) {
-    if (q == 0)
-      bl_launch<PZero>(act, [&](int i) { return (int)std::min<long long>(nblk(R[i].ntot / 4, 256), 1024); },
+    if (q == 0) {
+      auto blocks = [&](int i) { return lk_from_zero(K, i) ? 0 : (int)std::min<long long>(nblk(R[i].ntot / 4, 256), 1024); };
+      bl_launch<PZero>(act, blocks,
                        [&](int i) {
                          PZero p;
                          p.p = K.E[0][i]; p.n = R[i].ntot;
-                         p.gx = (int)std::min<long long>(nblk(R[i].ntot / 4, 256), 1024);
+                         p.gx = blocks(i);
                          return p;
                        },
                        [&](const BL<PZero> &L, int b) { kb_zero<<<b, 256, 0, K.st>>>(L); ctx->launches += 1; });
-    lk_vcycle(K, 0, act);
+    }
+    lk_vcycle(K, 0, act, q == 0);
   }
   for (int i : act) R[i].h->lv[0].e = K.E[0][i];
   lk_outer(K, act);

@@ -176,6 +176,8 @@ struct Args {
   const double *shift;
   float omega;
   void *out;              // the output e, of the storage type
+  int ez;                 // added to the plane coordinate of the loads of e: 0, or past the last plane where the
+                          // field is zero (the copies then fill zeros, nothing is read or cleared first)
   int *err;
 };
 
@@ -431,7 +433,7 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
   // padded coordinates: cell (i, j, k) at (i + OX, j + 1, k + 1); OX = 4
   auto load_e = [&](int plane, int b) {
     mbar_expect_tx(&s.bar_e[b], ebytes);
-    tma_load3(s.e[b], tm_e, &s.bar_e[b], x0, y0 - 1, plane + 1);
+    tma_load3(s.e[b], tm_e, &s.bar_e[b], x0, y0 - 1, plane + 1 + (COARSE ? 0 : a.ez));
     pend_e |= 1u << b;
   };
   auto load_r = [&](int plane, int b) {
