@@ -1789,29 +1789,56 @@ __global__ void k_pack(const double *src, LevelGeom g, double *dst, const uint8_
   pack_body(src, g, dst, mask, nonzero, HwGrid{});
 }
 
+// Unpacks stream padded arrays into the user's [k][j][i] array.  Blocks take PK_CELLS consecutive cells,
+// four per thread a block apart: the user's array is written contiguously over the warp, and four
+// loads are in flight before the first use.  Four cells along x per thread put a warp's 8-byte stores
+// 32 bytes apart, four passes over every sector: 4582 us at 1024^3 and 84 us (pairs) at 256^3; this takes
+// 3219 and 69 us.  The packs, which store 16 or 32 bytes per thread and whose scattered loads the L1
+// merges, are no faster this way (69 against 50 us for the pairs).
+constexpr int PK_THREADS = 256, PK_PER = 4, PK_CELLS = PK_THREADS * PK_PER;
+inline int pack_blocks(const LevelGeom &g, int wave) {
+  return (int)std::max<long long>(1, std::min<long long>(wave, ((long long)g.nx * g.ny * g.nz + PK_CELLS - 1) / PK_CELLS));
+}
+// ld(padded index, value slot) for a thread's cells, then st(cell, slot)
+template <class GR, class LD, class ST>
+__device__ __forceinline__ void pack_cells(const LevelGeom &g, const GR &grid, LD ld, ST st) {
+  const long long n = (long long)g.nx * g.ny * g.nz;
+  // quotients by multipliers, exact for x d < 2^32; longer rows or columns than 2^15 divide
+  const bool mul = g.nx < 32768 && g.ny < 32768;
+  const unsigned mx = 0xffffffffu / (unsigned)g.nx + 1u, my = 0xffffffffu / (unsigned)g.ny + 1u;   // 0 for 1
+  auto div = [&](unsigned x, unsigned d, unsigned m) { return d == 1u ? x : mul ? __umulhi(x, m) : x / d; };
+  for (long long q0 = grid.bx() * (long long)PK_CELLS; q0 < n; q0 += grid.gx() * (long long)PK_CELLS) {
+    const unsigned row0 = (unsigned)(q0 / g.nx), x0 = (unsigned)(q0 - (long long)row0 * g.nx);
+    const unsigned k0 = row0 / (unsigned)g.ny, j0 = row0 - k0 * (unsigned)g.ny;
+#pragma unroll
+    for (int u = 0; u < PK_PER; ++u) {
+      const unsigned x = x0 + u * PK_THREADS + threadIdx.x, dr = div(x, g.nx, mx), j = j0 + dr, dk = div(j, g.ny, my);
+      const long long id = (long long)(k0 + dk + 1) * g.sz + (long long)(j - dk * (unsigned)g.ny + 1) * g.sy + OX +
+                           (x - dr * (unsigned)g.nx);
+      const long long q = q0 + u * PK_THREADS + threadIdx.x;
+      if (q < n) ld(id, u);
+    }
+#pragma unroll
+    for (int u = 0; u < PK_PER; ++u) {
+      const long long q = q0 + u * PK_THREADS + threadIdx.x;
+      if (q < n) st(q, u);
+    }
+  }
+}
+
 // unpack with the gauge applied: dst = p - mean on active cells, 0 on plain solid cells
 template <class GR>
 __device__ __forceinline__ void unpack_gauge_body(const double *src, const uint8_t *mask, const LevelGeom &g,
                                                   const double *scal, double *dst, const GR &grid) {
-  const RowGroups rg(g.nx);
-  const int rows = g.ny * g.nz;
-  if (!rg.active()) return;
   const double mean = scal[S_MEANP];
-  for (int row = rg.first_row(grid); row < rows; row += rg.row_step(grid)) {
-    const int j = row % g.ny, k = row / g.ny;
-    const long long q0 = (long long)row * g.nx;
-    const long long base = (long long)(k + 1) * g.sz + (long long)(j + 1) * g.sy + OX;
-    for (int gr = rg.g0; gr < rg.G; gr += rg.gstep) {
-      const long long id = base + 4 * gr;
-      const uchar4 m = *reinterpret_cast<const uchar4 *>(mask + id);
-      const uint8_t mv[4] = {m.x, m.y, m.z, m.w};
-      double P[4];
-      Vec4<double>::ld(src + id, P);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (4 * gr + u < g.nx) dst[q0 + 4 * gr + u] = mv[u] == 1 ? 0.0 : P[u] - mean;
-    }
-  }
+  double P[PK_PER];
+  uint8_t m[PK_PER];
+  pack_cells(g, grid,
+             [&](long long id, int u) {
+               P[u] = src[id];
+               m[u] = mask[id];
+             },
+             [&](long long q, int u) { dst[q] = m[u] == 1 ? 0.0 : P[u] - mean; });
 }
 
 __global__ void k_unpack_gauge(const double *src, const uint8_t *mask, LevelGeom g, const double *scal, double *dst) {
@@ -2164,32 +2191,22 @@ template <class GR>
 __device__ __forceinline__ void unpack_gauge_df_body(const float *ph, const float *pl, const uint8_t *mask,
                                                      const LevelGeom &g, const double *scal, double *dst,
                                                      const GR &grid) {
-  const RowGroups rg(g.nx);
-  const int rows = g.ny * g.nz;
-  if (!rg.active()) return;
   float mh, ml;
   dfl::split(scal[S_MEANP], mh, ml);
-  for (int row = rg.first_row(grid); row < rows; row += rg.row_step(grid)) {
-    const int j = row % g.ny, k = row / g.ny;
-    const long long q0 = (long long)row * g.nx;
-    const long long base = (long long)(k + 1) * g.sz + (long long)(j + 1) * g.sy + OX;
-    for (int gr = rg.g0; gr < rg.G; gr += rg.gstep) {
-      const long long id = base + 4 * gr;
-      const uchar4 m = *reinterpret_cast<const uchar4 *>(mask + id);
-      const uint8_t mv[4] = {m.x, m.y, m.z, m.w};
-      float PH[4], PL[4];
-      Vec4<float>::ld(ph + id, PH);
-      Vec4<float>::ld(pl + id, PL);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (4 * gr + u >= g.nx) continue;
-        float s, t;
-        dfl::two_sum(PH[u], -mh, s, t);
-        t += PL[u] - ml;
-        dst[q0 + 4 * gr + u] = mv[u] == 1 ? 0.0 : dfl::join(s, t);
-      }
-    }
-  }
+  float H[PK_PER], L[PK_PER];
+  uint8_t m[PK_PER];
+  pack_cells(g, grid,
+             [&](long long id, int u) {
+               H[u] = ph[id];
+               L[u] = pl[id];
+               m[u] = mask[id];
+             },
+             [&](long long q, int u) {
+               float s, t;
+               dfl::two_sum(H[u], -mh, s, t);
+               t += L[u] - ml;
+               dst[q] = m[u] == 1 ? 0.0 : dfl::join(s, t);
+             });
 }
 
 __global__ void k_unpack_gauge_df(const float *ph, const float *pl, const uint8_t *mask, LevelGeom g,
@@ -4031,9 +4048,9 @@ void run_finish(Run &R, double *p_user, cudaStream_t st) {
     k_gauge_sum<<<row_blocks(L0.g, REDUCE_BLOCKS), REDUCE_THREADS, 0, st>>>(fine_view64(h), h->p64, part);
   k_gauge_finalize<<<1, 256, 0, st>>>(part, REDUCE_BLOCKS, scal);
   if (R.S.dfo)
-    k_unpack_gauge_df<<<R.ctx->wave, 256, 0, st>>>(hi_of(h->p64), lo_of(h->p64, ntot), L0.mask, L0.g, scal, p_user);
+    k_unpack_gauge_df<<<pack_blocks(L0.g, R.ctx->wave), PK_THREADS, 0, st>>>(hi_of(h->p64), lo_of(h->p64, ntot), L0.mask, L0.g, scal, p_user);
   else
-    k_unpack_gauge<<<R.ctx->wave, 256, 0, st>>>(h->p64, L0.mask, L0.g, scal, p_user);
+    k_unpack_gauge<<<pack_blocks(L0.g, R.ctx->wave), PK_THREADS, 0, st>>>(h->p64, L0.mask, L0.g, scal, p_user);
   R.ctx->launches += 3;
 }
 
@@ -4864,7 +4881,7 @@ void lk_finish(Lock &K, const std::vector<int> &all, double *const *p_user) {
                     });
   bl_launch<PGauge>(all, [](int) { return 1; }, fill,
                     [&](const BL<PGauge> &L, int b) { kb_gauge_finalize<<<b, 256, 0, K.st>>>(L); K.ctx->launches += 1; });
-  bl_launch<PUnpack>(all, [&](int i) { return row_blocks(R[i].h->lv[0].g, K.ctx->wave); },
+  bl_launch<PUnpack>(all, [&](int i) { return pack_blocks(R[i].h->lv[0].g, K.ctx->wave); },
                      [&](int i) {
                        Hierarchy *h = R[i].h;
                        PUnpack p{};
@@ -4874,7 +4891,7 @@ void lk_finish(Lock &K, const std::vector<int> &all, double *const *p_user) {
                        p.g = h->lv[0].g;
                        p.scal = R[i].S.scal;
                        p.dst = p_user[i];
-                       p.gx = row_blocks(p.g, K.ctx->wave);
+                       p.gx = pack_blocks(p.g, K.ctx->wave);
                        return p;
                      },
                      [&](const BL<PUnpack> &L, int b) { kb_unpack_gauge<<<b, 256, 0, K.st>>>(L); K.ctx->launches += 1; });

@@ -214,3 +214,23 @@ def test_cycles_that_start_from_zero(ctx, nu1, nu2, inner, krylov):
             d = (p - want).cpu().numpy()[fl]
             assert np.linalg.norm(d) < 1e-8 * np.linalg.norm(want.cpu().numpy()[fl]), (seed, prec)
     T.close()
+
+
+@pytest.mark.parametrize("shape", [(1030, 5, 6), (3, 31, 40), (257, 7, 9), (6, 5, 4)])
+def test_packs_by_row_length(ctx, shape):
+    """Packs and unpacks take blocks of 1024 consecutive cells: rows longer than a block, many rows in
+    a block, a last block in part.  A warm start is met at once and must come back
+    as it was but for its mean."""
+    pkg, c = ctx
+    n = max(shape)
+    f = [m / n * synth.faces_tanh(m, 1.2) for m in shape]
+    T = pkg.Tables(c, *f, [])
+    b = torch.from_numpy(synth.rhs_divergence(*f, 3)).cuda()
+    guess = synth.smooth_field(*f, 5) + synth.counter_normal(3, 1, np.arange(b.numel())).reshape(b.shape)
+    for prec in (0, 1, 2):
+        p = torch.from_numpy(guess.copy()).cuda()
+        T.solve(b, p, 1e30, pkg.SolveOpts(precision=prec))   # no cycle: pack, mean, unpack
+        d = p.cpu().numpy() - guess                          # minus the mean, a constant
+        # pairs carry 48 bits and the difference is rounded a few times
+        assert np.max(d) - np.min(d) <= 16 * 2.0**-48 * np.max(np.abs(guess)), prec
+    T.close()
