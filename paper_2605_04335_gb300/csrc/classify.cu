@@ -854,10 +854,16 @@ __device__ __forceinline__ double fallback_kappa(const GhostArgs &a, const doubl
   return -sqrt((fx * fx + fy * fy) + fz * fz);
 }
 
-// the closest of each ghost's candidates in FP64 (lowest index on exact ties) and its row, one
-// thread per ghost
+// The closest of each ghost's candidates in FP64 (lowest index on exact ties) and its row, L lanes per
+// ghost: one where there are ghosts enough to fill the FP64 pipe; with few of them the chain of
+// a thread's up to six distances decides (55 us whatever their number), and eight lanes take one each:
+// 28 us up to 8000 ghosts, 41 against 55 us at 8200, above which the two meet.
+constexpr int TABLE_LANES = 8;
+constexpr long long TABLE_FEW = 8192;
+template <int L>
 __global__ void __launch_bounds__(TABLE_THREADS) k_ghost_tables(GhostArgs a) {
-  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long g = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / L;
+  const int sub = (int)threadIdx.x & (L - 1);
   if (g >= a.ng) return;
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   long long lin = a.gcell[g];
@@ -867,7 +873,7 @@ __global__ void __launch_bounds__(TABLE_THREADS) k_ghost_tables(GhostArgs a) {
   double P[3] = {a.xc[gi], a.yc[gj], a.zc[gk]};
   double best = 1e300, BQ[3] = {0.0, 0.0, 0.0};
   int bidx = 0x7fffffff;
-  for (int q = 0; q < a.ncand[g]; ++q) {
+  for (int q = sub; q < a.ncand[g]; q += L) {
     const int t = a.cand[CAND_OUT * g + q];
     double d2, Q[3];
     closest_on_tri(P, a.tv + 9 * t, a.tv + 9 * t + 3, a.tv + 9 * t + 6, Q, d2);
@@ -875,6 +881,21 @@ __global__ void __launch_bounds__(TABLE_THREADS) k_ghost_tables(GhostArgs a) {
       best = d2; bidx = t;
       BQ[0] = Q[0]; BQ[1] = Q[1]; BQ[2] = Q[2];
     }
+  }
+  if constexpr (L > 1) {
+    const unsigned m = ((1u << L) - 1u) << ((int)threadIdx.x & 31 & ~(L - 1));   // the ghost's lanes
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) {
+      const double d2 = __shfl_xor_sync(m, best, o, L);
+      const int t = __shfl_xor_sync(m, bidx, o, L);
+      double Q[3];
+      for (int d = 0; d < 3; ++d) Q[d] = __shfl_xor_sync(m, BQ[d], o, L);
+      if (d2 < best || (d2 == best && t < bidx)) {
+        best = d2; bidx = t;
+        BQ[0] = Q[0]; BQ[1] = Q[1]; BQ[2] = Q[2];
+      }
+    }
+    if (sub) return;
   }
   double IP[3];
   for (int d = 0; d < 3; ++d) {
@@ -1810,7 +1831,8 @@ ibm_status classify_into(ibm_tables *T, const ibm_mesh *meshes, int nmesh, long 
     ga.base = T->gbase; ga.flags = T->gflags; ga.ref = T->gref;
     ga.kappa = T->gkappa; ga.tri = T->gtri; ga.wself = T->gwself;
     k_ghost_candidates<<<nblk(32 * ng, TABLE_THREADS), TABLE_THREADS, 0, st>>>(ga);
-    k_ghost_tables<<<nblk(ng, TABLE_THREADS), TABLE_THREADS, 0, st>>>(ga);
+    if (ng <= TABLE_FEW) k_ghost_tables<TABLE_LANES><<<nblk(TABLE_LANES * ng, TABLE_THREADS), TABLE_THREADS, 0, st>>>(ga);
+    else k_ghost_tables<1><<<nblk(ng, TABLE_THREADS), TABLE_THREADS, 0, st>>>(ga);
     CTRY(cudaGetLastError());
   }
   unsigned long long hc[2];

@@ -234,3 +234,13 @@ def test_packs_by_row_length(ctx, shape):
         # pairs carry 48 bits and the difference is rounded a few times
         assert np.max(d) - np.min(d) <= 16 * 2.0**-48 * np.max(np.abs(guess)), prec
     T.close()
+
+
+@pytest.mark.parametrize("n,r", [(20, 0.11), (56, 0.3), (88, 0.34), (96, 0.36)])
+def test_ghost_tables_by_number(ctx, n, r):
+    """Eight lanes per ghost up to 8192 ghosts, one above: bit for bit the oracle's tables on both sides."""
+    pkg, c = ctx
+    f = synth.faces_tanh(n, 1.3)
+    _, T, ex, ib, G = classify_both(pkg, c, f, f, f, [synth.octa_sphere(4, (0.5, 0.49, 0.51), r)])
+    assert_tables_equal(ex, ib, G)
+    T.close()
