@@ -771,20 +771,62 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 && FINEST ? 5 : 4)
   restrict8_body<T, FINEST, SF, SC>(f, e, r, shift, cv, rc, ec, partials, lg, HwGrid{});
 }
 
-// deterministic sum of nb partials (stride `stride`, offset `off`) in one block
-__device__ double block_sum_partials(const double *p, int nb, int stride, int off) {
-  __shared__ double sm[256];
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) s += p[b * stride + off];
-  sm[threadIdx.x] = s;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if (threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
-    __syncthreads();
+// Deterministic sums of N arrays of partials (nb of stride `stride` each) in one block of 256 threads: each
+// thread's share in order, then a halving tree.  Pure latency, and on the path of every level of a
+// V-cycle: the loads of all sums are in flight at once, and the tree is one barrier (a warp per sum
+// takes it from 256 values, by shuffles from 32 on).  The four sums of a residual: 7.5 us with a barrier per
+// halving and one sum after another, 4.8 now
+constexpr int SUM_THREADS = 256;
+template <int N>
+__device__ __forceinline__ void block_sums(const double *const (&p)[N], const int (&nb)[N], const int (&stride)[N],
+                                           double (&out)[N]) {
+  __shared__ double sm[N][SUM_THREADS], tot[N];
+  const int t = threadIdx.x, lane = t & 31;
+  int most = 0;
+  double s[N];
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    s[n] = 0.0;
+    most = max(most, nb[n]);
   }
-  double out = sm[0];
+  for (int b0 = t; b0 < most; b0 += 4 * SUM_THREADS) {
+    double v[N][4];
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int b = b0 + u * SUM_THREADS;
+        if (b < nb[n]) v[n][u] = p[n][(long long)b * stride[n]];
+      }
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (b0 + u * SUM_THREADS < nb[n]) s[n] += v[n][u];
+  }
+#pragma unroll
+  for (int n = 0; n < N; ++n) sm[n][t] = s[n];
   __syncthreads();
-  return out;
+#pragma unroll
+  for (int n = 0; n < N; ++n)
+    if ((t >> 5) == n) {
+      double q[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) q[k] = sm[n][lane + 32 * k] + sm[n][lane + 32 * k + 128];
+      double x = (q[0] + q[2]) + (q[1] + q[3]);
+#pragma unroll
+      for (int st = 16; st > 0; st >>= 1) x += __shfl_down_sync(0xffffffffu, x, st);
+      if (lane == 0) tot[n] = x;
+    }
+  __syncthreads();
+#pragma unroll
+  for (int n = 0; n < N; ++n) out[n] = tot[n];
+}
+// sum of nb partials (stride `stride`, offset `off`)
+__device__ __forceinline__ double block_sum_partials(const double *p, int nb, int stride, int off) {
+  double out[1];
+  block_sums<1>({p + off}, {nb}, {stride}, out);
+  return out[0];
 }
 
 __device__ __forceinline__ void finalize_shift_body(const double *partials, int nb, const double *fluid_vol,
@@ -1657,10 +1699,10 @@ __global__ void k_ghost_resid64(const long long *src, const long long *dst, cons
 // (cpart, ncb: block partials of the membrane cut cells, same layout as partials; ncb may be 0)
 __device__ __forceinline__ void finalize_resid_body(const double *partials, int nb, const double *gpart, int ngb,
                                                     double *scal, int update_lambda, const double *cpart, int ncb) {
-  double sv = block_sum_partials(partials, nb, 3, 0);
-  double s1 = block_sum_partials(partials, nb, 3, 1);
-  double s2 = block_sum_partials(partials, nb, 3, 2);
-  double sg = ngb > 0 ? block_sum_partials(gpart, ngb, 1, 0) : 0.0;
+  double sums[4];
+  block_sums<4>({partials, partials + 1, partials + 2, gpart}, {nb, nb, nb, ngb}, {3, 3, 3, 1}, sums);
+  double sv = sums[0], s1 = sums[1], s2 = sums[2];
+  const double sg = sums[3];   // 0 without ghost rows
   if (ncb > 0) {
     sv += block_sum_partials(cpart, ncb, 3, 0);
     s1 += block_sum_partials(cpart, ncb, 3, 1);
