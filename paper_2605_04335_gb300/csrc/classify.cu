@@ -857,7 +857,7 @@ __device__ __forceinline__ double fallback_kappa(const GhostArgs &a, const doubl
 // The closest of each ghost's candidates in FP64 (lowest index on exact ties) and its row, L lanes per
 // ghost: one where there are ghosts enough to fill the FP64 pipe; with few of them the chain of
 // a thread's up to six distances decides (55 us whatever their number), and eight lanes take one each:
-// 28 us up to 8000 ghosts, 41 against 55 us at 8200, above which the two meet.
+// 28 us up to 6000 ghosts, 41 near 8000, above which the two meet.
 constexpr int TABLE_LANES = 8;
 constexpr long long TABLE_FEW = 8192;
 template <int L>

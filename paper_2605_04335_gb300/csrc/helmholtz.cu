@@ -63,8 +63,8 @@ template <typename T> __device__ __forceinline__ T relax_rcp(T D);
 template <> __device__ __forceinline__ float relax_rcp<float>(float D) { return __frcp_rn(D); }
 template <> __device__ __forceinline__ double relax_rcp<double>(double D) { return (double)__frcp_rn((float)D); }
 
-// one Jacobi step of the fluid rows with relaxation w: un = u + w (f - H u) / D, each block a
-// 32 x 8 tile marching KCH planes in z with the z-neighbours in registers; the next plane's
+// one Jacobi step of the fluid rows with relaxation w (FP64, precision 0): un = u + w (f - H u) / D, each
+// block a 32 x 8 tile marching KCH planes in z with the z-neighbours in registers; the next plane's
 // value, mask and right-hand side are loaded one plane ahead
 template <typename T>
 __global__ void __launch_bounds__(TX *TY) k_hz_sweep(HzView<T> v, const T *u, T *un, const T *f, T w) {

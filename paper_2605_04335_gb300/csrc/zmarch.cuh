@@ -2,9 +2,9 @@
 // TMA-staged planes in shared memory, persistent CTAs over (x-y tile, z-chunk) items.  FP32
 // (the mixed solves' multigrid, two CTAs per SM) and FP64 (the FP64 solve's smoother on p,
 // one CTA per SM: its buffers take 190 KB of shared memory) share the code, for the finest
-// level and (FP32) the coarse levels of at least 2^18 cells; a coarse level may store its e
-// and r in BF16 (S = bf16: staged as BF16, widened exactly on load, rounded on store).  A
-// batched form (k_sweep_zmarch_batch) sweeps the same level of several problems in one launch.
+// level and (FP32) the coarse levels of at least 2^26 cells (of 2^18 when stored in BF16: staged as
+// BF16, S = bf16, widened exactly on load, rounded on store; smaller ones are relaxed strip by strip).
+// A batched form (k_sweep_zmarch_batch) sweeps the same level of several problems in one launch.
 //
 // One item is an x-y tile (TX x TY) and a z-range [k0, k1).  Step q of its march
 //   1. updates the red cells of plane q on the tile, and the one-cell ring that the tile's
