@@ -20,7 +20,7 @@
 //
 // Both passes are bound by the FP64 pipe (1.6 fused multiply-adds per clock and SM), so they spend
 // as few FP64 operations as they can: one warp marches 16 planes of 32 (first pass) or 31 cells of a
-// row.  First pass: one per cell for sum V b (weighed by dz in the march, by dx dy once).  Second
+// row, or of several short rows.  First pass: one per cell for sum V b (weighed by dz in the march, by dx dy once).  Second
 // pass, about 14: each difference along z serves two planes and each one along x two lanes (by a
 // shuffle; lane 0 only provides it), two along y, six products, and four for the two squares.  The
 // direct form of both passes (stencil, volumes and sums per cell, 36 operations) took 1340 us at
@@ -123,21 +123,28 @@ struct NaArgs {
   const double *gw, *gscale, *gd;
 };
 
-// one warp's march: cells i0 + lane of row j, planes [k0, k1); the warps of the grid take the marches
-// in turn (`cells` per warp and row)
+// One warp's march: planes [k0, k1) of 32 / w rows, w lanes (a power of two) along each.  Rows of up to 32
+// cells take the lanes they need; longer ones go in pieces of 32 cells, or of 31 after a lane that holds
+// the cell before them (before = 1).  The warps of the grid take the marches in turn.  With one row per
+// warp whatever its length, the second pass took 840 us over 4 x 1024 x 1024 cells and 251 us over
+// 8 x 512 x 512; now 128 and 68 us, as the same cells in long rows (120 us over 1024 x 1024 x 4).
 struct NaMarch {
   long long n;     // marches
-  int nxb, nzc;
-  __device__ NaMarch(const NaArgs &a, int cells) {
-    nxb = (a.nx + cells - 1) / cells;
-    nzc = (a.nz + NA_KZ - 1) / NA_KZ;
-    n = (long long)nxb * a.ny * nzc;
+  int nxb, nyb, lw, step, before;
+  __device__ NaMarch(const NaArgs &a, int before_) {
+    lw = a.nx > 16 ? 5 : 32 - __clz(a.nx - 1);
+    before = a.nx > 32 ? before_ : 0;
+    step = 32 - before;
+    nxb = a.nx > 32 ? (a.nx + step - 1) / step : 1;
+    nyb = (a.ny + (32 >> lw) - 1) >> (5 - lw);
+    n = (long long)nxb * nyb * ((a.nz + NA_KZ - 1) / NA_KZ);
   }
-  __device__ __forceinline__ void at(long long m, int cells, const NaArgs &a, int &i0, int &j, int &k0, int &k1) const {
-    i0 = (int)(m % nxb) * cells;
+  // the lane's column of march m (i or j may lie outside the grid)
+  __device__ __forceinline__ void at(long long m, const NaArgs &a, int lane, int &i, int &j, int &k0, int &k1) const {
+    i = (int)(m % nxb) * step - before + (lane & ((1 << lw) - 1));
     const long long q = m / nxb;
-    j = (int)(q % a.ny);
-    k0 = (int)(q / a.ny) * NA_KZ;
+    j = ((int)(q % nyb) << (5 - lw)) + (lane >> lw);
+    k0 = (int)(q / nyb) * NA_KZ;
     k1 = min(a.nz, k0 + NA_KZ);
   }
 };
@@ -168,13 +175,12 @@ __global__ void __launch_bounds__(NA_THREADS) k_na_pass1(double *scr, NaArgs a) 
   const long long ncell = (long long)a.nx * a.ny * a.nz, sy = a.nx, sz = (long long)a.nx * a.ny;
   const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, ts = (long long)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
-  const NaMarch M(a, 32);
+  const NaMarch M(a, 0);
   long long count = 0;
   for (long long m = t0 >> 5; m < M.n; m += ts >> 5) {
-    int i0, j, k0, k1;
-    M.at(m, 32, a, i0, j, k0, k1);
-    const int i = i0 + lane;
-    if (i >= a.nx) continue;
+    int i, j, k0, k1;
+    M.at(m, a, lane, i, j, k0, k1);
+    if (i >= a.nx || j >= a.ny) continue;
     const double dxy = ax[S1 + i] * ay[S1 + j];
     long long l = ((long long)k0 * a.ny + j) * a.nx + i;
     double sb = 0.0, sv = 0.0, flux = 0.0;
@@ -268,15 +274,16 @@ __global__ void __launch_bounds__(NA_THREADS) k_na_pass2(double *scr, NaArgs a) 
   const long long sz = (long long)a.nx * a.ny;
   const long long ts = (long long)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
-  const NaMarch M(a, 31);
+  const NaMarch M(a, 1);
+  const bool first = (lane & ((1 << M.lw) - 1)) == 0;   // of its row's lanes
   for (long long m = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; m < M.n; m += ts >> 5) {
-    int i0, j, k0, k1;
-    M.at(m, 31, a, i0, j, k0, k1);
-    // lane 0 is the cell before the first (or, at the wall, the first itself); lanes past the row
-    // repeat its last cell; coefficients across the walls are zero, and the cells read there the
-    // row's own
-    const int i = min(max(i0 - 1 + lane, 0), a.nx - 1);
-    const bool own = lane > 0 && i0 - 1 + lane < a.nx;
+    int ir, jr, k0, k1;
+    M.at(m, a, lane, ir, jr, k0, k1);
+    // long rows: the first lane is the cell before the piece (or, at the wall, its first cell), which
+    // it does not own; lanes past a row or past the last row repeat a cell there; coefficients across
+    // the walls are zero, and the cells read there the row's own
+    const int i = min(max(ir, 0), a.nx - 1), j = min(jr, a.ny - 1);
+    const bool own = !(M.before && first) && ir < a.nx && jr < a.ny;
     const long long xr = i < a.nx - 1 ? 1 : 0, ym = j > 0 ? -(long long)a.nx : 0, yp = j < a.ny - 1 ? a.nx : 0;
     const double cxm = ax[2 * S1 + i], cxp = ax[3 * S1 + i], cym = ay[2 * S1 + j], cyp = ay[3 * S1 + j];
     long long l = ((long long)k0 * a.ny + j) * a.nx + i;
@@ -288,7 +295,8 @@ __global__ void __launch_bounds__(NA_THREADS) k_na_pass2(double *scr, NaArgs a) 
       const double bl = a.b[l];
       const bool fluid = own && a.ib[l] == 0;
       const double dxp = px - pc, dzp = pz - pc;
-      const double dxm = __shfl_up_sync(full, dxp, 1);   // p_i - p_{i-1}
+      double dxm = __shfl_up_sync(full, dxp, 1);   // p_i - p_{i-1}
+      if (first) dxm = 0.0;   // from another row, or this lane's own
       double r = bl - mr;
       r = fma(cxm, dxm, r);
       r = fma(-cxp, dxp, r);
