@@ -16,6 +16,7 @@
 //   triangles, in ascending order, of f_t / 3.
 // Every FP64 operation is separately rounded (built with -fmad=false) in that order, so the
 // results are reproducible bit for bit by a plain implementation of the same definition.
+#include <type_traits>
 #include <vector>
 
 #include "ibm_internal.cuh"
@@ -184,62 +185,105 @@ __global__ void k_inc_fill(const int *tris, int ntri, const int *off, int *cur, 
   }
 }
 
+// ascending order of a thread's N values (Batcher's odd-even merge sort)
+template <int N>
+__device__ __forceinline__ void sort_ascending(int (&t)[N]) {
+#pragma unroll
+  for (int p = 1; p < N; p <<= 1)
+#pragma unroll
+    for (int k = p; k >= 1; k >>= 1)
+#pragma unroll
+      for (int j = k % p; j + k < N; j += 2 * k)
+#pragma unroll
+        for (int i = 0; i < k; ++i)
+          if (i + j + k < N && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+            const int lo = min(t[i + j], t[i + j + k]), hi = max(t[i + j], t[i + j + k]);
+            t[i + j] = lo;
+            t[i + j + k] = hi;
+          }
+}
+
 // F_i = sum of the shares of node i's triangles in ascending triangle order (the fill order is
-// arbitrary).  One warp per node, bound by the latency of its dependent loads and of the ordered
-// FP64 sum.  Up to 32 incident triangles each lane holds one: its rank (entries before it; equal
-// indices, a triangle naming the node twice, in list order) comes from shuffles, and the shares,
-// loaded by all lanes at once, are added in rank order through the warp.  More triangles: the
-// lanes rank 32 entries at a time against the whole list into sorted[], then sum it in chunks
-// of 32.  One thread per node that searched the list for each next triangle took 227 us on a
-// 4098-node mesh whose two poles have 128 triangles (all other nodes 6 or fewer), serial in the
-// square of the valence; this takes 27 us there.
-constexpr int NODE_THREADS = 128;
+// arbitrary).  Bound by the latency of its dependent loads on small meshes and by the FP64 adds and gathers
+// on large ones.  One thread per node of up to NODE_FEW triangles, nearly all of a mesh: it sorts them in
+// registers (the order of equal indices, a triangle naming the node twice, does not matter) and issues
+// the loads of eight shares before the first addition.  The block's nodes with more are taken by a warp
+// each: the lanes rank 32 entries at a time against the whole list into sorted[], then three of them sum
+// one component each.  With one thread per node whatever its triangles, searching the list for each next
+// one, a 4098-node mesh whose two poles have 128 (the others 6 or fewer) took 227 us, 262,146 nodes of 4
+// or 6 14 us; with a warp per node 27 and 297 us; this takes 25 and 16 us.
+constexpr int NODE_THREADS = 128, NODE_FEW = 16, NODE_LOADS = 8;
 __global__ void __launch_bounds__(NODE_THREADS) k_node_forces(const int *off, const int *list, const double *share,
                                                               long long nvert, int *sorted, double *F) {
+  __shared__ int many[NODE_THREADS], nmany;   // the block's nodes with more than NODE_FEW triangles
   const unsigned full = 0xffffffffu;
-  const long long i = (blockIdx.x * (long long)NODE_THREADS + threadIdx.x) >> 5;
+  const int none = 0x7fffffff;
+  const long long i0 = blockIdx.x * (long long)NODE_THREADS, i = i0 + threadIdx.x;
   const int lane = threadIdx.x & 31;
-  if (i >= nvert) return;   // whole warps
-  const int b = off[i], n = off[i + 1] - b;
-  const bool small = n <= 32;
-  int t = 0, rank = 0;
-  if (small) {
-    t = lane < n ? list[b + lane] : 0x7fffffff;
-    for (int k = 0; k < n; ++k) {
-      const int o = __shfl_sync(full, t, k);
-      rank += o < t || (o == t && k < lane);
+  const int b = i < nvert ? off[i] : 0, n = i < nvert ? off[i + 1] - b : 0;
+  if (threadIdx.x == 0) nmany = 0;
+  __syncthreads();
+  if (n > NODE_FEW) many[atomicAdd(&nmany, 1)] = (int)threadIdx.x;
+  __syncthreads();
+  auto few = [&](auto cap) {
+    constexpr int N = decltype(cap)::value;
+    int t[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) t[q] = q < n ? list[b + q] : none;
+    sort_ascending(t);
+    double acc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q0 = 0; q0 < N; q0 += NODE_LOADS) {
+      double v[NODE_LOADS][3];
+#pragma unroll
+      for (int q = 0; q < NODE_LOADS; ++q)
+        if (q0 + q < n)
+          for (int d = 0; d < 3; ++d) v[q][d] = share[3LL * t[q0 + q] + d];
+#pragma unroll
+      for (int q = 0; q < NODE_LOADS; ++q)
+        if (q0 + q < n)
+          for (int d = 0; d < 3; ++d) acc[d] = acc[d] + v[q][d];
     }
-  } else {
-    for (int k0 = 0; k0 < n; k0 += 32) {
+    for (int d = 0; d < 3; ++d) F[3 * i + d] = acc[d];
+  };
+  if (i < nvert && n <= NODE_LOADS) few(std::integral_constant<int, NODE_LOADS>{});
+  else if (i < nvert && n <= NODE_FEW) few(std::integral_constant<int, NODE_FEW>{});
+  for (int e = threadIdx.x >> 5; e < nmany; e += NODE_THREADS / 32) {   // whole warps
+    const long long I = i0 + many[e];
+    const int B = off[I], N = off[I + 1] - B;
+    for (int k0 = 0; k0 < N; k0 += 32) {
       const int k = k0 + lane;
-      const int tk = k < n ? list[b + k] : 0x7fffffff;
+      const int tk = k < N ? list[B + k] : none;
       int r = 0;
-      for (int m0 = 0; m0 < n; m0 += 32) {
-        const int tm = m0 + lane < n ? list[b + m0 + lane] : 0x7fffffff;
-        const int mc = min(32, n - m0);
+      for (int m0 = 0; m0 < N; m0 += 32) {
+        const int tm = m0 + lane < N ? list[B + m0 + lane] : none;
+        const int mc = min(32, N - m0);
         for (int q = 0; q < mc; ++q) {
           const int o = __shfl_sync(full, tm, q);
           r += o < tk || (o == tk && m0 + q < k);
         }
       }
-      if (k < n) sorted[b + r] = tk;
+      if (k < N) sorted[B + r] = tk;
     }
     __syncwarp();   // orders the lanes' writes of sorted[] before the reads below
-  }
-  double acc[3] = {0.0, 0.0, 0.0};
-  for (int k0 = 0; k0 < n; k0 += 32) {
-    const int kc = min(32, n - k0);
-    if (!small) t = lane < kc ? sorted[b + k0 + lane] : 0;
-    double v[3] = {0.0, 0.0, 0.0};
-    if (lane < kc)
-      for (int d = 0; d < 3; ++d) v[d] = share[3LL * t + d];
-    for (int q = 0; q < kc; ++q) {
-      const int from = small ? __ffs(__ballot_sync(full, lane < n && rank == q)) - 1 : q;
-      for (int d = 0; d < 3; ++d) acc[d] = acc[d] + __shfl_sync(full, v[d], from);
+    double acc = 0.0;
+    for (int k0 = 0; k0 < N; k0 += 32) {
+      const int held = k0 + lane < N ? sorted[B + k0 + lane] : 0, m = min(32, N - k0);
+#pragma unroll 1
+      for (int q0 = 0; q0 < m; q0 += 16) {
+        double v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          const int tq = __shfl_sync(full, held, q0 + q);
+          v[q] = q0 + q < m && lane < 3 ? share[3LL * tq + lane] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          if (q0 + q < m) acc = acc + v[q];
+      }
     }
+    if (lane < 3) F[3 * I + lane] = acc;
   }
-  if (lane == 0)
-    for (int d = 0; d < 3; ++d) F[3 * i + d] = acc[d];
 }
 
 inline unsigned nblocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -341,7 +385,7 @@ ibm_status surface_forces_impl(ibm_tables *T, const ibm_mesh *meshes, int nmesh,
     k_inc_fill<<<nblocks(ntri, 256), 256, 0, st>>>(dtris, (int)ntri, off, cur, list);
     ++launches;
   }
-  k_node_forces<<<nblocks(32 * nvert, NODE_THREADS), NODE_THREADS, 0, st>>>(off, list, share, nvert, sorted, f_node);
+  k_node_forces<<<nblocks(nvert, NODE_THREADS), NODE_THREADS, 0, st>>>(off, list, share, nvert, sorted, f_node);
   IBM_TRY(cudaGetLastError());
   T->ctx->launches += launches;
   // the staging vector is read by the copy above before it returns (pageable host memory)

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import synth
+from oracle import forces as OF
 from oracle import system as OY
 from tests.gpu_util import classify_both, require_gpu, torch
 
@@ -71,3 +72,52 @@ def test_noalloc_residual_takes_short_rows_as_fast_as_long_ones(ctx):
                                                                  b, p)))
         T.close()
     assert times[0] <= 2.0 * times[1], times
+
+
+def _cone(n, centre, size):
+    """Closed double cone of 2 n triangles: two apexes of n triangles each, ring nodes of four."""
+    a = 2.0 * np.pi * np.arange(n) / n
+    v = np.concatenate([np.stack([np.cos(a), np.sin(a), np.zeros(n)], 1), [[0.0, 0.0, 1.1], [0.0, 0.0, -0.9]]])
+    i, j = np.arange(n), (np.arange(n) + 1) % n
+    t = np.concatenate([np.stack([i, j, np.full(n, n)], 1), np.stack([j, i, np.full(n, n + 1)], 1)])
+    return synth.Mesh(size * v + np.asarray(centre), t[np.random.RandomState(n).permutation(2 * n)].astype(np.int32), 1)
+
+
+@pytest.mark.parametrize("valences", [(7, 8, 9, 10, 11, 12), (3, 40, 8, 33, 9, 150), (15, 16, 17, 18, 31, 64), (17,) * 6])
+def test_nodal_forces_by_triangles_per_node(ctx, valences):
+    """One thread per node of up to 16 triangles, a warp per node above (several such nodes in one block):
+    bit for bit the oracle's ordered sums."""
+    pkg, c = ctx
+    f = synth.faces_uniform(30)
+    at = [(x, y, z) for z in (0.25, 0.75) for y in (0.3, 0.7) for x in (0.25, 0.75)]
+    meshes = [_cone(n, at[q], 0.16 + 0.005 * q) for q, n in enumerate(valences)]
+    g, T, _, ib, _ = classify_both(pkg, c, f, f, f, meshes, oracle_ghosts=False)
+    p = synth.counter_normal(5, 0, np.arange(ib.size)).reshape(ib.shape)
+    out = T.surface_forces(meshes, torch.from_numpy(p).cuda())
+    ps, _, F = OF.surface_forces(g, ib, meshes, p)
+    assert np.array_equal(out["p_side"].cpu().numpy(), ps)
+    assert np.array_equal(out["f_node"].cpu().numpy(), F)
+    T.close()
+
+
+
+def test_nodal_sums_are_a_small_part_of_a_large_mesh(ctx):
+    """262,146 nodes of four or six triangles each: the ordered sums take less of the device than the surface
+    pressures of the 524,288 triangles (a warp per node took as long; one thread per node 14 us of 301)."""
+    from torch.profiler import ProfilerActivity, profile
+    pkg, c = ctx
+    f = synth.faces_uniform(64)
+    meshes = [synth.octa_sphere(8, (0.5, 0.5, 0.5), 0.33)]
+    T = pkg.Tables(c, f, f, f, meshes)
+    p = torch.ones(T.shape, dtype=torch.float64, device="cuda")
+    for _ in range(2):   # the first profile starts the profiler
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            for _ in range(3):
+                T.surface_forces(meshes, p)
+            torch.cuda.synchronize()
+    t = {k: sum(e.self_device_time_total for e in prof.key_averages() if k in e.key)
+         for k in ("k_node_forces", "k_tri_pressure")}
+    T.close()
+    if not all(t.values()):
+        pytest.skip("no kernel times from the profiler")
+    assert t["k_node_forces"] <= 0.25 * t["k_tri_pressure"], t
