@@ -2918,12 +2918,11 @@ static bool make_map(CUtensorMap *m, void *base, CUtensorMapDataType dt, int ele
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Finest levels of fewer cells are relaxed strip by strip.  FP32: 96 problems of edges 16 to 32 take 5.0
-// against 5.9 ms, single solves of 24^3 to 64^3 the same either way within 2 %, 24 problems of edges 64
-// to 96 10.2 against 11.3 ms for the fused sweep (a batch that mixes both forms pays two launches per stage,
-// so the line lies at 32^3).  FP64: 24^3 1.39 against 1.70 ms, 64^3 2.44 against 2.93, 80^3 3.25 against 3.64.
-template <typename T>
-constexpr long long fused_cells() { return sizeof(T) == 4 ? (1LL << 15) + 1 : 1LL << 19; }
+// FP64 finest levels of fewer cells are relaxed strip by strip: 64^3 solves take 2.30 ms by strips and 2.93 by
+// the fused sweep, 96^3 4.46 and 4.76, 40 x 130 x 130 3.86 and 4.94, 104^3 5.20 and 5.32, 112^3 5.78 and 5.56.
+// In FP32 a solve by itself takes the fused sweep whatever its size (24^3 0.77 ms against 0.82 by strips, 32^3 0.86
+// and 0.88, 64^3 1.14 and 1.12, 80^3 1.32 and 1.38; without a body, 24^3 0.53 and 0.50).
+constexpr long long FUSED64_CELLS = 1LL << 20;
 template <typename T>
 static void setup_zmarch(Hierarchy *h, void *e0, void *r0) {
   Level &L0 = h->lv[0];
@@ -2945,9 +2944,8 @@ static void setup_zmarch(Hierarchy *h, void *e0, void *r0) {
     h->zm_per_sm = per_sm;
   else
     h->zmarch = false;
-  // small grids: tiles of 128 x 14 leave most lanes idle, and the strip relaxation (the same bits)
-  // with its ghost rows in two launches takes less
-  if ((long long)L0.g.nx * L0.g.ny * L0.g.nz < fused_cells<T>()) h->zmarch = false;
+  // the strip relaxation leaves the same bits
+  if (sizeof(T) == 8 && (long long)L0.g.nx * L0.g.ny * L0.g.nz < FUSED64_CELLS) h->zmarch = false;
 }
 
 // Coarse levels swept by the fused z-march: levels >= 1 of at least ZM_COARSE_CELLS cells in
@@ -3358,6 +3356,7 @@ struct Solver {
   double *scal = nullptr, *part = nullptr;   // this solve's device scalars and block partials
   bool batched = false;                      // one of several problems advancing together
   int sweep_chunk = 0;                       // planes per z-chunk of the fine fused sweep (0: model)
+  bool strips = false;                       // the finest level strip by strip though its fused sweep could run
   const double *gd = nullptr;                // Neumann datum added by the level-0 ghost updates
                                              // (the V-cycle on p itself: precision 0 without GCR)
   // measurement only: events recorded on the stream around each fine-level sweep kernel
@@ -3382,11 +3381,18 @@ void ghost_update(Solver &S, T *e, const T *ghost_rhs) {
 // plane offset that puts every plane a sweep loads past the last one
 inline int sweep_zero_plane(int nz) { return 2 * nz + 64; }
 
+// is the finest level swept by the fused sweep: e and r the arrays its tensor maps cover (in FP64 the solution
+// and right-hand side of the V-cycle on p)
+inline bool fused_fine(const Solver &S, const void *e, const void *r) {
+  const Hierarchy *h = S.h;
+  return h->zmarch && !S.strips && (e == h->tm_base[0] || e == h->tm_base[1]) && r == h->tm_rbase;
+}
+
 // The first sweep of a correction cycle starts from e = 0.  The fused sweep then neither reads e nor
-// needs it cleared (at 1024^3 the clearing took 0.65 ms of a step's 85, at 256^3 12.7 us of 1240); the membranes' cut
-// cells read e, and small grids are relaxed in place, so these clear it.
-inline bool sweep_from_zero(const Hierarchy *h, const ibm_tables *t, const void *e, const void *r, int nu1) {
-  return h->zmarch && !t->membrane && nu1 > 0 && (e == h->tm_base[0] || e == h->tm_base[1]) && r == h->tm_rbase;
+// needs it cleared (at 1024^3 the clearing took 0.65 ms of a step's 85, at 256^3 12.7 us of 1240); the
+// membranes' cut cells read e, and strips are relaxed in place, so these clear it.
+inline bool sweep_from_zero(const Solver &S, const void *e, const void *r) {
+  return fused_fine(S, e, r) && !S.t->membrane && S.nu1 > 0;
 }
 
 // One fused red-black sweep of level l: the finest level (tensor maps of the hierarchy, ghost
@@ -3500,9 +3506,7 @@ void smooth_level(Solver &S, int l, T *&e, const T *r, const double *shift, bool
       if (timed) cudaEventRecord((*S.sweep_events)[2 * s + 1], S.st);
       continue;
     }
-    // the finest level's fused sweep, when e and r are the arrays its tensor maps cover (in
-    // FP64 the solution and right-hand side of the V-cycle on p)
-    if (fine && S.h->zmarch && (e == S.h->tm_base[0] || e == S.h->tm_base[1]) && (const void *)r == S.h->tm_rbase) {
+    if (fine && fused_fine(S, e, r)) {
       T *old = zero && s == 0 ? nullptr : e;
       sweep_zmarch<T>(S, 0, e, shift, zero && s == 0);
       if (timed) cudaEventRecord((*S.sweep_events)[2 * s + 1], S.st);
@@ -3882,6 +3886,19 @@ struct Run {
   ibm_status result = IBM_ERR_NOT_CONVERGED;
 };
 
+// finest-level sweeps of one step
+inline long long fine_sweeps(const Run &R) {
+  return (long long)(R.opts->nu1 + R.opts->nu2) * (R.prec != 0 ? std::max(1, R.opts->inner_cycles) : 1);
+}
+
+// An odd number of fused sweeps leaves e in the other buffer, so such a step cannot be replayed as a graph; on small
+// grids the replay gives more than the fused form, and strips, relaxed in place, allow it (sweeps 2 and 1, one V-cycle
+// per step: 24^3 0.87 against 1.08 ms, 32^3 0.90 against 1.17)
+inline bool small_odd(const Run &R) {
+  const LevelGeom &g = R.h->lv[0].g;
+  return R.prec != 0 && fine_sweeps(R) % 2 != 0 && (long long)g.nx * g.ny * g.nz <= (1LL << 15);
+}
+
 // phase 1: the hierarchy, the solver's fields and the scalars' host copy
 ibm_status run_prepare(Run &R, ibm_ctx *ctx, ibm_tables *t, const ibm_solve_opts *opts, double *scal, double *part,
                        double *hs, bool batched, cudaStream_t st) {
@@ -3897,6 +3914,7 @@ ibm_status run_prepare(Run &R, ibm_ctx *ctx, ibm_tables *t, const ibm_solve_opts
   R.S.scal = scal;
   R.S.part = part;
   R.S.batched = batched;
+  R.S.strips = small_odd(R);
   R.ntot = h->nslot;   // level-0 elements: padded cells and membrane entry slots
   // the scalars first: the packing of p records in S_PNZ whether any value is nonzero
   for (int q = 0; q < NSCAL; ++q) hs[q] = 0.0;
@@ -4049,7 +4067,7 @@ void run_step(Run &R, cudaStream_t bs) {
   } else {
     float *&e32 = reinterpret_cast<float *&>(L0.e);
     for (int q = 0; q < std::max(1, opts->inner_cycles); ++q) {
-      const bool zero = q == 0 && sweep_from_zero(h, R.t, e32, R.r32, S.nu1);
+      const bool zero = q == 0 && sweep_from_zero(S, e32, R.r32);
       if (q == 0 && !zero) cudaMemsetAsync(e32, 0, sizeof(float) * ntot, bs);
       vcycle<float>(S, 0, e32, R.r32, S.scal + S_MU, R.r32, zero);
     }
@@ -4099,9 +4117,7 @@ void run_finish(Run &R, double *p_user, cudaStream_t st) {
 // can one step be captured and replayed: the pointer swaps of the fused sweep cancel over a
 // step when its number of fine sweeps is even
 bool run_graphable(const Run &R) {
-  const ibm_solve_opts *o = R.opts;
-  const long long sweeps = (long long)(o->nu1 + o->nu2) * (R.prec != 0 ? std::max(1, o->inner_cycles) : 1);
-  return o->use_graph && R.ctx->cap_stream && (!R.h->zmarch || sweeps % 2 == 0);
+  return R.opts->use_graph && R.ctx->cap_stream && (!R.h->zmarch || R.S.strips || fine_sweeps(R) % 2 == 0);
 }
 
 // what a captured step depends on: the schedule, whether ghost rows exist and the addresses
@@ -4491,7 +4507,43 @@ const double *lk_shift(Lock &K, int i, int l) {
 
 // can a cycle's first sweep of problem i's finest level start from zero without clearing e
 bool lk_from_zero(Lock &K, int i) {
-  return sweep_from_zero(lk_h(K, i), (*K.R)[i].t, K.E[0][i], (*K.R)[i].r32, K.nu1);
+  return sweep_from_zero((*K.R)[i].S, K.E[0][i], (*K.R)[i].r32);
+}
+
+// plane steps of one fused sweep of level l of every problem in grp, each item two planes and about four steps'
+// start-up beyond its chunk, with the chunk length kz (the same for all) that takes the fewest
+long long lk_sweep_steps(Lock &K, int l, const std::vector<int> &grp, int &kz) {
+  const long long resident = l > 0 ? K.zmc_resident : K.zm_resident;
+  int nzmax = 1;
+  for (int i : grp) nzmax = std::max(nzmax, lk_h(K, i)->lv[l].g.nz);
+  long long best = -1;
+  for (int q = std::min(nzmax, zm::KZ_MAX); q >= 1; --q) {
+    long long items = 0;
+    for (int i : grp) {
+      const LevelGeom &g = lk_h(K, i)->lv[l].g;
+      items += (long long)((g.nx + zm::TX - 1) / zm::TX) * ((g.ny + zm::TY - 1) / zm::TY) * ((g.nz + q - 1) / q);
+    }
+    const long long cost = ((items + resident - 1) / resident) * (q + 6);
+    if (best < 0 || cost < best) { best = cost; kz = q; }
+  }
+  return best;
+}
+
+// Are the finest levels of the batch relaxed strip by strip, all in one form so that a stage stays one launch?  The
+// fused sweep takes about a microsecond per plane step, however little of its 128 x 14 tiles the problems fill; strips
+// about 10 us of launches and 6.5 us per million cells (a sweep of both colours with its ghost rows).  Batches, ms by
+// strips and fused: 96 problems of edges 16 to 32 6.5 and 7.5, of 32 to 40 9.7 and 10.5, of 24 to 96 20.9 and 20.1, of 64
+// to 96 39.2 and 35.1; 24 of 32 to 40 3.33 and 3.30, of 64 to 96 11.2 and 9.8; 4 of 32 to 40 1.82 and 1.75; one
+// of 24 to 48 1.67 and 1.51.  A form for each problem by its own size took two launches per stage of a mixed batch: 24 of
+// edges 24 to 48 3.85 ms, in one form 3.38.
+bool lk_by_strips(Lock &K, const std::vector<int> &grp) {
+  double cells = 0.0;
+  for (int i : grp) {
+    const LevelGeom &g = lk_h(K, i)->lv[0].g;
+    cells += (double)g.nx * g.ny * g.nz;
+  }
+  int kz = 1;
+  return 10.0 + 6.5e-6 * cells < (double)lk_sweep_steps(K, 0, grp, kz);
 }
 
 // one fused sweep of level l of every problem in grp (all swept by the z-march on that level); zero: e
@@ -4499,21 +4551,8 @@ bool lk_from_zero(Lock &K, int i) {
 void lk_zmarch(Lock &K, int l, const std::vector<int> &grp, bool zero) {
   const bool coarse = l > 0;
   const long long resident = coarse ? K.zmc_resident : K.zm_resident;
-  // one chunk length for the launch: the fewest rounds x steps over every problem's items, as
-  // for a single problem (coarse levels: chunks of at most ZM_COARSE_KZ planes)
-  int nzmax = 1;
-  for (int i : grp) nzmax = std::max(nzmax, lk_h(K, i)->lv[l].g.nz);
-  int best_kz = std::min(nzmax, zm::KZ_MAX);
-  long long best_cost = -1;
-  for (int kz = std::min(nzmax, zm::KZ_MAX); kz >= 1; --kz) {
-    long long items = 0;
-    for (int i : grp) {
-      const LevelGeom &g = lk_h(K, i)->lv[l].g;
-      items += (long long)((g.nx + zm::TX - 1) / zm::TX) * ((g.ny + zm::TY - 1) / zm::TY) * ((g.nz + kz - 1) / kz);
-    }
-    const long long cost = ((items + resident - 1) / resident) * (kz + 6);
-    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best_kz = kz; }
-  }
+  int best_kz = 1;
+  lk_sweep_steps(K, l, grp, best_kz);
   if (coarse) best_kz = std::min(best_kz, ZM_COARSE_KZ);
   zm::Batch<float> &B = *K.zb;
   size_t g = 0;
@@ -4593,7 +4632,7 @@ void lk_ghost_update(Lock &K, const std::vector<int> &grp) {
 void lk_smooth(Lock &K, int l, const std::vector<int> &grp, int sweeps, bool zero = false) {
   for (int s = 0; s < sweeps; ++s) {
     std::vector<int> zg, rg;
-    for (int i : grp) ((l == 0 ? lk_h(K, i)->zmarch : lk_h(K, i)->lv[l].zm) ? zg : rg).push_back(i);
+    for (int i : grp) ((l == 0 ? lk_h(K, i)->zmarch && !(*K.R)[i].S.strips : lk_h(K, i)->lv[l].zm) ? zg : rg).push_back(i);
     if (!zg.empty()) {
       std::vector<float *> old(K.E[l]);
       const bool z = zero && s == 0;
@@ -5002,6 +5041,8 @@ ibm_status lockstep_step(Lock &K, const std::vector<int> &act, int inner) {
   std::vector<Run> &R = *K.R;
   IBM_TRY(cudaMemsetAsync(ctx->lk_count, 0, sizeof(int) * LK_COUNTERS, K.st));
   K.ncount = 0;
+  const bool strips = lk_by_strips(K, act);
+  for (int i : act) R[i].S.strips = strips;
   for (int q = 0; q < std::max(1, inner); ++q) {
     if (q == 0) {
       auto blocks = [&](int i) { return lk_from_zero(K, i) ? 0 : (int)std::min<long long>(nblk(R[i].ntot / 4, 256), 1024); };
