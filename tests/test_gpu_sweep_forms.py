@@ -7,6 +7,7 @@ import pytest
 
 import synth
 from tests.gpu_util import require_gpu, torch
+from tests.test_gpu_sweep import _check
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-10
@@ -84,3 +85,37 @@ def test_small_solves_of_odd_schedules(ctx, prec, nu1, nu2, inner):
                               pkg.SolveOpts(precision=prec, nu1=nu1, nu2=nu2, inner_cycles=inner, max_cycles=200))
     assert torch.equal(out[0], out[1]) and torch.equal(out[0], p)
     T.close()
+
+
+def _sphere_at(xf, yf, zf, i, j, k, r):
+    return synth.octa_sphere(4, (xf[i], yf[j], 0.5 * (zf[k] + zf[k + 1])), r)
+
+
+@pytest.mark.parametrize("shape,prec,fused", [((200, 83, 65), 0, True), ((128, 96, 85), 0, False), ((200, 45, 37), 1, True),
+                                              ((37, 20, 9), 1, True), ((37, 20, 9), 2, True), ((5, 4, 6), 1, True)])
+def test_form_of_the_finest_sweep(ctx, shape, prec, fused):
+    """Fused: one kernel per sweep and one for the ghost rows; strips: one per colour, and two for the ghost rows.
+    FP64 fused from 2^20 cells, FP32 whatever the size."""
+    pkg, c = ctx
+    T, b = _problem(pkg, c, shape, 3)
+    n = []
+    for sweeps in (1, 1, 2):   # the first builds the hierarchy
+        n0 = pkg.ibm_ctx_launch_count(c.h)
+        pkg.ibm_smoother_apply(c.h, T.h, prec, sweeps, 1.3, torch.zeros_like(b), b, 0.0)
+        n.append(pkg.ibm_ctx_launch_count(c.h) - n0)
+    ghosts = T.nghost > 0
+    assert n[2] - n[1] == (1 + ghosts if fused else 2 + 2 * ghosts), (n, T.nghost)
+    T.close()
+
+
+def test_fused_fp64_sweep_across_tile_borders(ctx):
+    """200 x 83 x 65 cells in FP64 (the fused form, as its launches show above): 2 x 6 tiles, both ragged, bodies over the
+    x = 128 and y = 14, 42 borders and over chunk seams in z."""
+    xf, yf, zf = synth.faces_tanh(200, 1.5), synth.faces_uniform(83), synth.faces_tanh(65, 1.2)
+    _check(ctx, xf, yf, zf, [_sphere_at(xf, yf, zf, 128, 42, 31, 0.17), _sphere_at(xf, yf, zf, 60, 14, 20, 0.08)], 41,
+           precisions=(0,))
+
+
+def test_fused_fp64_sweep_without_a_body(ctx):
+    """301 x 57 x 62 cells in FP64, no body: three tiles in x and five in y, the last of each ragged."""
+    _check(ctx, synth.faces_uniform(301), synth.faces_tanh(57, 2.0), synth.faces_tanh(62, 1.4), [], 42, precisions=(0,))
