@@ -435,6 +435,12 @@ ibm_status ibm_ctx_launch_count(const ibm_ctx *ctx, int64_t *count);
  * Solves captured as CUDA graphs are recaptured when the setting changes. */
 ibm_status ibm_ctx_set_sweep_wait_limit(ibm_ctx *ctx, int32_t tries);
 
+/* Test hook (no counterpart in the paper): coarse FP32 levels of at least `cells` cells take the
+ * fused sweep, in the solver arrays that tables of this context build from now on (tables that
+ * have solved keep theirs).  The normal line, 2^26 cells, is beyond what a test can hold;
+ * cells < 0 restores it.  Levels from 2^18 cells leave the same bits in either form. */
+ibm_status ibm_ctx_set_coarse_fused_cells(ibm_ctx *ctx, int64_t cells);
+
 /* Relative projected residual of a pressure field, with NO device allocation.  The paper
  * has no counterpart: this exists for callers that cannot allocate device memory after
  * start-up -- e.g. a flow solver that owns a fixed device arena, where cudaMalloc/cudaFree

@@ -562,6 +562,12 @@ ibm_status ibm_ctx_set_sweep_wait_limit(ibm_ctx *ctx, int32_t tries) {
   return IBM_OK;
 }
 
+ibm_status ibm_ctx_set_coarse_fused_cells(ibm_ctx *ctx, int64_t cells) {
+  if (!ctx) return IBM_ERR_INVALID_ARG;
+  ctx->coarse_fused_cells = cells < 0 ? -1 : cells;
+  return IBM_OK;
+}
+
 ibm_status ibm_ctx_launch_count(const ibm_ctx *ctx, int64_t *count) {
   if (!ctx || !count) return IBM_ERR_INVALID_ARG;
   *count = ctx->launches;

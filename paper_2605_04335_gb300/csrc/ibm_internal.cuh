@@ -170,6 +170,8 @@ struct ibm_ctx {
   int *errflag = nullptr;       // device flag: a bounded device-side wait gave up
   int sweep_first_wait = -1;    // tries of the fused sweep's first wait per item (-1: the
                                 // normal limit; set only to test the timeout path)
+  long long coarse_fused_cells = -1;   // coarse FP32 levels of so many cells take the fused sweep (-1: the
+                                       // normal line; set only to test that form on small grids)
   std::string tune_cache;       // autotuner cache file (empty: none)
   cudaStream_t cap_stream = nullptr;   // private stream used only to capture CUDA graphs
   // batched solves: the streams the problems' step graphs run on, fork/join events, and

@@ -3105,7 +3105,8 @@ static ibm_status build_grid_t(ibm_tables *t, cudaStream_t st, Hierarchy **out, 
   // coarse levels swept by the fused sweep: a second e buffer
   for (int l = 1; l < nl; ++l) {
     Level &L = h->lv[l];
-    if (sizeof(T) == 4 && (L.bf16 || (long long)L.g.nx * L.g.ny * L.g.nz >= ZM_COARSE_CELLS)) {
+    const long long line = t->ctx->coarse_fused_cells >= 0 ? t->ctx->coarse_fused_cells : ZM_COARSE_CELLS;
+    if (sizeof(T) == 4 && (L.bf16 || (long long)L.g.nx * L.g.ny * L.g.nz >= line)) {
       if (L.bf16) HTRY(alloc_zero<bf16>(&L.ealt, L.g.ntot, st));
       else HTRY(alloc_zero<T>(&L.ealt, L.g.ntot, st));
       L.zm = true;

@@ -97,6 +97,7 @@ def load_library():
         "ibm_smoother_sweeps_timed": (I32, [P, P, I32, I32, P, C.POINTER(C.c_double)]),
         "ibm_ctx_launch_count": (I32, [P, C.POINTER(I64)]),
         "ibm_ctx_set_sweep_wait_limit": (I32, [P, I32]),
+        "ibm_ctx_set_coarse_fused_cells": (I32, [P, I64]),
         "ibm_smoother_apply": (I32, [P, P, I32, I32, D, P, P, D, P, P]),
         "ibm_measure_fp64_rate": (I32, [P, C.POINTER(C.c_double), P]),
         "ibm_residual_norm_noalloc": (I32, [C.POINTER(ibm_grid), P, I64, P, P, P, P, P, P, P,
@@ -317,6 +318,11 @@ def ibm_smoother_sweeps_timed(ctx, tables, precision: int, nsweeps: int, stream=
 def ibm_ctx_set_sweep_wait_limit(ctx, tries: int):
     """Test hook: tries of the fused sweep's first wait per item (0: give up at once; -1: normal)."""
     _check(load_library().ibm_ctx_set_sweep_wait_limit(ctx, int(tries)), "ibm_ctx_set_sweep_wait_limit")
+
+
+def ibm_ctx_set_coarse_fused_cells(ctx, cells: int):
+    """Test hook: cells from which coarse FP32 levels take the fused sweep (-1: normal)."""
+    _check(load_library().ibm_ctx_set_coarse_fused_cells(ctx, int(cells)), "ibm_ctx_set_coarse_fused_cells")
 
 
 def ibm_smoother_apply(ctx, tables, precision: int, nsweeps: int, omega: float, e, r, mu: float, stream=None):

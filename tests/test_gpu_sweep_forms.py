@@ -119,3 +119,65 @@ def test_fused_fp64_sweep_across_tile_borders(ctx):
 def test_fused_fp64_sweep_without_a_body(ctx):
     """301 x 57 x 62 cells in FP64, no body: three tiles in x and five in y, the last of each ragged."""
     _check(ctx, synth.faces_uniform(301), synth.faces_tanh(57, 2.0), synth.faces_tanh(62, 1.4), [], 42, precisions=(0,))
+
+
+@pytest.fixture
+def coarse_line(ctx):
+    """Sets the cells from which coarse levels take the fused sweep; the normal line afterwards."""
+    pkg, c = ctx
+    yield lambda cells: pkg.ibm_ctx_set_coarse_fused_cells(c.h, cells)
+    pkg.ibm_ctx_set_coarse_fused_cells(c.h, -1)
+
+
+def _solve_both(pkg, c, coarse_line, shape, seed, prec):
+    """(p, report, kernels launched) by strips and by the fused sweep on level 1."""
+    out = []
+    for line in (-1, 1 << 18):
+        coarse_line(line)
+        T, b = _problem(pkg, c, shape, seed, 0.36)
+        for _ in range(2):   # the first builds the hierarchy
+            p = torch.zeros_like(b)
+            n0 = pkg.ibm_ctx_launch_count(c.h)
+            rep = T.solve(b, p, TOL, pkg.SolveOpts(precision=prec, use_graph=0))
+            n = pkg.ibm_ctx_launch_count(c.h) - n0
+        out.append((p, rep, n))
+        T.close()
+    return out
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("shape", [(300, 64, 130), (140, 132, 126)])
+def test_fused_coarse_level_leaves_the_bits_of_the_strips(ctx, coarse_line, shape, prec):
+    """Level 1 of 150 x 32 x 65 (two by three tiles, a body over their borders) and of 70 x 66 x 63 cells: the solve's
+    pressure, cycles and history are the strips' bit for bit, with one kernel less for each of the eight sweeps
+    a step takes on the level."""
+    pkg, c = ctx
+    (p0, r0, n0), (p1, r1, n1) = _solve_both(pkg, c, coarse_line, shape, 5, prec)
+    assert r0["cycles"] == r1["cycles"] and np.array_equal(r0["history"], r1["history"])
+    assert torch.equal(p0, p1)
+    assert n0 - n1 == 8 * r0["cycles"], (n0, n1, r0["cycles"])
+
+
+def test_fused_coarse_level_in_lockstep(ctx, coarse_line):
+    """The batched form of the coarse fused sweep, two problems of other shapes in one launch: each problem's pressure is
+    its own solve's, by strips, bit for bit."""
+    pkg, c = ctx
+    shapes = [(300, 64, 130), (140, 132, 126)]
+    coarse_line(-1)
+    want = []
+    for q, shape in enumerate(shapes):
+        T, b = _problem(pkg, c, shape, q, 0.36)
+        p = torch.zeros_like(b)
+        want.append((p, T.solve(b, p, TOL, pkg.SolveOpts(precision=1))))
+        T.close()
+    steps = []
+    for line in (-1, 1 << 18):
+        coarse_line(line)
+        tabs, rhs = zip(*(_problem(pkg, c, shape, q, 0.36) for q, shape in enumerate(shapes)))
+        ps = [torch.zeros_like(b) for b in rhs]
+        _, reps = pkg.poisson_solve_batched(c.h, [t.h for t in tabs], rhs, TOL, ps, pkg.SolveOpts(precision=1))
+        for p, rep, (w, r) in zip(ps, reps, want):
+            assert rep["cycles"] == r["cycles"] and torch.equal(p, w)
+        steps.append(_launches_per_step(pkg, c, tabs, rhs))
+        _close(tabs)
+    assert steps[0] - steps[1] == 8, steps
