@@ -181,3 +181,25 @@ def test_fused_coarse_level_in_lockstep(ctx, coarse_line):
         steps.append(_launches_per_step(pkg, c, tabs, rhs))
         _close(tabs)
     assert steps[0] - steps[1] == 8, steps
+
+
+@pytest.mark.parametrize("count,shapes,by_strips", [(12, [(96, 88, 90), (90, 97, 85)], False), (38, [(32, 31, 31), (31, 32, 29)], True)])
+def test_lockstep_strips_of_two_planes(ctx, count, shapes, by_strips):
+    """Strips take two planes per thread where a launch holds 2^20 cells or more, here by the sum over the batch (level 1
+    of 12 problems; the finest level of 38) of levels that take one plane in their own solves, with odd numbers of
+    planes: every problem gets its own solve's bits."""
+    pkg, c = ctx
+    level = [tuple((n + (not by_strips)) // (1 if by_strips else 2) for n in shapes[q % 2]) for q in range(count)]
+    assert sum(int(np.prod(s)) for s in level) >= 1 << 20 and all(np.prod(s) < 1 << 18 for s in level)
+    assert any(s[2] % 2 for s in level)
+    tabs, rhs = zip(*(_problem(pkg, c, shapes[q % 2], q) for q in range(count)))
+    few = _launches_per_step(pkg, c, tabs[:2], rhs[:2])
+    # strips: two kernels more per sweep of the finest level (its ghost rows too), and one that clears e
+    assert _launches_per_step(pkg, c, tabs, rhs) - few == (8 * 2 + 1 if by_strips else 0)
+    ps = [torch.zeros_like(b) for b in rhs]
+    _, reps = pkg.poisson_solve_batched(c.h, [t.h for t in tabs], rhs, TOL, ps, pkg.SolveOpts(precision=1))
+    for t, b, p, rep in zip(tabs, rhs, ps, reps):
+        own = torch.zeros_like(b)
+        r = t.solve(b, own, TOL, pkg.SolveOpts(precision=1))
+        assert r["cycles"] == rep["cycles"] and torch.equal(own, p)
+    _close(tabs)
