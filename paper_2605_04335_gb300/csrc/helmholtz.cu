@@ -507,8 +507,8 @@ __global__ void k_hz_update_df(float *uh, float *ul, const float *e, long long n
 }
 
 // Packs and unpacks stream 33 and 17 bytes per cell: a thread takes one cell of four rows of a plane,
-// all loads before the stores (one row per thread keeps a quarter of the bytes in flight: 180 and 97 us at 256^3, this 103 and 57);
-// the split into pairs runs on the integer pipe (dfloat.cuh)
+// all loads before the stores (one row per thread keeps a quarter of the bytes in flight: 180 and 97 us
+// at 256^3, this 103 and 57); the split into pairs runs on the integer pipe (dfloat.cuh)
 constexpr int HZ_PK = 128, HZ_PKR = 4;   // grid: (x blocks, row groups, nz)
 template <class LD, class ST>
 __device__ __forceinline__ void hz_rows(int nx, int ny, LevelGeom g, const uint8_t *mask, LD ld, ST st) {
@@ -570,7 +570,9 @@ __global__ void __launch_bounds__(HZ_PK) k_hz_unpack(const double *up, int nx, i
           [&](long long l, long long, bool, bool active, double2 x) { u[l] = active ? x.x : 0.0; });
 }
 
-// u += e on every slot (e is zero off the active rows)
+// u += e on every slot.  Off the active rows (and membranes' entries) e may hold an earlier solve's values, since a
+// correction that starts from zero is not cleared: u is then as undefined there, and nothing reads it
+// (neighbours and sources of active rows are active, the packs rewrite every cell, the unpacks write zeros)
 __global__ void k_hz_update(double *u, const float *e, long long n) {
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
     u[q] += (double)e[q];
@@ -730,7 +732,8 @@ ibm_status helmholtz_solve_impl(ibm_ctx *ctx, ibm_tables *t, double alpha, const
   std::vector<double> om(K);
   for (int k = 0; k < K; ++k) om[k] = 1.0 / (1.0 + rho * std::cos(3.141592653589793 * (2.0 * k + 1.0) / (2.0 * K)));
   const dim3 sweep_grid(nb_of(nx, TX), nb_of(ny, TY), nb_of(nz, KCH)), sweep_block(TX, TY);
-  const int rest_blocks = (int)std::max<long long>(1, std::min<long long>(HZ_BLOCKS, nb_of((cuts ? h->cutcap : 0) + ng, HZ_THREADS)));
+  const int rest_blocks =
+      (int)std::max<long long>(1, std::min<long long>(HZ_BLOCKS, nb_of((cuts ? h->cutcap : 0) + ng, HZ_THREADS)));
   // the FP32 sweep's grid; the double-FP32 residual's: one wave of two blocks per SM, and the planes per
   // march that give the fewest plane steps
   const long long strips = (long long)(nx4 / 4) * ny;

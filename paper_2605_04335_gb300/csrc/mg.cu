@@ -254,8 +254,7 @@ __global__ void k_fractions(const uint8_t *mf, const T *ffx, const T *ffy, const
 // the lowest row, so the result is deterministic.  Bound by its chain of m = n + 1 columns with
 // five barriers each: a warp takes whole rows (no division per entry) from the pivot's column on (the
 // columns before it are never read again), the cells are staged once and neighbours looked up by
-// cell.  267 us on
-// 105 cells, 496 us with one flat loop over the matrix
+// cell.  267 us on 105 cells, 496 us with one flat loop over the matrix
 template <typename T>
 __global__ void __launch_bounds__(1024) k_coarsest_setup(LV<T> v, int *cidx, int *ncount, T *Minv, T *gj) {
   extern __shared__ __align__(16) unsigned char gj_smem[];
@@ -535,9 +534,11 @@ __global__ void __launch_bounds__(RELAX_THREADS) k_relax(LV<T> v, T *e, const T 
 }
 
 // the order of a level's sums: the fused sweep's (the diagonal's part first, the separable diagonal
-// of regular cells) in FP64 and from 2^18 cells, below it the neighbours' parts first and the
-// diagonal as their sum.  Which of the two is not a question of speed: near the tolerance a
-// Krylov-accelerated solve turns a changed rounding of the coarse levels into one step more or fewer
+// of regular cells) in FP64 and from 2^18 cells, where coarse levels of either form meet (the fused one
+// when stored in BF16 or from 2^26 cells), below it the neighbours' parts first and the diagonal as
+// their sum.  Which of the two is not a question of speed: near the tolerance a Krylov-accelerated
+// solve turns a changed rounding of the coarse levels into one step more or fewer, so each level
+// keeps the order its results have had
 template <typename T>
 inline bool relax_sep(const LevelGeom &g) { return sizeof(T) == 8 || (long long)g.nx * g.ny * g.nz >= (1LL << 18); }
 
@@ -583,7 +584,8 @@ __device__ __forceinline__ void ghost_pp_body(const long long *src, const long l
   const long long d = dst[g];
   if (ngp && g >= *ngp) return;
   const T b = rhs ? rhs[d] : (T)0;
-  T s = row.template sum<T>([&](long long q) { return (q & GHOST_CORNER) ? (eold ? eold[q & ~GHOST_CORNER] : (T)0) : enew[q]; });
+  T s = row.template sum<T>(
+      [&](long long q) { return (q & GHOST_CORNER) ? (eold ? eold[q & ~GHOST_CORNER] : (T)0) : enew[q]; });
   if (rhs) s += b;
   if (gd) s += (T)gd[g];     // the row's Neumann datum
   enew[d] = s;
@@ -631,8 +633,8 @@ inline int row_lg(int n) {
 }
 
 // Restriction of the level-f residual to level c, one thread per coarse cell (I,J,K) with
-// coarse rows strided over blockIdx.y (2^lg threads along x, 128 / 2^lg rows per block): rc = sum over the fluid children of V_f r_f / V_c,
-// with r_f = r - shift - (A e)_f; ec = 0 (the coarse correction starts from zero); block
+// coarse rows strided over blockIdx.y (2^lg threads along x, 128 / 2^lg rows per block):
+// rc = sum over the fluid children of V_f r_f / V_c, with r_f = r - shift - (A e)_f; ec = 0 (the coarse correction starts from zero); block
 // partials of sum V_c rc at partials[by * gx + bx] (block (bx, by) of a gx x gy grid).  Every load of a
 // coarse cell (the 2x2x2 children of e, r and mask and their 24 face neighbours) is issued
 // before the arithmetic; children past an odd fine extent are halo cells (mask 1) whose
@@ -1660,7 +1662,9 @@ __device__ __forceinline__ void clear_ghost_partials(double *gpart, int bx, int 
     for (int b = bx + gx; b < FIXED_BLOCKS; b += gx) gpart[b] = 0.0;
 }
 // blocks of the ghost residual over ng rows (a launch for a count read on the device takes FIXED_BLOCKS)
-inline int ghost_resid_blocks(long long ng) { return (int)std::max<long long>(1, std::min<long long>(FIXED_BLOCKS, nblk(ng, REDUCE_THREADS))); }
+inline int ghost_resid_blocks(long long ng) {
+  return (int)std::max<long long>(1, std::min<long long>(FIXED_BLOCKS, nblk(ng, REDUCE_THREADS)));
+}
 
 // ghost rows r_G = sum w v - g; block partials of (s_G r_G)^2 at gpart[b]
 template <typename R, class G>
@@ -4102,16 +4106,17 @@ void run_finish(Run &R, double *p_user, cudaStream_t st) {
   Level &L0 = h->lv[0];
   const long long ntot = R.ntot;
   double *scal = R.S.scal, *part = R.S.part;
+  const int sum_blocks = row_blocks(L0.g, REDUCE_BLOCKS), out_blocks = pack_blocks(L0.g, R.ctx->wave);
+  const float *ph = hi_of(h->p64), *pl = lo_of(h->p64, ntot);
   if (R.S.dfo)
-    k_gauge_sum_df<<<row_blocks(L0.g, REDUCE_BLOCKS), REDUCE_THREADS, 0, st>>>(fine_view_df(h), hi_of(h->p64), lo_of(h->p64, ntot),
-                                                             part);
+    k_gauge_sum_df<<<sum_blocks, REDUCE_THREADS, 0, st>>>(fine_view_df(h), ph, pl, part);
   else
-    k_gauge_sum<<<row_blocks(L0.g, REDUCE_BLOCKS), REDUCE_THREADS, 0, st>>>(fine_view64(h), h->p64, part);
+    k_gauge_sum<<<sum_blocks, REDUCE_THREADS, 0, st>>>(fine_view64(h), h->p64, part);
   k_gauge_finalize<<<1, 256, 0, st>>>(part, REDUCE_BLOCKS, scal);
   if (R.S.dfo)
-    k_unpack_gauge_df<<<pack_blocks(L0.g, R.ctx->wave), PK_THREADS, 0, st>>>(hi_of(h->p64), lo_of(h->p64, ntot), L0.mask, L0.g, scal, p_user);
+    k_unpack_gauge_df<<<out_blocks, PK_THREADS, 0, st>>>(ph, pl, L0.mask, L0.g, scal, p_user);
   else
-    k_unpack_gauge<<<pack_blocks(L0.g, R.ctx->wave), PK_THREADS, 0, st>>>(h->p64, L0.mask, L0.g, scal, p_user);
+    k_unpack_gauge<<<out_blocks, PK_THREADS, 0, st>>>(h->p64, L0.mask, L0.g, scal, p_user);
   R.ctx->launches += 3;
 }
 

@@ -87,6 +87,7 @@ constexpr int KZ_MAX = 256;     // planes per item at most (the z-coefficient ta
 constexpr int DP = 2;
 constexpr int NE = 3 + DP;
 constexpr int NR = 1 + DP;
+static_assert(NE == 3 + DP && NR == 1 + DP, "a step refills the buffers of planes q-2 (e) and q-1 (rhs, mask)");
 
 constexpr int pad128(int bytes) { return (bytes + 127) / 128 * 128; }
 template <typename T> constexpr int esz() { return pad128(EY * BX * (int)sizeof(T)) / (int)sizeof(T); }  // per e buffer
@@ -456,8 +457,9 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
   // prologue: e planes k0-2 .. k0-1+DP and rhs/mask planes k0-1 .. k0-2+DP.  Step q waits
   // for e plane q+1 and rhs/mask plane q and, after the step's barrier (so no thread still
   // reads the buffers being refilled), prefetches e plane q+1+DP (into the buffer of plane
-  // q-2, last read in step q-1) and rhs/mask plane q+DP (buffer of plane q-2, last read by
-  // the red pass of step q-1).  Every load is issued once and waited for once.
+  // q-2, last read in step q-1) and rhs/mask plane q+DP (into the buffer of plane q-1, read by
+  // the red passes of step q-1, so not before this step's barrier).  Every load is issued once
+  // and waited for once.
   if (issuer) {
     fence_proxy_async();
     for (int pl = k0 - 2, b = se0; pl <= min(k0 - 1 + DP, k1 + 1); ++pl, b = wrap_e(b + 1)) load_e(pl, b);
@@ -599,11 +601,11 @@ __device__ __forceinline__ void march_item(Smem<T, S> &s, const Args<T> &a, cons
         const unsigned mm = *reinterpret_cast<const unsigned *>(M + imq0) | s.ccu[lane][h];
         const long long gid = (long long)(q + 1) * a.sz + (long long)(y0 + yr + 1) * a.sy + (x0 + xs + 4);
         if (((y0 + yr + q) & 1) == 0)
-          relax_strip<0, COARSE>(C, ld1(P + iq0 - 1), N, So, Zm, Zp, Rr.x, Rr.z, mm, X, cc[0], cc[1], cc[2] + szr, zmr, zpr, sh, om,
-                                 a, gid);
+          relax_strip<0, COARSE>(C, ld1(P + iq0 - 1), N, So, Zm, Zp, Rr.x, Rr.z, mm, X, cc[0], cc[1], cc[2] + szr, zmr,
+                                 zpr, sh, om, a, gid);
         else
-          relax_strip<1, COARSE>(C, ld1(P + iq0 + 4), N, So, Zm, Zp, Rr.y, Rr.w, mm, X, cc[0], cc[1], cc[2] + szr, zmr, zpr, sh, om,
-                                 a, gid);
+          relax_strip<1, COARSE>(C, ld1(P + iq0 + 4), N, So, Zm, Zp, Rr.y, Rr.w, mm, X, cc[0], cc[1], cc[2] + szr, zmr,
+                                 zpr, sh, om, a, gid);
         sts4(P + iq0, C);
       }
       // ring column cell (x = -1 or TX): the red one of the lane's pair of rows
