@@ -4522,13 +4522,15 @@ long long lk_sweep_steps(Lock &K, int l, const std::vector<int> &grp, int &kz) {
   const long long resident = l > 0 ? K.zmc_resident : K.zm_resident;
   int nzmax = 1;
   for (int i : grp) nzmax = std::max(nzmax, lk_h(K, i)->lv[l].g.nz);
+  std::vector<std::pair<int, int>> ps;   // tiles and planes
+  for (int i : grp) {
+    const LevelGeom &g = lk_h(K, i)->lv[l].g;
+    ps.emplace_back(((g.nx + zm::TX - 1) / zm::TX) * ((g.ny + zm::TY - 1) / zm::TY), g.nz);
+  }
   long long best = -1;
   for (int q = std::min(nzmax, zm::KZ_MAX); q >= 1; --q) {
     long long items = 0;
-    for (int i : grp) {
-      const LevelGeom &g = lk_h(K, i)->lv[l].g;
-      items += (long long)((g.nx + zm::TX - 1) / zm::TX) * ((g.ny + zm::TY - 1) / zm::TY) * ((g.nz + q - 1) / q);
-    }
+    for (const auto &[tiles, nz] : ps) items += (long long)tiles * ((nz + q - 1) / q);
     const long long cost = ((items + resident - 1) / resident) * (q + 6);
     if (best < 0 || cost < best) { best = cost; kz = q; }
   }
@@ -5047,8 +5049,6 @@ ibm_status lockstep_step(Lock &K, const std::vector<int> &act, int inner) {
   std::vector<Run> &R = *K.R;
   IBM_TRY(cudaMemsetAsync(ctx->lk_count, 0, sizeof(int) * LK_COUNTERS, K.st));
   K.ncount = 0;
-  const bool strips = lk_by_strips(K, act);
-  for (int i : act) R[i].S.strips = strips;
   for (int q = 0; q < std::max(1, inner); ++q) {
     if (q == 0) {
       auto blocks = [&](int i) { return lk_from_zero(K, i) ? 0 : (int)std::min<long long>(nblk(R[i].ntot / 4, 256), 1024); };
@@ -5179,6 +5179,8 @@ ibm_status solve_batched_impl(ibm_ctx *ctx, int n, ibm_tables *const *ts, const 
     if ((s = lockstep_setup(K, R)) != IBM_OK) return s;
     IBM_TRY(cudaMemcpyAsync(ctx->bscal, ctx->bhscal, sizeof(double) * NSCAL * n, cudaMemcpyHostToDevice, st));
     lk_pack(K, all, rhs, p_user);
+    const bool strips = lk_by_strips(K, all);   // while the packing runs
+    for (Run &r : R) r.S.strips = strips;
   } else {
     for (int p = 0; p < n; ++p)
       if ((s = run_pack(R[p], rhs[p], p_user[p], st)) != IBM_OK) return s;
