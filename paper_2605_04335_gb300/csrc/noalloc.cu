@@ -24,8 +24,8 @@
 // pass, about 14: each difference along z serves two planes and each one along x two lanes (by a
 // shuffle; lane 0 only provides it), two along y, six products, and four for the two squares.  The
 // direct form of both passes (stencil, volumes and sums per cell, 36 operations) took 1340 us at
-// 256^3 with its single-thread sums over the blocks; this takes 777 us (the second
-// pass 499, 90 % of the FP64 rate).
+// 256^3 with its single-thread sums over the blocks; this takes 735 us (the first
+// pass 111, the second 489, 91 % of the FP64 rate).
 #include <cmath>
 #include <mutex>
 
